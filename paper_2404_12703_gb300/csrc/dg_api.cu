@@ -196,6 +196,9 @@ static void build_ops(int N, int gauss, Ops& o) {
     for (int i = 0; i < n; ++i) gam += w[i] * L[mm * n + i] * L[mm * n + i];
     for (int i = 0; i < n; ++i) o.Vinv[mm * n + i] = (double)(w[i] * L[mm * n + i] / gam);
   }
+  // the shock indicator's threshold and sharpness (Sec. 2.3)
+  o.ind_T = 0.5 * std::pow(10.0, -1.8 * std::pow((double)n, 0.25));
+  o.ind_s = std::log((1.0 - 1e-4) / 1e-4);
 }
 
 int set_error(int code, const std::string& msg) { return fail(code, msg); }

@@ -233,7 +233,7 @@ do {
         al = a.alpha_force;
       } else {
         double* X1 = reinterpret_cast<double*>(Wk);  // the workspace is free here
-        al = element_alpha<n>(U[0] * p_full, X1, X1 + n3, X1 + 2 * n3, sVi, t, a.alpha_min, a.alpha_max);
+        al = element_alpha<n>(U[0] * p_full, X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
       }
       if (valid && t == 0) a.alpha[e] = al;
       if (__syncthreads_or(al > 0)) {
@@ -248,13 +248,12 @@ do {
           const double* fm = FVm + (size_t)(d * (n - 1) + (right ? id : n - 2)) * 3 * n2 + line;
           const double mv[3] = {fm[0], fm[n2], fm[2 * n2]};
           const double sAd = sqrt(mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2]);
-          const float nu[3] = {float(mv[0] / sAd), float(mv[1] / sAd), float(mv[2] / sAd)};
-          const int nb = right ? t + sd : t;
-          double UR[5];
-          const double* ur = a.U + (size_t)e * 5 * n3 + nb;
-  #pragma unroll
-          for (int k = 0; k < 5; ++k) UR[k] = ur[k * n3];
-          const SPrim<float> qR = shifted_prim<float>(UR, a.gm1, a.Rinv, cp);
+          const double sAi = 1.0 / sAd;  // one FP64 division instead of three
+          const float nu[3] = {float(mv[0] * sAi), float(mv[1] * sAi), float(mv[2] * sAi)};
+          // the right neighbour's primitives from the halved planes (exact)
+          const int vr = pad_idx<n>(right ? t + sd : t);
+          const float4 ar = P4[vr], br = Q4[vr];
+          const SPrim<float> qR{2.0f * ar.x, 2.0f * ar.y, 2.0f * ar.z, 2.0f * ar.w, 2.0f * br.x, 2.0f * br.y, br.z};
           float fb[5];
           lf_flux_s(me, qR, nu, a.f_gamma, cp.fpr, fb);
           if (right) {

@@ -839,15 +839,20 @@ __global__ void __launch_bounds__(256) k_surf_flux(StageArgs a) {
 
 // ---------------------------------------------------------------------------
 // Hennemann indicator on rho p (modal energy of the top modes), Sec. 2.3, in
-// FP64 on both paths.  Every thread of the element runs the same
-// instructions (no single-thread branch in front of a barrier): row sums are
-// formed by all threads (rows are formed twice or more, with identical
-// values), then every thread adds the row sums itself.
-// sT1 / sT2: n3 doubles each, sRow: 4 n2 doubles.
+// FP64 on both paths.  The FP64 unit bounds it (one FP64 operation per thread
+// takes an SM as long as 60 FP32 ones), so only the modal transform runs on
+// every thread; the n^2 rows of modes are summed by one thread each, the rows
+// by 3 n threads, and one thread forms the element's factor, with the
+// threshold's constants from the host.  Every thread adding all row sums and
+// evaluating pow, log and exp itself took 1,617 us per volume kernel launch
+// on the 64 x 8 x 8 N = 5 shock tube and 338 us per element kernel launch on
+// 8^3 N = 7 in FP32-bulk; this form 1,010 and 65 us.
+// All threads call it (it holds barriers); the scratch (sT1 / sT2: n3 doubles
+// each, sRow: 4 n2 doubles) may be reused after the caller's next barrier.
 // ---------------------------------------------------------------------------
 template <int n>
-__device__ double element_alpha(double rp, double* sT1, double* sT2, double* sRow, const double* sVinv, int t,
-                                double amin, double amax) {
+__device__ double element_alpha(double rp, double* sT1, double* sT2, double* sRow, const double* sVinv,
+                                const Ops* ops, int t, double amin, double amax) {
   constexpr int n2 = n * n, N = n - 1;
   const int i = t % n, j = (t / n) % n, k = t / n2;
   sT1[t] = rp;
@@ -868,43 +873,44 @@ __device__ double element_alpha(double rp, double* sT1, double* sT2, double* sRo
   sT2[t] = s * s;  // energy of mode (i, j, k)
   __syncwarp();
   __syncthreads();
-  {
-    // row r = (j, k): sums over i by the maximum degree max(i, j, k)
-    const int r = t % n2, rj = r % n, rk = r / n;
-    double mN = 0, mN1 = 0, tot = 0, tot1 = 0;
-    for (int x = 0; x < n; ++x) {
-      const int dv = max(x, max(rj, rk));
-      const double m2 = sT2[x + n * r];
-      tot += m2;
-      tot1 += dv <= N - 1 ? m2 : 0.0;
-      mN += dv == N ? m2 : 0.0;
-      mN1 += dv == N - 1 ? m2 : 0.0;
-    }
-    sRow[r] = mN;
-    sRow[n2 + r] = mN1;
-    sRow[2 * n2 + r] = tot;
-    sRow[3 * n2 + r] = tot1;
+  if (t < n2) {
+    // row (j, k) = (t % n, t / n): the energies of maximum degree N, N - 1
+    // and below, from its last two modes and the sum of the others
+    const double* m2 = sT2 + n * t;
+    double low = 0.0;
+    for (int x = 0; x < N - 1; ++x) low += m2[x];
+    const int mx = max(t % n, t / n);
+    const double below = low + m2[N - 1];
+    sRow[t] = mx == N ? below + m2[N] : m2[N];
+    sRow[n2 + t] = mx == N ? 0.0 : (mx == N - 1 ? below : m2[N - 1]);
+    sRow[2 * n2 + t] = mx < N - 1 ? low : 0.0;
   }
   __syncwarp();
   __syncthreads();
-  double mN = 0, mN1 = 0, tot = 0, tot1 = 0;
-  for (int r = 0; r < n2; ++r) {
-    mN += sRow[r];
-    mN1 += sRow[n2 + r];
-    tot += sRow[2 * n2 + r];
-    tot1 += sRow[3 * n2 + r];
+  if (t < 3 * n) {
+    const double* r = sRow + (t / n) * n2 + (t % n) * n;
+    double a = 0.0;
+    for (int x = 0; x < n; ++x) a += r[x];
+    sT1[t] = a;
   }
-  const double e1 = tot > 0 ? mN / tot : 0.0;
-  const double e2 = tot1 > 0 ? mN1 / tot1 : 0.0;
-  const double E = e1 > e2 ? e1 : e2;
-  const double T = 0.5 * pow(10.0, -1.8 * pow((double)(N + 1), 0.25));
-  const double sh = log((1.0 - 1e-4) / 1e-4);
-  double al = 1.0 / (1.0 + exp(-sh * (E - T) / T));
-  if (al < amin) al = 0.0;
-  if (al > amax) al = amax;
   __syncwarp();
-  __syncthreads();  // sT1 / sT2 / sRow may be reused after this
-  return al;
+  __syncthreads();
+  if (t == 0) {
+    double mN = 0.0, mN1 = 0.0, rest = 0.0;
+    for (int x = 0; x < n; ++x) mN += sT1[x], mN1 += sT1[n + x], rest += sT1[2 * n + x];
+    const double tot1 = rest + mN1, tot = tot1 + mN;
+    const double e1 = tot > 0 ? mN / tot : 0.0;
+    const double e2 = tot1 > 0 ? mN1 / tot1 : 0.0;
+    const double E = e1 > e2 ? e1 : e2;
+    const double T = ops->ind_T;
+    double al = 1.0 / (1.0 + exp(-ops->ind_s * (E - T) / T));
+    if (al < amin) al = 0.0;
+    if (al > amax) al = amax;
+    sT2[0] = al;
+  }
+  __syncwarp();
+  __syncthreads();
+  return sT2[0];
 }
 
 // shared-memory layout of k_volume: FP64 part first, then the T arrays
@@ -1213,7 +1219,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     } else {
       double* X1 = sX + le * (2 * n3 + 4 * n2);
       // all threads of the block take part in the barriers inside
-      al = element_alpha<n>(U[0] * p_full, X1, X1 + n3, X1 + 2 * n3, sVi, t, a.alpha_min, a.alpha_max);
+      al = element_alpha<n>(U[0] * p_full, X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
     }
     if (valid && t == 0) a.alpha[e] = al;
     // block-uniform condition: the FV pass has barriers, and the elements of
@@ -1232,7 +1238,8 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
         const double* fm = FVm + (size_t)(d * (n - 1) + (right ? id : n - 2)) * 3 * n2 + line;
         const double mv[3] = {fm[0], fm[n2], fm[2 * n2]};
         const double sAd = sqrt(mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2]);
-        const T nu[3] = {T(mv[0] / sAd), T(mv[1] / sAd), T(mv[2] / sAd)};
+        const double sAi = 1.0 / sAd;  // one FP64 division instead of three
+        const T nu[3] = {T(mv[0] * sAi), T(mv[1] * sAi), T(mv[2] * sAi)};
         const int nb = right ? t + str[d] : t;
         double UR[5];
         const double* ur = a.U + (size_t)e * 5 * n3 + nb;

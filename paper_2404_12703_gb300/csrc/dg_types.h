@@ -21,6 +21,7 @@ struct Ops {
   double Dsplit[NPMAX * NPMAX];  // 2 D + corner corrections (diagonal zero), LGL
   double Dlo[NPMAX * NPMAX];     // D - (double)D (double-double tail)
   double Vinv[NPMAX * NPMAX];    // nodal -> orthonormal Legendre modes
+  double ind_T, ind_s;           // shock indicator: threshold T(N), sharpness s
   double Lp[NPMAX], Lm[NPMAX];   // l_i(+1), l_i(-1) (unit vectors on LGL)
   // geometry: the LGL derivative matrix (double-double) and the
   // interpolation from the LGL nodes to the solution nodes (double-double;
