@@ -261,7 +261,7 @@ int dg_set_sponge(dg_ctx* ctx, const double* sigma, const double* U_base);
    every launch variant on the context's current state and keeps the fastest:
    elements per thread block of the lifting and volume kernels (the default,
    about 256 threads, or twice as many elements), the volume kernel's thread
-   mapping for the split-form sums (FP64: one task per line pair, or one per
+   form of the line sums (FP64: 64-bit fixed point, or FP64 sums per
    node) and the side kernels' block size (128 or 256 threads).  In the
    two-kernel FP32-bulk stage (see dg_stage_form) the volume entries apply to
    its element kernel and the side entry to its side kernel.  Only scratch
@@ -277,7 +277,7 @@ int dg_set_sponge(dg_ctx* ctx, const double* sigma, const double* U_base);
 int dg_autotune(dg_ctx* ctx, int* config, double* ms);
 
 /* Sets or reads back the launch configuration, 7 ints: lift elements per
-   block, volume elements per block, line pairs (1) or per node (0), side
+   block, volume elements per block, FP64's fixed-point sums (1) or FP64 sums per node (0), side
    block size (0 / -1 entries select the defaults), the FP32-bulk stage form
    (0: the two-kernel stage where it applies, else four kernels; 1: always
    the four-kernel stage), the two-kernel stage's L2 prefetch of the next

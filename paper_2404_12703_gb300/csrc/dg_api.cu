@@ -196,6 +196,43 @@ static void build_ops(int N, int gauss, Ops& o) {
     for (int i = 0; i < n; ++i) gam += w[i] * L[mm * n + i] * L[mm * n + i];
     for (int i = 0; i < n; ++i) o.Vinv[mm * n + i] = (double)(w[i] * L[mm * n + i] / gam);
   }
+  // fixed-point operators
+  ld Ms[NPMAX * NPMAX], Mh[NPMAX * NPMAX];
+  for (int i = 0; i < n; ++i)
+    for (int a = 0; a < n; ++a) {
+      Mh[i * n + a] = -(w[a] / w[i]) * D[a * n + i];
+      // antisymmetric to the last bit (the diagonal is zero; not formed here,
+      // where it would cancel to rounding)
+      Ms[i * n + a] = gauss ? 0 : i < a ? 2 * w[i] * D[i * n + a] : i > a ? -Ms[a * n + i] : 0;
+    }
+  auto row_sum = [n](const ld* M) {
+    ld most = 0;
+    for (int i = 0; i < n; ++i) {
+      ld row = 0;
+      for (int a = 0; a < n; ++a) row += std::fabs(M[i * n + a]);
+      most = std::max(most, row);
+    }
+    return most;
+  };
+  auto fixed = [](const ld* M, int count, ld most, long long* out) {
+    int k = 0;
+    std::frexp(most, &k);  // most < 2^k
+    for (int i = 0; i < count; ++i) out[i] = std::llrint(std::ldexp(M[i], 62 - k));
+    return 62 - k;
+  };
+  ld wi[NPMAX];
+  for (int i = 0; i < n; ++i) wi[i] = 1 / w[i];
+  o.fxS_bits = fixed(Ms, n * n, row_sum(Ms), o.fxS);
+  o.fxH_bits = fixed(Mh, n * n, row_sum(Mh), o.fxH);
+  o.fxW_bits = fixed(wi, n, *std::max_element(wi, wi + n), o.fxW);
+  o.fxS_row = (float)std::ldexp(row_sum(Ms), o.fxS_bits - 62) * 1.00001f;
+  const int h = n / 2;
+  for (int i = 0; i < h && n % 2 == 0; ++i)
+    for (int j = 0; j < h; ++j) {
+      const ld p = Mh[i * n + j], m = Mh[i * n + n - 1 - j];
+      o.fxHe[i * h + j] = std::llrint(std::ldexp((p + m) / 2, o.fxH_bits));
+      o.fxHo[i * h + j] = std::llrint(std::ldexp((p - m) / 2, o.fxH_bits));
+    }
   // the shock indicator's threshold and sharpness (Sec. 2.3)
   o.ind_T = 0.5 * std::pow(10.0, -1.8 * std::pow((double)n, 0.25));
   o.ind_s = std::log((1.0 - 1e-4) / 1e-4);

@@ -233,7 +233,8 @@ do {
         al = a.alpha_force;
       } else {
         double* X1 = reinterpret_cast<double*>(Wk);  // the workspace is free here
-        al = element_alpha<n>(U[0] * p_full, X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
+        X1[t] = U[0] * p_full;
+        al = element_alpha<n>(X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
       }
       if (valid && t == 0) a.alpha[e] = al;
       if (__syncthreads_or(al > 0)) {

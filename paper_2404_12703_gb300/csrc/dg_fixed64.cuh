@@ -1,0 +1,999 @@
+// dg_fixed64.cuh -- the FP64 element kernels on LGL nodes with their line sums
+// and two-point fluxes in 64-bit fixed point on the integer pipe (included by
+// dg_stage.cuh).
+//
+// Why.  A GB300 SM finishes 1.96 FP64 operations per clock and 61 products
+// 32 x 32 -> 64 bits with a 64-bit addition (mad.wide), 59 additions of 64-bit
+// integers (measured).  A product of two 62-bit fixed-point numbers, rounded
+// to 64 bits, is three mad.wide and a shift: eight times cheaper than one
+// FP64 multiplication, and with more bits.  The kernels here were bound by
+// the FP64 unit (84 - 96 % busy); what they keep on it is ConsToPrim, the
+// stress tensor and the Runge-Kutta update.  Measured per launch on 24^3
+// elements, N = 7 (7.08 M nodes): volume kernel 7.70 -> 2.89 ms, lifting
+// 4.12 -> 1.45 ms; now bound by latency at two blocks per SM (issue 44 % busy,
+// FP64 unit 42 %).
+//
+// Numbers.  Every element scales each group of quantities (density, velocity,
+// pressure, enthalpy, metrics, ...) by the power of two that brings the
+// group's largest magnitude in the element below 2^60 or 2^61; a value is
+// that many bits of a two's complement 64-bit integer.  The error of a
+// conversion is below one unit, 2^-60 of the largest value, where FP64 rounds
+// each value to 2^-53 of itself; products keep 64 bits and are rounded, sums
+// are exact.  Results are rounded to FP64 once, at the end.  Scales depend on
+// the element alone, so results do not depend on the launch shape.
+// The bounds on every intermediate value stand beside it; none can overflow.
+// Error against the long-double oracle, N = 1 .. 7, Ma 0.1 - 1.25, viscous,
+// Roe and LF: 0.72 of the FP64 kernels' in the mean, at most 1.001.
+// An element with a non-finite value, or with a group whose largest value is
+// outside 2^-200 .. 2^200, is done in FP64 in the same kernels, with FP64's
+// own treatment of such values.
+#pragma once
+
+namespace dg {
+
+// A 64-bit integer x as hi 2^32 + lo with lo in [-2^31, 2^31)
+struct Fx {
+  int lo, hi;
+};
+__device__ __forceinline__ Fx fx_split(long long x) {
+  const int lo = (int)x;
+  return {lo, (int)(x >> 32) + (int)((unsigned)lo >> 31)};
+}
+// Sum of products a b 2^-64: h in units of 1, x in units of 2^-32 (the
+// products of the low words, below half a unit each, are left out).  get: the
+// sum times 2^S.  FxSum<S> rounds (x starts at half a unit of the result);
+// FxSumS takes S at run time and truncates.
+__device__ __forceinline__ long long fx_get(long long h, long long x, int S) {
+  return (long long)((unsigned long long)h << S) + (x >> (32 - S));
+}
+template <int S>
+struct FxSum {
+  long long h = 0, x = 1LL << (31 - S);
+  __device__ __forceinline__ void add(Fx a, Fx b) {
+    h += (long long)a.hi * b.hi;
+    x += (long long)a.hi * b.lo;
+    x += (long long)a.lo * b.hi;
+  }
+  __device__ __forceinline__ long long get() const { return fx_get(h, x, S); }
+};
+struct FxSumS {
+  long long h = 0, x = 0;
+  __device__ __forceinline__ void add(Fx a, Fx b) {
+    h += (long long)a.hi * b.hi;
+    x += (long long)a.hi * b.lo;
+    x += (long long)a.lo * b.hi;
+  }
+  __device__ __forceinline__ long long get(int S) const { return fx_get(h, x, S); }
+};
+
+// Biased FP64 exponent of the largest magnitude from the maximum of the high words
+__device__ __forceinline__ unsigned fx_field(unsigned hi_max) { return hi_max >> 20; }
+__device__ __forceinline__ unsigned fx_mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+// exponents outside 2^-200 .. 2^200 (zero is inside)
+__device__ __forceinline__ bool fx_bad(unsigned hi_max) {
+  const unsigned f = fx_field(hi_max);
+  return f > 1223u || (f < 823u && hi_max != 0u);
+}
+// e with every |v| of the group < 2^e (an all-zero group: the smallest)
+__device__ __forceinline__ int fx_exp(unsigned hi_max) { return max((int)fx_field(hi_max), 823) - 1022; }
+
+// v 2^(BITS - e), |v| < 2^e, truncated towards zero
+template <int BITS>
+__device__ __forceinline__ long long fx_from(double v, int e) {
+  const int hi = __double2hiint(v);
+  const int r = min(e + 1022 - ((hi >> 20) & 0x7ff), 63);  // >= 0 within the group
+  const unsigned long long m =
+      ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(v)) << (BITS - 53);
+  const long long q = (long long)(m >> (r & 63));
+  const long long s = hi >> 31;
+  return (q ^ s) - s;
+}
+// x 2^-p rounded to FP64 (|p| < 900)
+__device__ __forceinline__ double fx_to(long long x, int p) {
+  const long long s = x >> 63;
+  const unsigned long long m = (unsigned long long)((x ^ s) - s);
+  const int lz = __clzll((long long)m);
+  const unsigned long long f = m << (lz & 63);                     // leading one at bit 63
+  const unsigned long long q = (f >> 11) + ((f >> 10) & 1ull);     // 53 bits, rounded (a carry gives 2^53)
+  // the implicit bit adds one to the exponent field
+  const unsigned long long b = q + ((unsigned long long)(unsigned)(1023 + 63 - lz - p - 1) << 52);
+  return m ? __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull))) : 0.0;
+}
+
+// a node plane with pads (fx_pad), an even number of words: planes of 16-byte
+// pairs start 16-byte aligned behind any number of planes
+template <int n>
+__host__ __device__ constexpr int fx_plane() {
+  return (n * n * n + n * n + n + 1) & ~1;
+}
+
+// Threads per element: a multiple of a warp (so that a warp's maxima are one
+// element's) or, at N = 1, eight.  The two-point sums give each warp whole
+// lines (LW lanes): the threads per element are those that leave few lanes
+// idle there and in the node loops.
+template <int N>
+struct Fix {
+  static constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
+  static constexpr int TPE = n == 2 ? 8 : n == 3 ? 32 : n == 4 ? 64 : n == 5 ? 160 : n == 6 ? 128 : n == 7 ? 224 : 256;
+  static constexpr int W = TPE >= 32 ? TPE / 32 : 1;            // warps per element
+  static constexpr int LW = TPE >= 32 ? 32 / n * n : TPE;       // lanes of a warp (or element) that hold whole lines
+  static constexpr int R = (n3 + TPE - 1) / TPE;                // nodes per thread
+  static constexpr int RL = (n3 + W * LW - 1) / (W * LW);       // the same in whole lines per warp
+  static constexpr int Pn = fx_plane<n>();
+  static constexpr int D = Shape<N>::EPB_DEFAULT;
+  static constexpr bool lift2 = 2 * D * n3 <= 1024, vol2 = 2 * D * n3 <= 512;
+  // launch bounds: the largest block of the variants
+  static constexpr int TL = TPE * (lift2 ? 2 * D : D), TV = TPE * (vol2 ? 2 * D : D);
+  static constexpr int min_blocks(int threads) { return threads <= 256 ? 2 : 1; }
+};
+
+// padded plane index: one pad after each line and each layer of nodes, so
+// that lines along all three directions fall in distinct banks
+template <int n>
+__device__ __forceinline__ int fx_pad(int v) {
+  return v + v / n + v / (n * n);
+}
+
+// The maxima of Q values over the element's threads: each thread gives its
+// own in m; they are in out[Q] (the element's shared memory) for the threads
+// of the element's first warp when the call returns.  red: [W][Q] words.
+template <int N, int Q>
+__device__ __forceinline__ void fx_reduce(unsigned m[Q], unsigned* red, unsigned* out, int t) {
+  using F = Fix<N>;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    if constexpr (F::TPE < 32) {
+#pragma unroll
+      for (int o = F::TPE / 2; o > 0; o >>= 1) m[k] = max(m[k], __shfl_xor_sync(0xffffffffu, m[k], o));
+    } else {
+      m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+    }
+  }
+  if (t % 32 == 0) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) red[(t / 32) * Q + k] = m[k];
+  }
+  __syncwarp();
+  __syncthreads();
+  if (t < 32)
+    for (int k = t; k < Q; k += F::TPE < 32 ? F::TPE : 32) {
+      unsigned x = red[k];
+#pragma unroll
+      for (int w = 1; w < F::W; ++w) x = max(x, red[w * Q + k]);
+      out[k] = x;
+    }
+  __syncwarp();
+}
+// the largest magnitude of a group (its high word) over 2^e, from above
+__device__ __forceinline__ float fx_frac(unsigned hi, int e) {
+  const int x = (int)fx_field(hi) - 1022 - e;
+  return hi == 0u || x < -100 ? 0.0f : __uint_as_float(((unsigned)(126 + x) << 23) | ((hi & 0xfffffu) << 3)) * 1.00001f;
+}
+// the largest S in 0 .. 31 with b 2^S <= 2^top
+__device__ __forceinline__ int fx_room(float b, int top) {
+  const int l = (int)((__float_as_uint(b) + 0x7fffffu) >> 23) - 127;  // b <= 2^l
+  return max(0, min(31, top - l));
+}
+
+// ConsToPrim in FP64 (the FP64 path's references are zero)
+struct Prim64 {
+  double rho, u, v, w, p, ri;
+};
+__device__ __forceinline__ Prim64 prim64(const double U[5], double gm1) {
+  Prim64 q;
+  q.rho = U[0];
+  q.ri = 1.0 / U[0];
+  q.u = U[1] * q.ri, q.v = U[2] * q.ri, q.w = U[3] * q.ri;
+  q.p = gm1 * (U[4] - 0.5 * (U[1] * q.u + U[2] * q.v + U[3] * q.w));
+  return q;
+}
+template <int n>
+__device__ __forceinline__ void load_state64(const StageArgs& a, int e, int v, double U[5]) {
+  constexpr int n3 = n * n * n;
+  const double* u = a.U + (size_t)e * 5 * n3 + v;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) U[k] = u[k * n3];
+}
+template <int n>
+__device__ __forceinline__ int line_base(int d, int l) {
+  const int lp = l % n, lq = l / n;
+  return d == 0 ? n * l : (d == 1 ? lp + n * n * lq : l);
+}
+
+// the element of a block's slot and whether its results are stored (slots
+// past the end redo the last element; free slots of a serving pool and
+// elements of cases that sit the step out store nothing)
+struct ElemRef {
+  int e, ce;
+  bool valid, busy;
+};
+__device__ __forceinline__ ElemRef elem_ref(const StageArgs& a, int slot) {
+  ElemRef r;
+  const int ei = slot < a.E ? slot : a.E - 1;
+  r.e = a.elem_list ? a.elem_list[ei] : ei;
+  r.ce = a.elem_case ? a.elem_case[r.e] : 0;
+  r.valid = slot < a.E && r.ce >= 0;
+  r.busy = r.valid && !(a.cases && a.cases[r.ce].dt == 0.0);
+  return r;
+}
+
+// ---------------------------------------------------------------------------
+// Lifted gradients (Eq. lifting)
+// ---------------------------------------------------------------------------
+// shared memory: the tables, the reduction words, then per element the q
+// planes (4), two buffers of one direction's metric planes (2 x 3) and the
+// sums (12), all padded node planes
+template <int N>
+struct LiftFix {
+  using F = Fix<N>;
+  static constexpr int h = F::n / 2;
+  static constexpr int ntab = F::n % 2 == 0 ? 2 * h * h : F::n2;  // split table entries
+  static constexpr int planes = 22;
+  static constexpr int Q = 5, nred = F::W * Q + Q;  // maxima: velocity, temperature, metrics by Cartesian component
+  static constexpr size_t head(int epb) { return (8 * ntab + 4 * (size_t)epb * nred + 15) & ~size_t(15); }
+  static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * planes * F::Pn; }
+};
+
+template <int n>
+__device__ void lift_direct(const StageArgs& a, int e, int v, double acc[12]);
+
+template <int N>
+__global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_lift_fx(StageArgs a) {
+  using F = Fix<N>;
+  using L = LiftFix<N>;
+  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn, h = L::h;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
+  Fx* sD = reinterpret_cast<Fx*>(smraw);
+  unsigned* red = reinterpret_cast<unsigned*>(smraw + 8 * L::ntab) + le * L::nred;
+  long long* q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::planes * Pn;
+  long long* J = q + 4 * Pn;   // [2][3][Pn]
+  long long* W = J + 6 * Pn;   // [12][Pn]
+  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
+  if (a.elem_case && __syncthreads_and(!er.busy)) return;
+  const int e = er.e;
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+  for (int k = threadIdx.x; k < L::ntab; k += blockDim.x)
+    sD[k] = n % 2 == 0 ? fx_split(k < h * h ? a.ops->fxHe[k] : a.ops->fxHo[k - h * h]) : fx_split(a.ops->fxH[k]);
+  // primitives (FP64, in the q planes until the scales are known) and maxima
+  unsigned m[5] = {0, 0, 0, 0, 0};
+  for (int v = t; v < n3; v += TPE) {
+    double U[5];
+    load_state64<n>(a, e, v, U);
+    const Prim64 pr = prim64(U, a.gm1);
+    const double T = pr.p * pr.ri * a.Rinv;
+    double* qd = reinterpret_cast<double*>(q) + fx_pad<n>(v);
+    qd[0] = pr.u, qd[Pn] = pr.v, qd[2 * Pn] = pr.w, qd[3 * Pn] = T;
+    m[0] = max(max(m[0], fx_mag(pr.u)), max(fx_mag(pr.v), fx_mag(pr.w)));
+    m[1] = max(m[1], fx_mag(T));
+#pragma unroll
+    for (int c = 0; c < 9; ++c) m[2 + c % 3] = max(m[2 + c % 3], fx_mag(Me[c * n3 + v]));
+  }
+  unsigned* fin = red + F::W * L::Q;
+  fx_reduce<N, 5>(m, red, fin, t);
+  __syncthreads();
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) bad = bad || fx_bad(fin[k]);
+  const int eU = fx_exp(fin[0]), eT = fx_exp(fin[1]), eJ[3] = {fx_exp(fin[2]), fx_exp(fin[3]), fx_exp(fin[4])};
+  for (int v = t; v < n3; v += TPE) {
+    const int pv = fx_pad<n>(v);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      long long* x = q + k * Pn + pv;
+      *x = fx_from<61>(__longlong_as_double(*x), k < 3 ? eU : eT);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) J[c * Pn + pv] = fx_from<60>(Me[c * n3 + v], eJ[c]);
+  }
+  __syncwarp();
+  __syncthreads();
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    const int sd = dir_stride<n>(d);
+    const long long* Jd = J + (d & 1) * 3 * Pn;
+    for (int task = t; task < 4 * n2; task += TPE) {
+      const int qv = task / n2, bl = line_base<n>(d, task % n2);
+      Fx ql[n];
+#pragma unroll
+      for (int al = 0; al < n; ++al) ql[al] = fx_split(q[qv * Pn + fx_pad<n>(bl + al * sd)]);
+#pragma unroll 1
+      for (int x = 0; x < 3; ++x) {
+        long long P[n];  // Ja^d_x q: |P| <= 2^(60 + 61 - 64 + 2)
+#pragma unroll
+        for (int al = 0; al < n; ++al) {
+          FxSum<2> s;
+          s.add(fx_split(Jd[x * Pn + fx_pad<n>(bl + al * sd)]), ql[al]);
+          P[al] = s.get();
+        }
+        long long* w = W + (qv * 3 + x) * Pn;
+        auto put = [&](int i, long long y) {
+          long long* o = w + fx_pad<n>(bl + i * sd);
+          *o = d == 0 ? y : *o + y;
+        };
+        // the rows of Dhat sum to at most 2^62: |y| <= 2^(62 + 59 - 64 + 3), three directions below 2^62
+        if constexpr (n % 2 == 0) {
+          // Dhat is centro-antisymmetric: even and odd halves (dg_types.h)
+          Fx E[h], O[h];
+#pragma unroll
+          for (int j = 0; j < h; ++j) E[j] = fx_split(P[j] + P[n - 1 - j]), O[j] = fx_split(P[j] - P[n - 1 - j]);
+#pragma unroll
+          for (int i = 0; i < h; ++i) {
+            FxSum<3> ev, od;
+#pragma unroll
+            for (int j = 0; j < h; ++j) ev.add(sD[i * h + j], E[j]), od.add(sD[h * h + i * h + j], O[j]);
+            const long long ye = ev.get(), yo = od.get();
+            put(i, yo + ye);
+            put(n - 1 - i, yo - ye);
+          }
+        } else {
+          Fx Ps[n];
+#pragma unroll
+          for (int j = 0; j < n; ++j) Ps[j] = fx_split(P[j]);
+#pragma unroll
+          for (int i = 0; i < n; ++i) {
+            FxSum<3> s;
+#pragma unroll
+            for (int j = 0; j < n; ++j) s.add(sD[i * n + j], Ps[j]);
+            put(i, s.get());
+          }
+        }
+      }
+    }
+    if (d < 2) {  // the next direction's metrics into the other buffer
+      long long* Jn = J + ((d + 1) & 1) * 3 * Pn;
+      for (int v = t; v < n3; v += TPE)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Jn[c * Pn + fx_pad<n>(v)] = fx_from<60>(Me[(3 * d + 3 + c) * n3 + v], eJ[c]);
+    }
+    __syncwarp();
+    __syncthreads();
+  }
+  if (!er.valid) return;
+  const int pU = a.ops->fxH_bits - 2 - eU, pT = a.ops->fxH_bits - 2 - eT;
+  const double* Lf = a.lflux;
+  for (int v = t; v < n3; v += TPE) {
+    const int pv = fx_pad<n>(v);
+    double acc[12];
+    if (bad) {
+      double d12[12];
+      lift_direct<n>(a, e, v, d12);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[k] = d12[k];
+    } else {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[k] = fx_to(W[k * Pn + pv], (k < 9 ? pU : pT) - eJ[k % 3]);
+    }
+    // surface part: on LGL nodes only face nodes receive it
+    const int idx[3] = {v % n, (v / n) % n, v / n2};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int id = idx[d];
+      if (id != 0 && id != n - 1) continue;
+      const int f = 2 * d + (id == n - 1 ? 1 : 0);
+      const int es = a.elem_side[(size_t)e * 6 + f];
+      int p, qq;
+      face_pq(d, idx, p, qq);
+      int pm = p, qm = qq;
+      if (es_slave(es)) flip_to_master<n>(es_flip(es), p, qq, pm, qm);
+      const double sg = es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id];
+      const double* Lr = Lf + (size_t)es_side(es) * 12 * n2 + pm + n * qm;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) acc[k] += sg * Lr[k * n2];
+    }
+    const double Ji = Me[9 * n3 + v];
+    double* g = a.g + (size_t)e * 12 * n3 + v;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) g[k * n3] = acc[k] * Ji;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Volume integral + SurfInt + ApplyJac (+ RK update)
+// ---------------------------------------------------------------------------
+// Scales of an element's two-point sums, from its groups' maxima.  For each
+// direction the shifts bring every product's bound (from the actual maxima,
+// component by component) next to 2^62, so that no bits go to loose bounds
+// or to anisotropic metrics; the directions' sums are aligned at the end.
+struct DirScale {
+  int eJ;                      // exponent of the direction's metrics
+  int s1, s2, s3, s4, s5, s6;  // shifts of un, fr, t, pressure, momentum, energy (kep_fx)
+  int kc;                      // right shift of t in the momentum flux (aligns it with the pressure)
+  int aM, aV, aE;              // right shifts of the direction's mass, momentum and energy sums
+};
+struct VolScale {
+  DirScale d[3];
+  int eR, eU, eP, eH;
+  int pM, pV, pE;  // results: sums times 2^-p
+  int c[3][3];     // the directions' own scales
+  int bad;
+};
+enum { VQ_RHO, VQ_U, VQ_V, VQ_W, VQ_P, VQ_H, VQ_RHOH, VQ_MOM, VQ_J, VQ_N = VQ_J + 9 };
+
+// threads 0 .. 2 of the element, one direction each; Q = maxima
+__device__ __forceinline__ void vol_scale(VolScale& s, const unsigned* m, const Ops* o, int t) {
+  const int eR = fx_exp(m[VQ_RHO]), eU = fx_exp(max(max(m[VQ_U], m[VQ_V]), m[VQ_W])), eP = fx_exp(m[VQ_P]),
+            eH = fx_exp(m[VQ_H]);
+  const unsigned* mj = m + VQ_J + 3 * t;
+  const int eJ = fx_exp(max(max(mj[0], mj[1]), mj[2]));
+  const float fR = fx_frac(m[VQ_RHO], eR), fP = fx_frac(m[VQ_P], eP), fH = fx_frac(m[VQ_H], eH), fS = o->fxS_row;
+  const float u0 = fx_frac(m[VQ_U], eU), u1 = fx_frac(m[VQ_V], eU), u2 = fx_frac(m[VQ_W], eU);
+  const float j0 = fx_frac(mj[0], eJ), j1 = fx_frac(mj[1], eJ), j2 = fx_frac(mj[2], eJ);
+  DirScale& d = s.d[t];
+  d.eJ = eJ;
+  // bounds in units of 2^58 (un), 2^60 and 2^61 (the others)
+  float b = u0 * j0 + u1 * j1 + u2 * j2;
+  d.s1 = fx_room(b, 4);
+  b = fR * ldexpf(b, d.s1 - 4);  // fr / 2^60
+  d.s2 = fx_room(b, 2);
+  b = fS * ldexpf(b, d.s2 - 2);  // t / 2^60, summed over a row
+  d.s3 = fx_room(b, 1);
+  const float bt = ldexpf(b, d.s3 - 1);  // t / 2^61
+  const float bp0 = fS * fP;             // pressure / 2^60
+  d.s4 = fx_room(bp0, 2);
+  // scales: value times 2^a
+  const int a3 = o->fxS_bits + 61 - eR + 56 - eU - eJ + d.s1 - 128 + d.s2 + d.s3;
+  const int b3 = o->fxS_bits + 61 - eP - 64 + d.s4;
+  const int delta = (a3 - eU + 2) - (b3 - eJ);
+  d.kc = min(max(delta, 0), 62);
+  const int kp = max(-delta, 0);
+  float bp = ldexpf(bp0, d.s4 - 1);  // pressure / 2^61
+  bp = ldexpf(bp, -kp);
+  d.s4 -= kp;  // (below zero: a right shift, see kep_fx)
+  const float bm = ldexpf(bt, -d.kc) * fmaxf(u0, fmaxf(u1, u2)) + bp * fmaxf(j0, fmaxf(j1, j2));  // momentum / 2^58
+  d.s5 = fx_room(bm, 3);
+  const float be = bt * fH;  // energy / 2^59
+  d.s6 = fx_room(be, 2);
+  // the means' factors 1/8 (mass), 1/4 (pressure) and 1/16 (energy) included; 1/w (fxW)
+  const int w = o->fxW_bits - 62;
+  s.c[t][0] = a3 + 3 + w;
+  s.c[t][1] = b3 - kp - eJ - 2 + d.s5 + w;
+  s.c[t][2] = a3 - eH + 1 + d.s6 + w;
+  __syncwarp(__activemask());
+  int p[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) p[k] = min(min(s.c[0][k], s.c[1][k]), s.c[2][k]);
+  d.aM = min(s.c[t][0] - p[0], 63), d.aV = min(s.c[t][1] - p[1], 63), d.aE = min(s.c[t][2] - p[2], 63);
+  if (t == 0) {
+    s.eR = eR, s.eU = eU, s.eP = eP, s.eH = eH;
+    s.pM = p[0], s.pV = p[1], s.pE = p[2];
+    // In FP64: groups out of range, and elements whose largest fluxes lie far
+    // below the product of their groups' maxima (light and fast or hot fluid
+    // beside dense fluid, ratios above four): their scale would leave the
+    // fluxes fewer bits than FP64 gives them.
+    bool bad = false;
+    for (int k = 0; k < VQ_N; ++k) bad = bad || fx_bad(m[k]);
+    const int eX = fx_exp(m[VQ_RHOH]), eM = fx_exp(m[VQ_MOM]);
+    const int lh = min(max(eR + eH - eX, -60), 60), lm = min(max(eR + eU - eM, -60), 60);
+    bad = bad || fR * fH * ldexpf(1.0f, lh) > 4.0f * fx_frac(m[VQ_RHOH], eX);
+    bad = bad || fR * fmaxf(u0, fmaxf(u1, u2)) * ldexpf(1.0f, lm) > 4.0f * fx_frac(m[VQ_MOM], eM);
+    s.bad = bad;
+  }
+}
+
+// shared memory: S = w Dsplit, 1/w and Dhat split (Fx), Vinv, the reduction
+// words and scales, then per element: the metrics (3 directions of (m0, m1)
+// pairs and of m2), the primitives (pairs (rho, p), (u, v), (w, H)) and the
+// two-point sums (5), all padded.  The viscous fluxes of one direction (pairs
+// (f1, f2), (f3, f4), padded), the stress tensor and heat vector (9 planes,
+// each thread's own nodes only) and the shock scratch take the place of the
+// primitives and sums afterwards.
+template <int N>
+struct VolFix {
+  using F = Fix<N>;
+  static constexpr int offP = 9 * F::Pn;  // in 64-bit words
+  static constexpr int offA = offP + 6 * F::Pn;
+  static constexpr int offT = offP + 4 * F::Pn;  // after the viscous fluxes
+  static constexpr int end1 = offA + 5 * F::Pn, end2 = offT + 9 * F::n3, end3 = offP + 2 * F::n3 + 4 * F::n2;
+  static constexpr int end12 = end1 > end2 ? end1 : end2;
+  static constexpr int per_elem = ((end12 > end3 ? end12 : end3) + 1) & ~1;
+  static constexpr int nred = F::W * VQ_N + VQ_N;
+  static constexpr int nscale = (int)(sizeof(VolScale) / 4);
+  static constexpr int ntab = 3 * F::n2 + F::n;
+  static constexpr size_t head(int epb) { return (8 * ntab + 4 * (size_t)epb * (nred + nscale) + 15) & ~size_t(15); }
+  static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * per_elem; }
+  static_assert(offP % 2 == 0 && per_elem % 2 == 0 && (6 * F::Pn) % 2 == 0, "16-byte alignment of the pair planes");
+};
+
+// One two-point flux of KEP type, times S: (t, f1, f2, f3, f4)
+struct KepNode {
+  longlong2 a0, a1, a2, j0;  // (rho, p), (u, v), (w, H), (m0, m1)
+  long long j1;              // m2
+};
+template <int n>
+__device__ __forceinline__ KepNode kep_load(const longlong2* P, const longlong2* Jab, const long long* Jc, int pv) {
+  constexpr int Pn = fx_plane<n>();
+  return {P[pv], P[Pn + pv], P[2 * Pn + pv], Jab[pv], Jc[pv]};
+}
+__device__ __forceinline__ void kep_flux_fx(const KepNode& x, const KepNode& y, Fx S, const DirScale& d, long long f[5]) {
+  // sums of two values: u and m below 2^61, rho, p and H below 2^62; every
+  // result below 2^62 by the choice of its shift
+  const Fx m0 = fx_split(x.j0.x + y.j0.x), m1 = fx_split(x.j0.y + y.j0.y), m2 = fx_split(x.j1 + y.j1);
+  const Fx u0 = fx_split(x.a1.x + y.a1.x), u1 = fx_split(x.a1.y + y.a1.y), u2 = fx_split(x.a2.x + y.a2.x);
+  FxSumS un, fr, tt, pd, f1, f2, f3, f4;
+  un.add(u0, m0), un.add(u1, m1), un.add(u2, m2);
+  fr.add(fx_split(x.a0.x + y.a0.x), fx_split(un.get(d.s1)));
+  tt.add(S, fx_split(fr.get(d.s2)));
+  f[0] = tt.get(d.s3);
+  const Fx tk = fx_split(f[0] >> d.kc);
+  pd.add(S, fx_split(x.a0.y + y.a0.y));
+  const Fx ps = fx_split(d.s4 >= 0 ? pd.get(d.s4) : pd.get(0) >> min(-d.s4, 63));
+  f1.add(tk, u0), f1.add(ps, m0);
+  f2.add(tk, u1), f2.add(ps, m1);
+  f3.add(tk, u2), f3.add(ps, m2);
+  f[1] = f1.get(d.s5), f[2] = f2.get(d.s5), f[3] = f3.get(d.s5);
+  f4.add(fx_split(f[0]), fx_split(x.a2.y + y.a2.y));
+  f[4] = f4.get(d.s6);
+}
+
+// Split-form KEP sums of all nodes: each thread takes one node of a line that
+// its warp holds whole, forms the fluxes to the partners 1 .. (n - 1) / 2
+// places on (cyclically), adds them to its own sums and passes them to the
+// partner, whose S has the opposite sign (S = w Dsplit is antisymmetric); for
+// even n the partner n / 2 places on is taken from both sides.  That is 3 + 1
+// fluxes per node and direction at n = 8 where every node summing over all
+// its partners takes 7.
+template <int N>
+__device__ __forceinline__ void kep_fx(const longlong2* P, const longlong2* Jab, const long long* Jc, long long* A,
+                                       const Fx* sS, const Fx* sW, const VolScale* sc, int t, bool skip) {
+  using F = Fix<N>;
+  constexpr int n = F::n, n3 = F::n3, Pn = F::Pn, LW = F::LW;
+  const int lane = F::TPE >= 32 ? t & 31 : t;
+  const int lane0 = F::TPE >= 32 ? 0 : (threadIdx.x & 31) - t;  // the element's first lane
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    const DirScale ds = sc->d[d];
+    const int sd = dir_stride<n>(d);
+    const longlong2* Jd = Jab + d * Pn;
+    const long long* Jcd = Jc + d * Pn;
+#pragma unroll 1
+    for (int r = 0; r < F::RL; ++r) {
+      const int slot = ((t / 32) + r * F::W) * LW + lane;
+      const bool on = lane < LW && slot < n3 && !skip;
+      const int line = on ? slot / n : 0, id = lane % n, base = line_base<n>(d, line);
+      const int pv = fx_pad<n>(base + id * sd);
+      long long acc[5] = {0, 0, 0, 0, 0};
+      const KepNode me = kep_load<n>(P, Jd, Jcd, pv);
+#pragma unroll 1
+      for (int k = 1; k <= (n - 1) / 2; ++k) {
+        const int al = id + k < n ? id + k : id + k - n, from = id >= k ? id - k : id - k + n;
+        long long f[5];
+        kep_flux_fx(me, kep_load<n>(P, Jd, Jcd, fx_pad<n>(base + al * sd)), sS[id * n + al], ds, f);
+        const int src = min(lane0 + lane - id + from, 31);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[c] += f[c] - __shfl_sync(0xffffffffu, f[c], src);
+      }
+      if constexpr (n % 2 == 0) {
+        const int al = id < n / 2 ? id + n / 2 : id - n / 2;
+        long long f[5];
+        kep_flux_fx(me, kep_load<n>(P, Jd, Jcd, fx_pad<n>(base + al * sd)), sS[id * n + al], ds, f);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[c] += f[c];
+      }
+      if (on) {
+        const Fx wi = sW[id];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          FxSum<2> y;  // 2^(61 + 62 - 64 + 2)
+          y.add(wi, fx_split(acc[c]));
+          const long long z = y.get() >> (c == 0 ? ds.aM : c == 4 ? ds.aE : ds.aV);
+          A[c * Pn + pv] = d == 0 ? z : A[c * Pn + pv] + z;
+        }
+      }
+    }
+    __syncwarp();
+    __syncthreads();
+  }
+}
+// the same in FP64, one node: P and J hold FP64 values
+template <int n>
+__device__ void kep_f64(const double2* P, const double2* Jab, const double* Jc, const double* Dsplit, int v,
+                        double conv[5]) {
+  constexpr int Pn = fx_plane<n>();
+  const int pv = fx_pad<n>(v);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) conv[k] = 0.0;
+  const double2 a0 = P[pv], a1 = P[Pn + pv], a2 = P[2 * Pn + pv];
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    const int id = dir_index<n>(v, d), sd = dir_stride<n>(d), base = v - id * sd;
+    const double2 j0 = Jab[d * Pn + pv];
+    const double j1 = Jc[d * Pn + pv];
+#pragma unroll 1
+    for (int al = 0; al < n; ++al) {
+      if (al == id) continue;
+      const int pa = fx_pad<n>(base + al * sd);
+      const double2 b0 = P[pa], b1 = P[Pn + pa], b2 = P[2 * Pn + pa], c0 = Jab[d * Pn + pa];
+      const double m0 = j0.x + c0.x, m1 = j0.y + c0.y, m2 = j1 + Jc[d * Pn + pa];  // twice the means
+      const double u0 = a1.x + b1.x, u1 = a1.y + b1.y, u2 = a2.x + b2.x;
+      const double D = 0.125 * Dsplit[id * n + al], p = 2.0 * (a0.y + b0.y);
+      const double fr = (a0.x + b0.x) * (u0 * m0 + u1 * m1 + u2 * m2), hf = 0.5 * fr;
+      conv[0] += D * fr;
+      conv[1] += D * (hf * u0 + p * m0);
+      conv[2] += D * (hf * u1 + p * m1);
+      conv[3] += D * (hf * u2 + p * m2);
+      conv[4] += D * (hf * (a2.y + b2.y));
+    }
+  }
+}
+
+template <int N, int MODE>
+__global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_volume_fx(StageArgs a) {
+  using F = Fix<N>;
+  using L = VolFix<N>;
+  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn, R = F::R;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
+  Fx* sS = reinterpret_cast<Fx*>(smraw);  // [n2] w Dsplit
+  Fx* sDh = sS + n2;                      // [n2] Dhat
+  Fx* sW = sDh + n2;                      // [n] 1 / w
+  double* sVi = reinterpret_cast<double*>(sW + n);
+  unsigned* red = reinterpret_cast<unsigned*>(sVi + n2) + le * (L::nred + L::nscale);
+  unsigned* fin = red + F::W * VQ_N;
+  VolScale* sc = reinterpret_cast<VolScale*>(fin + VQ_N);
+  long long* mine = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::per_elem;
+  longlong2* Jab = reinterpret_cast<longlong2*>(mine);  // [3][Pn] (m0, m1)
+  long long* Jc = mine + 6 * Pn;                        // [3][Pn] m2
+  long long* PT = mine + L::offP;
+  longlong2* P = reinterpret_cast<longlong2*>(PT);      // [3][Pn]
+  long long* A = mine + L::offA;                        // [5][Pn]
+  longlong2* G = P;                                     // [2][Pn] (after the two-point sums)
+  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
+  if (a.elem_case && __syncthreads_and(!er.busy)) return;
+  const int e = er.e;
+  const CaseParams cp = case_params(a, er.ce);
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+  for (int k = threadIdx.x; k < n2; k += blockDim.x) {
+    sS[k] = fx_split(a.ops->fxS[k]);
+    sDh[k] = fx_split(a.ops->fxH[k]);
+    sVi[k] = a.ops->Vinv[k];
+    if (k < n) sW[k] = fx_split(a.ops->fxW[k]);
+  }
+  // ---- primitives (FP64 in their planes until the scales are known), maxima ----
+  {
+    unsigned m[VQ_N];
+#pragma unroll
+    for (int k = 0; k < VQ_N; ++k) m[k] = 0;
+    for (int v = t; v < n3; v += TPE) {
+      double U[5];
+      load_state64<n>(a, e, v, U);
+      const Prim64 pr = prim64(U, a.gm1);
+      const double rH = U[4] + pr.p, H = rH * pr.ri;
+      double2* Pd = reinterpret_cast<double2*>(P) + fx_pad<n>(v);
+      Pd[0] = make_double2(pr.rho, pr.p);
+      Pd[Pn] = make_double2(pr.u, pr.v);
+      Pd[2 * Pn] = make_double2(pr.w, H);
+      m[VQ_RHO] = max(m[VQ_RHO], fx_mag(pr.rho));
+      m[VQ_U] = max(m[VQ_U], fx_mag(pr.u));
+      m[VQ_V] = max(m[VQ_V], fx_mag(pr.v));
+      m[VQ_W] = max(m[VQ_W], fx_mag(pr.w));
+      m[VQ_P] = max(m[VQ_P], fx_mag(pr.p));
+      m[VQ_H] = max(m[VQ_H], fx_mag(H));
+      m[VQ_RHOH] = max(m[VQ_RHOH], fx_mag(rH));
+      m[VQ_MOM] = max(max(m[VQ_MOM], fx_mag(U[1])), max(fx_mag(U[2]), fx_mag(U[3])));
+#pragma unroll
+      for (int c = 0; c < 9; ++c) m[VQ_J + c] = max(m[VQ_J + c], fx_mag(Me[c * n3 + v]));
+    }
+    fx_reduce<N, VQ_N>(m, red, fin, t);
+    if (t < 3) vol_scale(*sc, fin, a.ops, t);
+    __syncwarp();
+    __syncthreads();
+  }
+  const bool bad = sc->bad != 0;
+  for (int v = t; v < n3; v += TPE) {
+    const int pv = fx_pad<n>(v);
+    double mt[9];
+#pragma unroll
+    for (int c = 0; c < 9; ++c) mt[c] = Me[c * n3 + v];
+    if (bad) {  // FP64 values
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        reinterpret_cast<double2*>(Jab)[d * Pn + pv] = make_double2(mt[3 * d], mt[3 * d + 1]);
+        reinterpret_cast<double*>(Jc)[d * Pn + pv] = mt[3 * d + 2];
+      }
+    } else {
+      const double2* Pd = reinterpret_cast<const double2*>(P) + pv;
+      const double2 x0 = Pd[0], x1 = Pd[Pn], x2 = Pd[2 * Pn];
+      P[pv] = make_longlong2(fx_from<61>(x0.x, sc->eR), fx_from<61>(x0.y, sc->eP));
+      P[Pn + pv] = make_longlong2(fx_from<60>(x1.x, sc->eU), fx_from<60>(x1.y, sc->eU));
+      P[2 * Pn + pv] = make_longlong2(fx_from<60>(x2.x, sc->eU), fx_from<61>(x2.y, sc->eH));
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int eJ = sc->d[d].eJ;
+        Jab[d * Pn + pv] = make_longlong2(fx_from<60>(mt[3 * d], eJ), fx_from<60>(mt[3 * d + 1], eJ));
+        Jc[d * Pn + pv] = fx_from<60>(mt[3 * d + 2], eJ);
+      }
+    }
+  }
+  __syncwarp();
+  __syncthreads();
+  // ---- split-form KEP volume integral ----
+  kep_fx<N>(P, Jab, Jc, A, sS, sW, sc, t, bad);
+  double conv[R][5];  // convective DG volume term
+  double visc[R][4];  // viscous volume term
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int v = t + r * TPE, pv = fx_pad<n>(v < n3 ? v : 0);
+    if (bad) {
+      double c5[5] = {0, 0, 0, 0, 0};
+      if (v < n3)
+        kep_f64<n>(reinterpret_cast<const double2*>(P), reinterpret_cast<const double2*>(Jab),
+                   reinterpret_cast<const double*>(Jc), a.ops->Dsplit, v, c5);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) conv[r][k] = c5[k];
+    } else {
+      conv[r][0] = fx_to(A[pv], sc->pM);
+#pragma unroll
+      for (int k = 1; k < 4; ++k) conv[r][k] = fx_to(A[k * Pn + pv], sc->pV);
+      conv[r][4] = fx_to(A[4 * Pn + pv], sc->pE);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) visc[r][k] = 0.0;
+  }
+  __syncwarp();
+  __syncthreads();  // the primitives' and sums' planes are free
+  // ---- viscous volume term: collocated weak form, per direction ----
+  if (a.viscous) {
+    long long* T = mine + L::offT;  // [9][n3]: tau, W; each thread reads back its own nodes only
+    {
+      unsigned mv[2] = {0, 0};
+      for (int v = t; v < n3; v += TPE) {
+        double g[12], U[5];
+        const double* pg = a.g + (size_t)e * 12 * n3 + v;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) g[k] = pg[k * n3];
+        load_state64<n>(a, e, v, U);
+        const Prim64 pr = prim64(U, a.gm1);
+        double tau[6], W[3], vmu, vlam;
+        visc_coeffs<double>(a, cp, a.sutherland ? pr.p * pr.ri * a.Rinv : 0.0, vmu, vlam);
+        viscous_parts(g, pr.u, pr.v, pr.w, vmu, vlam, tau, W);
+        double* Td = reinterpret_cast<double*>(T) + v;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) Td[k * n3] = tau[k], mv[0] = max(mv[0], fx_mag(tau[k]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) Td[(6 + k) * n3] = W[k], mv[1] = max(mv[1], fx_mag(W[k]));
+      }
+      fx_reduce<N, 2>(mv, red, fin, t);
+      __syncthreads();
+    }
+    // (an element that leaves the range only here has its metrics in fixed
+    // point: the FP64 sums then read them from memory)
+    const bool vbad = bad || fx_bad(fin[0]) || fx_bad(fin[1]);
+    const int eT = fx_exp(fin[0]), eW = fx_exp(fin[1]), eJm = max(max(sc->d[0].eJ, sc->d[1].eJ), sc->d[2].eJ);
+    long long acc[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[r][k] = 0;
+    if (!vbad)
+      for (int v = t; v < n3; v += TPE)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) T[k * n3 + v] = fx_from<60>(__longlong_as_double(T[k * n3 + v]), k < 6 ? eT : eW);
+#pragma unroll 1
+    for (int d = 0; d < 3; ++d) {
+      for (int v = t; v < n3; v += TPE) {
+        const int pv = fx_pad<n>(v);
+        if (vbad) {
+          const double* Td = reinterpret_cast<const double*>(T) + v;
+          double tau[6], W[3], fv[4];
+          const double nv[3] = {Me[3 * d * n3 + v], Me[(3 * d + 1) * n3 + v], Me[(3 * d + 2) * n3 + v]};
+#pragma unroll
+          for (int k = 0; k < 6; ++k) tau[k] = Td[k * n3];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) W[k] = Td[(6 + k) * n3];
+          viscous_flux_n(tau, W, nv, fv);
+          reinterpret_cast<double2*>(G)[pv] = make_double2(fv[0], fv[1]);
+          reinterpret_cast<double2*>(G)[Pn + pv] = make_double2(fv[2], fv[3]);
+        } else {
+          const longlong2 jab = Jab[d * Pn + pv];
+          const Fx j0 = fx_split(jab.x), j1 = fx_split(jab.y), j2 = fx_split(Jc[d * Pn + pv]);
+          Fx x[9];
+#pragma unroll
+          for (int k = 0; k < 9; ++k) x[k] = fx_split(T[k * n3 + v]);
+          FxSum<2> f1, f2, f3, f4;  // 3 2^(60 + 60 - 64 + 2) < 2^59.6
+          f1.add(x[0], j0), f1.add(x[3], j1), f1.add(x[4], j2);
+          f2.add(x[3], j0), f2.add(x[1], j1), f2.add(x[5], j2);
+          f3.add(x[4], j0), f3.add(x[5], j1), f3.add(x[2], j2);
+          f4.add(x[6], j0), f4.add(x[7], j1), f4.add(x[8], j2);
+          G[pv] = make_longlong2(f1.get(), f2.get());
+          G[Pn + pv] = make_longlong2(f3.get(), f4.get());
+        }
+      }
+      __syncwarp();
+      __syncthreads();
+      const int sd = dir_stride<n>(d);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int v = t + r * TPE;
+        if (v < n3) {
+          const int id = dir_index<n>(v, d), base = v - id * sd;
+          if (vbad) {
+            const double2* Gd = reinterpret_cast<const double2*>(G);
+            for (int al = 0; al < n; ++al) {
+              const double c = a.ops->Dhat[id * n + al];
+              const double2 g0 = Gd[fx_pad<n>(base + al * sd)], g1 = Gd[Pn + fx_pad<n>(base + al * sd)];
+              visc[r][0] += c * g0.x, visc[r][1] += c * g0.y, visc[r][2] += c * g1.x, visc[r][3] += c * g1.y;
+            }
+          } else {
+            FxSum<3> s1, s2, s3, s4;  // 2^(62 + 59.6 - 64 + 3) per direction
+#pragma unroll
+            for (int al = 0; al < n; ++al) {
+              const int pa = fx_pad<n>(base + al * sd);
+              const longlong2 g0 = G[pa], g1 = G[Pn + pa];
+              const Fx c = sDh[id * n + al];
+              s1.add(c, fx_split(g0.x)), s2.add(c, fx_split(g0.y)), s3.add(c, fx_split(g1.x)), s4.add(c, fx_split(g1.y));
+            }
+            const int sh = min(eJm - sc->d[d].eJ, 63);  // the directions' metrics have their own exponents
+            acc[r][0] += s1.get() >> sh, acc[r][1] += s2.get() >> sh, acc[r][2] += s3.get() >> sh, acc[r][3] += s4.get() >> sh;
+          }
+        }
+      }
+      __syncwarp();
+      __syncthreads();
+    }
+    const int pT = a.ops->fxH_bits - 3 - eT - eJm, pW = a.ops->fxH_bits - 3 - eW - eJm;
+    if (!vbad) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) visc[r][k] = fx_to(acc[r][k], k < 3 ? pT : pW);
+    }
+  }
+  // ---- shock capturing: indicator and FV sub-cell blending (Sec. 2.3) ----
+  if (a.shock) {
+    double al;
+    if (a.alpha_force >= 0) {
+      al = a.alpha_force;
+    } else {
+      double* X1 = reinterpret_cast<double*>(PT);
+      for (int v = t; v < n3; v += TPE) {
+        double U[5];
+        load_state64<n>(a, e, v, U);
+        X1[v] = U[0] * prim64(U, a.gm1).p;
+      }
+      al = element_alpha<n, TPE>(X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
+    }
+    if (er.valid && t == 0) a.alpha[e] = al;
+    // block-uniform condition: the FV pass has barriers, and the elements of
+    // one block may have different blending factors
+    if (__syncthreads_or(al > 0)) {
+      double* Gf = reinterpret_cast<double*>(PT);  // [5][n3]
+      double vfv[R][5];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) vfv[r][k] = 0.0;
+      const double* FVm = a.fvmetric + (size_t)e * 3 * (n - 1) * 3 * n2;
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        const int sd = dir_stride<n>(d);
+        // the flux through interface id + 1/2 is formed by the node on its left
+        for (int v = t; v < n3; v += TPE) {
+          const int id = dir_index<n>(v, d);
+          if (id == n - 1) continue;
+          const int idx[3] = {v % n, (v / n) % n, v / n2};
+          const int line = d == 0 ? idx[1] + n * idx[2] : (d == 1 ? idx[0] + n * idx[2] : idx[0] + n * idx[1]);
+          const double* fm = FVm + (size_t)(d * (n - 1) + id) * 3 * n2 + line;
+          const double mv[3] = {fm[0], fm[n2], fm[2 * n2]};
+          const double sAd = sqrt(mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2]);
+          const double sAi = 1.0 / sAd;
+          const double nu[3] = {mv[0] * sAi, mv[1] * sAi, mv[2] * sAi};
+          double UL[5], UR[5], fb[5];
+          load_state64<n>(a, e, v, UL);
+          load_state64<n>(a, e, v + sd, UR);
+          lf_flux_s(shifted_prim<double>(UL, a.gm1, a.Rinv, cp), shifted_prim<double>(UR, a.gm1, a.Rinv, cp), nu,
+                    a.gamma, cp.pr, fb);
+#pragma unroll
+          for (int k = 0; k < 5; ++k) Gf[k * n3 + v] = fb[k] * sAd;
+        }
+        __syncwarp();
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int v = t + r * TPE;
+          if (v < n3) {
+            const int id = dir_index<n>(v, d);
+            const double wi = a.ops->winv[id];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+              if (id < n - 1) vfv[r][k] += Gf[k * n3 + v] * wi;
+              if (id > 0) vfv[r][k] -= Gf[k * n3 + v - sd] * wi;
+            }
+          }
+        }
+        __syncwarp();
+        __syncthreads();
+      }
+      if (al > 0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int k = 0; k < 5; ++k) conv[r][k] = (1 - al) * conv[r][k] + al * vfv[r][k];
+      }
+    }
+  }
+  if (!er.valid) return;
+  // a serving case that finished or sits this step out keeps its state
+  if (MODE == 1 && !er.busy) return;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int v = t + r * TPE;
+    if (v >= n3) break;
+    double s[5] = {conv[r][0], conv[r][1] - visc[r][0], conv[r][2] - visc[r][1], conv[r][3] - visc[r][2],
+                   conv[r][4] - visc[r][3]};
+    // ---- SurfInt: face nodes receive +-f* lhat ----
+    const int idx[3] = {v % n, (v / n) % n, v / n2};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int id = idx[d];
+      if (id != 0 && id != n - 1) continue;
+      const int f = 2 * d + (id == n - 1 ? 1 : 0);
+      const int es = a.elem_side[(size_t)e * 6 + f];
+      int p, qq;
+      face_pq(d, idx, p, qq);
+      int pm = p, qm = qq;
+      if (es_slave(es)) flip_to_master<n>(es_flip(es), p, qq, pm, qm);
+      const double sg = es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id];
+      const double* Fs = a.fstar + (size_t)es_side(es) * 5 * n2 + pm + n * qm;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) s[k] += sg * Fs[k * n2];
+    }
+    // ---- ApplyJac, sources, Ut or the RK update ----
+    const double Ji = -Me[9 * n3 + v];
+    double Ut[5], U[5];
+    load_state64<n>(a, e, v, U);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) Ut[k] = s[k] * Ji;
+    if (a.sponge_sigma) {  // sponge source -sigma (U - U_base)
+      const double sg = a.sponge_sigma[(size_t)e * n3 + v];
+      const double* ub = a.sponge_base + (size_t)e * 5 * n3 + v;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) Ut[k] -= sg * (U[k] - ub[k * n3]);
+    }
+    if (a.source) {  // manufactured-solution source
+      double Q[5];
+      mms_source(a, a.xyzs + ((size_t)e * n3 + v) * 3, stage_time(a, MODE), Q);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) Ut[k] += Q[k];
+    }
+    if (MODE == 0) {
+      double* o = a.Ut + (size_t)e * 5 * n3 + v;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) o[k * n3] = Ut[k];
+    } else {
+      const double dt = case_dt(a, er.ce);
+      double* du = a.dU + (size_t)e * 5 * n3 + v;
+      double* uo = a.Urk + (size_t)e * 5 * n3 + v;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const double x = a.first_stage ? dt * Ut[k] : a.rkA * du[k * n3] + dt * Ut[k];
+        du[k * n3] = x;
+        uo[k * n3] = U[k] + a.rkB * x;
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The lifting's sums of one node in FP64, for elements outside the fixed-point range
+// ---------------------------------------------------------------------------
+template <int n>
+__device__ __noinline__ void lift_direct(const StageArgs& a, int e, int v, double acc[12]) {
+  constexpr int n3 = n * n * n;
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+  for (int k = 0; k < 12; ++k) acc[k] = 0.0;
+  for (int d = 0; d < 3; ++d) {
+    const int id = dir_index<n>(v, d), sd = dir_stride<n>(d);
+    for (int al = 0; al < n; ++al) {
+      const int va = v + (al - id) * sd;
+      double U[5];
+      load_state64<n>(a, e, va, U);
+      const Prim64 pr = prim64(U, a.gm1);
+      const double q[4] = {pr.u, pr.v, pr.w, pr.p * pr.ri * a.Rinv}, c = a.ops->Dhat[id * n + al];
+      for (int k = 0; k < 4; ++k)
+        for (int x = 0; x < 3; ++x) acc[3 * k + x] += c * (Me[(3 * d + x) * n3 + va] * q[k]);
+    }
+  }
+}
+
+}  // namespace dg

@@ -458,165 +458,9 @@ __global__ void __launch_bounds__(256) k_surf_prims(StageArgs a) {
 // ---------------------------------------------------------------------------
 // Lifted gradients (weak form, Eq. lifting)
 // ---------------------------------------------------------------------------
-// FP64 shared-memory layout of k_lift (line tasks): the tables (Dhat, then
-// for even n its even and odd half matrices), then per element the q planes
-// (4), the metric planes (9) and the sums (12), each a padded node plane of
-// n^3 + n^2 doubles (one pad after every line of n nodes: the tasks' 64-bit
-// loads along any direction then fall in distinct banks)
-template <int N, int EPB_ = 0>
-struct Lift64Smem {
-  using S = Shape<N, EPB_>;
-  static constexpr int h = S::n / 2, Pn = S::n3 + S::n2;
-  static constexpr int ntab = (S::n2 + 2 * h * h + 1) & ~1;
-  static constexpr size_t bytes = sizeof(double) * (ntab + (size_t)S::EPB * 25 * Pn);
-};
-
-// The FP64 lifting (Eq. lifting, volume part, then the surface part and
-// 1/J) by line tasks: per direction d, one task per (line, variable) loads
-// the line's q and Ja^d once, forms the three products and applies Dhat;
-// for even n through its even and odd half matrices (Dhat is
-// centro-antisymmetric on LGL nodes: with e_j = P_j + P_(n-1-j) and
-// o_j = P_j - P_(n-1-j), y_i = (De e)_i / 2 + (Do o)_i / 2 and
-// y_(n-1-i) = (Do o)_i / 2 - (De e)_i / 2, with De_ij = Dhat_ij +
-// Dhat_i(n-1-j) and Do_ij = Dhat_ij - Dhat_i(n-1-j)): 6 n + 3 n / 2 FP64
-// operations per line and product column instead of n^2, where the lifting
-// is bound by the FP64 unit.  The sums collect in shared memory (written for
-// the first direction, added for the others).
-template <int N, int EPB_>
-__device__ __forceinline__ void lift_lines64(const StageArgs& a) {
-  using S = Shape<N, EPB_>;
-  using L = Lift64Smem<N, EPB_>;
-  constexpr int n = S::n, n2 = S::n2, n3 = S::n3, EPB = S::EPB, Pn = L::Pn, h = L::h;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double* sD = reinterpret_cast<double*>(smraw);  // [n][n] Dhat
-  double* sDe = sD + n2;                          // [h][h] even half
-  double* sDo = sDe + h * h;                      // [h][h] odd half, each halved
-  const int le = threadIdx.x / n3, t = threadIdx.x % n3;
-  double* q = sD + L::ntab + (size_t)le * 25 * Pn;  // [4][Pn] u, v, w, T'
-  double* J = q + 4 * Pn;                           // [9][Pn] Ja^d_c
-  double* W = J + 9 * Pn;                           // [12][Pn] the sums
-  const int ei = blockIdx.x * EPB + le < a.E ? blockIdx.x * EPB + le : a.E - 1;
-  const int e = a.elem_list ? a.elem_list[ei] : ei;
-  const int ce = a.elem_case ? a.elem_case[e] : 0;
-  const bool valid = blockIdx.x * EPB + le < a.E && ce >= 0;
-  const bool busy = valid && !(a.cases && a.cases[ce].dt == 0.0);
-  if (a.elem_case && __syncthreads_and(!busy)) return;
-  const CaseParams cp = case_params(a, ce);
-  for (int k = threadIdx.x; k < n2; k += blockDim.x) sD[k] = a.ops->Dhat[k];
-  for (int k = threadIdx.x; k < h * h; k += blockDim.x) {
-    const int i = k / h, j = k % h;
-    const double* D = a.ops->Dhat + i * n;
-    sDe[k] = 0.5 * (D[j] + D[n - 1 - j]);
-    sDo[k] = 0.5 * (D[j] - D[n - 1 - j]);
-  }
-  const int vp = t + t / n;  // padded index of node t
-  {
-    double U[5];
-    const double* u = a.U + (size_t)e * 5 * n3 + t;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) U[k] = u[k * n3];
-    const SPrim<double> pr = shifted_prim<double>(U, a.gm1, a.Rinv, cp);
-    q[vp] = pr.u, q[Pn + vp] = pr.v, q[2 * Pn + vp] = pr.w, q[3 * Pn + vp] = pr.Tt;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) J[c * Pn + vp] = metric_at<double>(a, e, c, t, n3);
-  }
-  const double Ji = metric_at<double>(a, e, 9, t, n3);
-  __syncwarp();
-  __syncthreads();
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    const int sd = d == 0 ? 1 : (d == 1 ? n : n2);
-    for (int task = t; task < 4 * n2; task += n3) {
-      const int qv = task / n2, l = task % n2, lp = l % n, lq = l / n;
-      const int bl = d == 0 ? n * (lp + n * lq) : (d == 1 ? lp + n2 * lq : lp + n * lq);
-      double P0[n], P1[n], P2[n];
-#pragma unroll
-      for (int al = 0; al < n; ++al) {
-        const int v = bl + al * sd, pv = v + v / n;
-        const double qq = q[qv * Pn + pv];
-        P0[al] = J[(3 * d) * Pn + pv] * qq;
-        P1[al] = J[(3 * d + 1) * Pn + pv] * qq;
-        P2[al] = J[(3 * d + 2) * Pn + pv] * qq;
-      }
-      auto put = [&](int i, double y0, double y1, double y2) {
-        const int v = bl + i * sd;
-        double* w = W + (qv * 3) * Pn + v + v / n;
-        if (d == 0) {
-          w[0] = y0, w[Pn] = y1, w[2 * Pn] = y2;
-        } else {
-          w[0] += y0, w[Pn] += y1, w[2 * Pn] += y2;
-        }
-      };
-      if constexpr (n % 2 == 0) {
-        double E0[h], E1[h], E2[h], O0[h], O1[h], O2[h];
-#pragma unroll
-        for (int j = 0; j < h; ++j) {
-          E0[j] = P0[j] + P0[n - 1 - j], O0[j] = P0[j] - P0[n - 1 - j];
-          E1[j] = P1[j] + P1[n - 1 - j], O1[j] = P1[j] - P1[n - 1 - j];
-          E2[j] = P2[j] + P2[n - 1 - j], O2[j] = P2[j] - P2[n - 1 - j];
-        }
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-          double e0 = 0.0, e1 = 0.0, e2 = 0.0, p0 = 0.0, p1 = 0.0, p2 = 0.0;
-#pragma unroll
-          for (int j = 0; j < h; ++j) {
-            const double ce = sDe[i * h + j], co = sDo[i * h + j];
-            e0 += ce * E0[j], e1 += ce * E1[j], e2 += ce * E2[j];
-            p0 += co * O0[j], p1 += co * O1[j], p2 += co * O2[j];
-          }
-          put(i, p0 + e0, p1 + e1, p2 + e2);
-          put(n - 1 - i, p0 - e0, p1 - e1, p2 - e2);
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-          double y0 = 0.0, y1 = 0.0, y2 = 0.0;
-#pragma unroll
-          for (int al = 0; al < n; ++al) {
-            const double c = sD[i * n + al];
-            y0 += c * P0[al], y1 += c * P1[al], y2 += c * P2[al];
-          }
-          put(i, y0, y1, y2);
-        }
-      }
-    }
-    __syncwarp();
-    __syncthreads();
-  }
-  if (!valid) return;
-  double acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = W[k * Pn + vp];
-  // surface part: on LGL nodes only face nodes receive it
-  const int idx[3] = {t % n, (t / n) % n, t / n2};
-  const double* Lf = a.lflux;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int id = idx[d];
-    if (id != 0 && id != n - 1) continue;
-    const int f = 2 * d + (id == n - 1 ? 1 : 0);
-    const int es = a.elem_side[(size_t)e * 6 + f];
-    const int s = es_side(es);
-    const int p = d == 0 ? idx[1] : idx[0];
-    const int qq = d == 2 ? idx[1] : idx[2];
-    int pm = p, qm = qq;
-    if (es_slave(es)) flip_to_master<n>(es_flip(es), p, qq, pm, qm);
-    const double sg = es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id];
-    const double* Lr = Lf + (size_t)s * 12 * n2 + pm + n * qm;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] += sg * Lr[k * n2];
-  }
-  double* g = a.g + (size_t)e * 12 * n3 + t;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) g[k * n3] = acc[k] * Ji;
-}
-
+// (FP32-bulk; the FP64 lifting is k_lift_fx in dg_fixed64.cuh)
 template <int N, typename T, int EPB_ = 0>
 __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
-  if constexpr (sizeof(T) == sizeof(double)) {
-    lift_lines64<N, EPB_>(a);
-    return;
-  }
   using S = Shape<N, EPB_>;
   constexpr int n = S::n, n2 = S::n2, n3 = S::n3, EPB = S::EPB;
   constexpr int n2p = (n2 + 3) & ~3;  // keeps the arrays below 16-byte aligned
@@ -847,43 +691,42 @@ __global__ void __launch_bounds__(256) k_surf_flux(StageArgs a) {
 // evaluating pow, log and exp itself took 1,617 us per volume kernel launch
 // on the 64 x 8 x 8 N = 5 shock tube and 338 us per element kernel launch on
 // 8^3 N = 7 in FP32-bulk; this form 1,010 and 65 us.
-// All threads call it (it holds barriers); the scratch (sT1 / sT2: n3 doubles
-// each, sRow: 4 n2 doubles) may be reused after the caller's next barrier.
+// The element's TPE threads call it (it holds barriers) with rho p of their
+// nodes t, t + TPE, ... in sT1; the scratch (sT1 / sT2: n3 doubles each, sRow:
+// 4 n2 doubles) may be reused after the caller's next barrier.
 // ---------------------------------------------------------------------------
-template <int n>
-__device__ double element_alpha(double rp, double* sT1, double* sT2, double* sRow, const double* sVinv,
-                                const Ops* ops, int t, double amin, double amax) {
-  constexpr int n2 = n * n, N = n - 1;
-  const int i = t % n, j = (t / n) % n, k = t / n2;
-  sT1[t] = rp;
+template <int n, int TPE = n * n * n>
+__device__ double element_alpha(double* sT1, double* sT2, double* sRow, const double* sVinv, const Ops* ops, int t,
+                                double amin, double amax) {
+  constexpr int n2 = n * n, n3 = n2 * n, N = n - 1;
   __syncwarp();
   __syncthreads();
-  double s = 0.0;
-  for (int x = 0; x < n; ++x) s += sVinv[i * n + x] * sT1[x + n * (j + n * k)];
-  sT2[t] = s;
-  __syncwarp();
-  __syncthreads();
-  s = 0.0;
-  for (int x = 0; x < n; ++x) s += sVinv[j * n + x] * sT2[i + n * (x + n * k)];
-  sT1[t] = s;
-  __syncwarp();
-  __syncthreads();
-  s = 0.0;
-  for (int x = 0; x < n; ++x) s += sVinv[k * n + x] * sT1[i + n * (j + n * x)];
-  sT2[t] = s * s;  // energy of mode (i, j, k)
-  __syncwarp();
-  __syncthreads();
-  if (t < n2) {
-    // row (j, k) = (t % n, t / n): the energies of maximum degree N, N - 1
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double* in = d == 1 ? sT2 : sT1;
+    double* out = d == 1 ? sT1 : sT2;
+    const int sd = d == 0 ? 1 : (d == 1 ? n : n2);
+    for (int v = t; v < n3; v += TPE) {
+      const int id = (v / sd) % n, base = v - id * sd;
+      double s = 0.0;
+#pragma unroll
+      for (int x = 0; x < n; ++x) s += sVinv[id * n + x] * in[base + x * sd];
+      out[v] = d == 2 ? s * s : s;  // at the end the energy of mode v = (i, j, k)
+    }
+    __syncwarp();
+    __syncthreads();
+  }
+  for (int r = t; r < n2; r += TPE) {
+    // row (j, k) = (r % n, r / n): the energies of maximum degree N, N - 1
     // and below, from its last two modes and the sum of the others
-    const double* m2 = sT2 + n * t;
+    const double* m2 = sT2 + n * r;
     double low = 0.0;
     for (int x = 0; x < N - 1; ++x) low += m2[x];
-    const int mx = max(t % n, t / n);
+    const int mx = max(r % n, r / n);
     const double below = low + m2[N - 1];
-    sRow[t] = mx == N ? below + m2[N] : m2[N];
-    sRow[n2 + t] = mx == N ? 0.0 : (mx == N - 1 ? below : m2[N - 1]);
-    sRow[2 * n2 + t] = mx < N - 1 ? low : 0.0;
+    sRow[r] = mx == N ? below + m2[N] : m2[N];
+    sRow[n2 + r] = mx == N ? 0.0 : (mx == N - 1 ? below : m2[N - 1]);
+    sRow[2 * n2 + r] = mx < N - 1 ? low : 0.0;
   }
   __syncwarp();
   __syncthreads();
@@ -914,13 +757,12 @@ __device__ double element_alpha(double rp, double* sT1, double* sT2, double* sRo
 }
 
 // shared-memory layout of k_volume: FP64 part first, then the T arrays
-template <int N, typename T, int EPB_ = 0, bool PAIRS = sizeof(T) == sizeof(double)>
+template <int N, typename T, int EPB_ = 0>
 struct VolumeSmem {
   using S = Shape<N, EPB_>;
   // FP32: node-major primitives (float4 + float2) and metrics (one float4 per
   // direction), so a partner is read with three loads
   static constexpr bool aos = sizeof(T) == sizeof(float);
-  static_assert(!(aos && PAIRS), "the line-pair two-point sums are an FP64 mapping");
   static constexpr int n2p = (S::n2 + 3) & ~3;
   static constexpr int nJ = aos ? 12 : 9;
   // Vinv, indicator scratch, FP32: the node's state and RK register copied in
@@ -933,25 +775,23 @@ struct VolumeSmem {
   // viscous / FV fluxes: FP32 keeps the four viscous components of a node in
   // one float4 (element stride padded like the primitives)
   static constexpr int gstride = aos ? 5 * ((S::n3 + 3) & ~3) : 5 * S::n3;
-  // per-direction two-point sums: only the line-pair tasks need them (the
-  // per-node sums stay in registers)
-  static constexpr int nA = PAIRS ? 15 : 0;
-  static constexpr size_t n_t = 2 * n2p + S::EPB * (pstride + nJ * S::n3 + gstride + nA * S::n3);
+  static constexpr size_t n_t = 2 * n2p + S::EPB * (pstride + nJ * S::n3 + gstride);
   static constexpr size_t bytes = sizeof(double) * n_dbl + sizeof(T) * n_t;
 };
 
 // ---------------------------------------------------------------------------
 // Volume integral + SurfInt + ApplyJac (+ RK update)
 // ---------------------------------------------------------------------------
-// PAIRS: each unordered pair of a line forms its two-point flux once (one
-// task per line, FP64); otherwise each node sums over all its partners.
-template <int N, int MODE, typename T, int EPB_ = 0, bool PAIRS = sizeof(T) == sizeof(double)>
+// One node per thread, which sums over all its partners: FP32-bulk, and FP64's
+// other mapping (dg_set_config; the default FP64 kernel is k_volume_fx in
+// dg_fixed64.cuh).
+template <int N, int MODE, typename T, int EPB_ = 0>
 __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::template vol_min_blocks<T>())
     k_volume(StageArgs a) {
   using S = Shape<N, EPB_>;
   constexpr int n = S::n, n2 = S::n2, n3 = S::n3, EPB = S::EPB;
   extern __shared__ __align__(16) unsigned char smraw[];
-  using L = VolumeSmem<N, T, EPB_, PAIRS>;
+  using L = VolumeSmem<N, T, EPB_>;
   constexpr bool aos = L::aos;
   double* sVi = reinterpret_cast<double*>(smraw);  // [n2] Vinv (FP64)
   double* sX = sVi + n2;                           // [EPB][2 n3 + 4 n2] indicator scratch (FP64)
@@ -960,7 +800,6 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   T* sP = sDh + L::n2p;                  // [EPB][6][n3] rho u v w p' H', halved (FP32: [n3] float4 + [n3] float2)
   T* sJ = sP + EPB * L::pstride;         // [EPB][9][n3] metrics, halved (FP32: [3][n3] float4)
   T* sG = sJ + EPB * L::nJ * n3;         // [EPB][5][n3] viscous / FV fluxes (FP32 viscous: [n3] float4)
-  T* sA = sG + EPB * L::gstride;         // [EPB][3][5][n3] two-point sums (FP64 only)
   const int le = threadIdx.x / n3, t = threadIdx.x % n3;
   double* sUd = sX + EPB * (2 * n3 + 4 * n2) + le * L::nUd;  // FP32: [2][5][n3] U and dU of the element
   // slots past the last element redo the last element, free slots of a
@@ -992,7 +831,6 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     if constexpr (aos) return reinterpret_cast<const float*>(J4 + d * n3 + node)[c];
     else return Jm[(d * 3 + c) * n3 + node];
   };
-  T* A = sA + le * L::nA * n3;
   const double H_ref = cp.Hr;
   double U[5];
   double p_full;
@@ -1056,15 +894,8 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     visc_coeffs<T>(a, cp, me.Tt, vmu, vlam);
     viscous_parts(g, me.u, me.v, me.w, vmu, vlam, tau, W);
   }
-  // ---- split-form KEP volume integral ----
-  // FP64 (bound by the FP64 pipe): one line per task; every unordered pair
-  // (i, alpha) of the line forms the symmetric two-point flux once and adds
-  // Dsplit_{i alpha} f to node i and Dsplit_{alpha i} f to node alpha, which
-  // halves the flux evaluations.  FP32 (bound by latency, not arithmetic):
-  // one node per thread over all its partners, which keeps every thread busy.
-  // Each direction has its own sum array.
-  constexpr bool kPairs = PAIRS;
-  if constexpr (!kPairs) {
+  // ---- split-form KEP volume integral, one node per thread over its partners ----
+  {
     const int idl[3] = {t % n, (t / n) % n, t / n2};
     // halved primitives and direction-d metrics of a node, either layout
     auto node = [&](int d, int v, T& r, T& u0, T& u1, T& u2, T& pp, T& H, T& j0, T& j1, T& j2) {
@@ -1103,7 +934,6 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
         s3 += dv * (fr * u2 + pp * m2);
         s4 += dv * (fr * H);
       }
-      // same association as the line-pair path's (A_0 + A_1) + A_2
       if (d == 0) {
         accC[0] = s0, accC[1] = s1, accC[2] = s2, accC[3] = s3, accC[4] = s4;
       } else {
@@ -1111,60 +941,6 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
       }
     }
   }
-  if constexpr (kPairs)
-  for (int lt = t; lt < 3 * n2; lt += n3) {
-    const int d = lt / n2, line = lt % n2;
-    const int lp = line % n, lq = line / n;
-    const int base = d == 0 ? n * (lp + n * lq) : (d == 1 ? lp + n2 * lq : lp + n * lq);
-    const int st = d == 0 ? 1 : (d == 1 ? n : n2);
-    const T* J0 = Jm + (d * 3 + 0) * n3;
-    const T* J1 = Jm + (d * 3 + 1) * n3;
-    const T* J2 = Jm + (d * 3 + 2) * n3;
-    // this task is the only writer of the line's nodes in direction d's array:
-    // node i keeps its sums in registers, partner contributions go straight
-    // to shared memory
-    T* Ad = A + d * 5 * n3;
-#pragma unroll
-    for (int i = 0; i < n; ++i)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) Ad[k * n3 + base + i * st] = T(0);
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const int vi = base + i * st;
-      const T ri = P[vi], ui = P[n3 + vi], vvi = P[2 * n3 + vi], wi = P[3 * n3 + vi];
-      const T pi = P[4 * n3 + vi], Hi = P[5 * n3 + vi];
-      const T j0 = J0[vi], j1 = J1[vi], j2 = J2[vi];
-      T ai0 = T(0), ai1 = T(0), ai2 = T(0), ai3 = T(0), ai4 = T(0);
-#pragma unroll
-      for (int al = i + 1; al < n; ++al) {
-        const int va = base + al * st;
-        const T m0 = j0 + J0[va], m1 = j1 + J1[va], m2 = j2 + J2[va];
-        const T rho = ri + P[va];
-        const T u0 = ui + P[n3 + va], u1 = vvi + P[2 * n3 + va], u2 = wi + P[3 * n3 + va];
-        const T pp = pi + P[4 * n3 + va];
-        const T H = Hi + P[5 * n3 + va];
-        const T fr = rho * (u0 * m0 + u1 * m1 + u2 * m2);
-        const T f1 = fr * u0 + pp * m0, f2 = fr * u1 + pp * m1, f3 = fr * u2 + pp * m2, f4 = fr * H;
-        const T dia = sDs[i * n + al], dai = sDs[al * n + i];
-        ai0 += dia * fr;
-        ai1 += dia * f1;
-        ai2 += dia * f2;
-        ai3 += dia * f3;
-        ai4 += dia * f4;
-        Ad[va] += dai * fr;
-        Ad[n3 + va] += dai * f1;
-        Ad[2 * n3 + va] += dai * f2;
-        Ad[3 * n3 + va] += dai * f3;
-        Ad[4 * n3 + va] += dai * f4;
-      }
-      Ad[vi] += ai0;
-      Ad[n3 + vi] += ai1;
-      Ad[2 * n3 + vi] += ai2;
-      Ad[3 * n3 + vi] += ai3;
-      Ad[4 * n3 + vi] += ai4;
-    }
-  }
-
   // ---- viscous volume term: collocated weak form, per direction ----
   if (a.viscous) {
 #pragma unroll 1
@@ -1206,10 +982,6 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   }
   __syncwarp();
   __syncthreads();
-  if constexpr (kPairs) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) accC[k] = (A[k * n3 + t] + A[(5 + k) * n3 + t]) + A[(10 + k) * n3 + t];
-  }
 
   // ---- shock capturing: indicator and FV sub-cell blending (Sec. 2.3) ----
   if (a.shock) {
@@ -1219,7 +991,8 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     } else {
       double* X1 = sX + le * (2 * n3 + 4 * n2);
       // all threads of the block take part in the barriers inside
-      al = element_alpha<n>(U[0] * p_full, X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
+      X1[t] = U[0] * p_full;
+      al = element_alpha<n>(X1, X1 + n3, X1 + 2 * n3, sVi, a.ops, t, a.alpha_min, a.alpha_max);
     }
     if (valid && t == 0) a.alpha[e] = al;
     // block-uniform condition: the FV pass has barriers, and the elements of
@@ -1341,6 +1114,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
 
 #include "dg_stage_gl.cuh"
 #include "dg_fused32.cuh"
+#include "dg_fixed64.cuh"
 
 namespace dg {
 
@@ -1428,13 +1202,12 @@ inline StageArgs make_stage_args(dg_ctx* c, const double* U) {
 template <int N, typename T, int E = 0>
 inline size_t lift_smem_bytes() {
   using S = Shape<N, E>;
-  if constexpr (sizeof(T) == sizeof(double)) return Lift64Smem<N, E>::bytes;
   return sizeof(T) * (((S::n2 + 3) & ~3) + S::EPB * 16 * S::n3);
 }
 
 // Launch variants the autotuner chooses among: the default elements per
-// block D and 2D (lifting up to 1024 threads, volume up to 512), and for FP64
-// the volume kernel's two thread mappings.
+// block D and 2D (lifting up to 1024 nodes, volume up to 512), and for FP64
+// the volume kernel's two forms (fixed point, or FP64 sums per node).
 template <int N, typename T>
 struct Variants {
   static constexpr int D = Shape<N>::EPB_DEFAULT;
@@ -1444,16 +1217,48 @@ struct Variants {
   static constexpr bool fp64 = sizeof(T) == sizeof(double);
 };
 
+// SMs of the current device
+inline int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        sms <= 0)
+      sms = 152;
+  }
+  return sms;
+}
+// Elements per block of the fixed-point kernels: E, fewer while the grid
+// would leave SMs without two blocks (the elements of a block share one
+// SM's units; 4^3 elements at N = 3 in blocks of four used 16 of 152 SMs).
+// At N = 1 four elements share a warp.
+template <int N>
+inline int fx_epb(int E, int64_t elems) {
+  const int least = Fix<N>::TPE < 32 ? 32 / Fix<N>::TPE : 1;
+  while (E > least && (elems + E - 1) / E < 2 * sm_count()) E = std::max(least, E / 2 / least * least);
+  return E;
+}
 template <int N, typename T, int E>
 inline void launch_lift(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
-  k_lift<N, T, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, lift_smem_bytes<N, T, E>(), st>>>(a);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    const int epb = fx_epb<N>(S::EPB, a.E);
+    k_lift_fx<N><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, LiftFix<N>::bytes(epb), st>>>(a);
+  } else {
+    k_lift<N, T, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, lift_smem_bytes<N, T, E>(), st>>>(a);
+  }
 }
-template <int N, int MODE, typename T, int E, bool PR>
+// FX: the fixed-point form (FP64)
+template <int N, int MODE, typename T, int E, bool FX>
 inline void launch_vol(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
-  k_volume<N, MODE, T, E, PR>
-      <<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, VolumeSmem<N, T, E, PR>::bytes, st>>>(a);
+  if constexpr (FX) {
+    const int epb = fx_epb<N>(S::EPB, a.E);
+    k_volume_fx<N, MODE><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(a);
+  } else {
+    k_volume<N, MODE, T, E>
+        <<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
+  }
 }
 template <int N, typename T, bool GL = false>
 inline void launch_side(const StageArgs& a, int block, cudaStream_t st, bool prims) {
@@ -1507,19 +1312,22 @@ cudaError_t stage_set_attrs() {
   auto lift = [&](auto kern, size_t bytes) {
     if (bytes <= (size_t)maxsm) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  lift(k_lift<N, T, 0>, lift_smem_bytes<N, T, 0>());
-  if constexpr (V::lift2) lift(k_lift<N, T, 2 * V::D>, lift_smem_bytes<N, T, 2 * V::D>());
+  if constexpr (V::fp64) {
+    lift(k_lift_fx<N>, LiftFix<N>::bytes(V::lift2 ? 2 * V::D : V::D));
+    const size_t vb = VolFix<N>::bytes(V::vol2 ? 2 * V::D : V::D);
+    lift(k_volume_fx<N, 0>, vb);
+    lift(k_volume_fx<N, 1>, vb);
+  } else {
+    lift(k_lift<N, T, 0>, lift_smem_bytes<N, T, 0>());
+    if constexpr (V::lift2) lift(k_lift<N, T, 2 * V::D>, lift_smem_bytes<N, T, 2 * V::D>());
+    lift(k_volume<N, 0, T, 0>, VolumeSmem<N, T, 0>::bytes);
+  }
   lift(k_prolong_gl<N>, gl_prolong_smem<N>());
   lift(k_lift_gl<N, T>, gl_lift_smem<N, T>());
   lift(k_volume_gl<N, 0, T>, gl_volume_smem<N, T>());
   lift(k_volume_gl<N, 1, T>, gl_volume_smem<N, T>());
-  lift(k_volume<N, 0, T, 0, V::fp64>, VolumeSmem<N, T, 0, V::fp64>::bytes);
-  lift(k_volume<N, 1, T, 0, V::fp64>, VolumeSmem<N, T, 0, V::fp64>::bytes);
-  if constexpr (V::fp64) lift(k_volume<N, 1, T, 0, false>, VolumeSmem<N, T, 0, false>::bytes);
-  if constexpr (V::vol2) {
-    lift(k_volume<N, 1, T, 2 * V::D, V::fp64>, VolumeSmem<N, T, 2 * V::D, V::fp64>::bytes);
-    if constexpr (V::fp64) lift(k_volume<N, 1, T, 2 * V::D, false>, VolumeSmem<N, T, 2 * V::D, false>::bytes);
-  }
+  lift(k_volume<N, 1, T, 0>, VolumeSmem<N, T, 0>::bytes);
+  if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D>, VolumeSmem<N, T, 2 * V::D>::bytes);
   if constexpr (!V::fp64) {
     lift(k_fprep<N>, FusedSmem<N>::bytes);
     lift(k_felem<N, 0, 0>, FusedSmem<N, 0>::bytes);

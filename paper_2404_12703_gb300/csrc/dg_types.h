@@ -22,6 +22,16 @@ struct Ops {
   double Dlo[NPMAX * NPMAX];     // D - (double)D (double-double tail)
   double Vinv[NPMAX * NPMAX];    // nodal -> orthonormal Legendre modes
   double ind_T, ind_s;           // shock indicator: threshold T(N), sharpness s
+  // fixed point (dg_fixed64.cuh): S_ij = w_i Dsplit_ij (antisymmetric) and
+  // Dhat times 2^bits, rounded, with every row's absolute sum at most 2^62
+  // (fxS_row: the largest of S's over 2^62, rounded up), 1 / w times 2^bits
+  // (at most 2^62); and for even n the even and odd
+  // halves of Dhat (centro-antisymmetric): with e_j = P_j + P_(n-1-j) and
+  // o_j = P_j - P_(n-1-j), y_i = He e + Ho o and y_(n-1-i) = Ho o - He e with
+  // He_ij = (Dhat_ij + Dhat_i(n-1-j)) / 2, Ho_ij = (Dhat_ij - Dhat_i(n-1-j)) / 2
+  long long fxS[NPMAX * NPMAX], fxH[NPMAX * NPMAX], fxW[NPMAX], fxHe[NPMAX * NPMAX / 4], fxHo[NPMAX * NPMAX / 4];
+  int fxS_bits, fxH_bits, fxW_bits;
+  float fxS_row;
   double Lp[NPMAX], Lm[NPMAX];   // l_i(+1), l_i(-1) (unit vectors on LGL)
   // geometry: the LGL derivative matrix (double-double) and the
   // interpolation from the LGL nodes to the solution nodes (double-double;
