@@ -1228,6 +1228,16 @@ inline int sm_count() {
   }
   return sms;
 }
+// Threads per block of the side kernels: the configured 128 or 256, halved
+// while the grid would leave SMs without two blocks.  A block's side nodes
+// share one SM's units: at 4^3 elements, N = 3, 256-thread blocks put the
+// 3,072 side nodes on 12 of 152 SMs (FP64 flux kernel 26.3 us, 32-thread
+// blocks 16.4 us).
+inline int side_threads(int block, int64_t nodes) {
+  int b = block == 128 ? 128 : 256;
+  while (b > 32 && (nodes + b - 1) / b < 2 * sm_count()) b /= 2;
+  return b;
+}
 // Elements per block of the fixed-point kernels: E, fewer while the grid
 // would leave SMs without two blocks (the elements of a block share one
 // SM's units; 4^3 elements at N = 3 in blocks of four used 16 of 152 SMs).
@@ -1263,7 +1273,7 @@ inline void launch_vol(const StageArgs& a, cudaStream_t st) {
 template <int N, typename T, bool GL = false>
 inline void launch_side(const StageArgs& a, int block, cudaStream_t st, bool prims) {
   const int64_t side_nodes = (int64_t)a.S * Shape<N>::n2;
-  const int b = block == 128 ? 128 : 256;
+  const int b = side_threads(block, side_nodes);
   const unsigned g = (unsigned)((side_nodes + b - 1) / b);
   if (prims) k_surf_prims<N, T, GL><<<g, b, 0, st>>>(a);
   else k_surf_flux<N, T, GL><<<g, b, 0, st>>>(a);
@@ -1435,7 +1445,7 @@ inline void launch_felem(StageArgs a, int prefetch, cudaStream_t st) {
 template <int N>
 inline void launch_fflux(const StageArgs& a, int block, cudaStream_t st) {
   const int64_t side_nodes = (int64_t)a.S * Shape<N>::n2;
-  const int b = block == 128 ? 128 : 256;
+  const int b = side_threads(block, side_nodes);
   k_fflux<N><<<(unsigned)((side_nodes + b - 1) / b), b, 0, st>>>(a);
 }
 // face data of state U: every element of the context (a serving pool: its
