@@ -226,6 +226,16 @@ static void build_ops(int N, int gauss, Ops& o) {
   o.fxH_bits = fixed(Mh, n * n, row_sum(Mh), o.fxH);
   o.fxW_bits = fixed(wi, n, *std::max_element(wi, wi + n), o.fxW);
   o.fxS_row = (float)std::ldexp(row_sum(Ms), o.fxS_bits - 62) * 1.00001f;
+  ld le[2 * NPMAX], ll[2 * NPMAX], se = 0, ml = 0;
+  for (int i = 0; i < n; ++i) {
+    le[i] = gauss ? lagrange(n, x, i, -1) : (i == 0 ? 1 : 0);
+    le[n + i] = gauss ? lagrange(n, x, i, 1) : (i == N ? 1 : 0);
+    se += std::fabs(le[i]);  // (the other end's are the same in reverse)
+    ll[i] = le[i] / w[i], ll[n + i] = le[n + i] / w[i];
+    ml = std::max(ml, std::max(std::fabs(ll[i]), std::fabs(ll[n + i])));
+  }
+  o.fxE_bits = fixed(le, 2 * n, se * (1 + 1e-15L), o.fxE);
+  o.fxL_bits = fixed(ll, 2 * n, 4 * ml, o.fxL);
   const int h = n / 2;
   for (int i = 0; i < h && n % 2 == 0; ++i)
     for (int j = 0; j < h; ++j) {

@@ -217,6 +217,44 @@ __device__ __forceinline__ ElemRef elem_ref(const StageArgs& a, int slot) {
   return r;
 }
 
+// ApplyJac of a node's sums s, the sources, and Ut or the RK update
+template <int n, int MODE>
+__device__ __forceinline__ void finish_node64(const StageArgs& a, int e, int ce, int v, const double s[5]) {
+  constexpr int n3 = n * n * n;
+  const double Ji = -a.metric[((size_t)e * 10 + 9) * n3 + v];
+  double Ut[5], U[5];
+  load_state64<n>(a, e, v, U);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) Ut[k] = s[k] * Ji;
+  if (a.sponge_sigma) {  // sponge source -sigma (U - U_base)
+    const double sg = a.sponge_sigma[(size_t)e * n3 + v];
+    const double* ub = a.sponge_base + (size_t)e * 5 * n3 + v;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) Ut[k] -= sg * (U[k] - ub[k * n3]);
+  }
+  if (a.source) {  // manufactured-solution source
+    double Q[5];
+    mms_source(a, a.xyzs + ((size_t)e * n3 + v) * 3, stage_time(a, MODE), Q);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) Ut[k] += Q[k];
+  }
+  if (MODE == 0) {
+    double* o = a.Ut + (size_t)e * 5 * n3 + v;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) o[k * n3] = Ut[k];
+  } else {
+    const double dt = case_dt(a, ce);
+    double* du = a.dU + (size_t)e * 5 * n3 + v;
+    double* uo = a.Urk + (size_t)e * 5 * n3 + v;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const double x = a.first_stage ? dt * Ut[k] : a.rkA * du[k * n3] + dt * Ut[k];
+      du[k * n3] = x;
+      uo[k * n3] = U[k] + a.rkB * x;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Lifted gradients (Eq. lifting)
 // ---------------------------------------------------------------------------
@@ -237,27 +275,24 @@ struct LiftFix {
 template <int n>
 __device__ void lift_direct(const StageArgs& a, int e, int v, double acc[12]);
 
+// Dhat split in shared memory: for even n its even and odd halves
 template <int N>
-__global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_lift_fx(StageArgs a) {
-  using F = Fix<N>;
+__device__ __forceinline__ void lift_table_fx(const Ops* o, Fx* sD) {
   using L = LiftFix<N>;
-  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn, h = L::h;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
-  Fx* sD = reinterpret_cast<Fx*>(smraw);
-  unsigned* red = reinterpret_cast<unsigned*>(smraw + 8 * L::ntab) + le * L::nred;
-  long long* q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::planes * Pn;
-  long long* J = q + 4 * Pn;   // [2][3][Pn]
-  long long* W = J + 6 * Pn;   // [12][Pn]
-  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
-  if (a.elem_case && __syncthreads_and(!er.busy)) return;
-  const int e = er.e;
-  const double* Me = a.metric + (size_t)e * 10 * n3;
+  constexpr int h = L::h;
   for (int k = threadIdx.x; k < L::ntab; k += blockDim.x)
-    sD[k] = n % 2 == 0 ? fx_split(k < h * h ? a.ops->fxHe[k] : a.ops->fxHo[k - h * h]) : fx_split(a.ops->fxH[k]);
-  // primitives (FP64, in the q planes until the scales are known) and maxima
-  unsigned m[5] = {0, 0, 0, 0, 0};
-  for (int v = t; v < n3; v += TPE) {
+    sD[k] = Fix<N>::n % 2 == 0 ? fx_split(k < h * h ? o->fxHe[k] : o->fxHo[k - h * h]) : fx_split(o->fxH[k]);
+}
+// (u, v, w, T) of the element's nodes, in FP64, to the q planes, and the
+// maxima of velocity, temperature and the metrics by Cartesian component
+template <int N>
+__device__ __forceinline__ void lift_prims_fx(const StageArgs& a, int e, long long* q, unsigned m[5], int t) {
+  using F = Fix<N>;
+  constexpr int n = F::n, n3 = F::n3, Pn = F::Pn;
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) m[k] = 0;
+  for (int v = t; v < n3; v += F::TPE) {
     double U[5];
     load_state64<n>(a, e, v, U);
     const Prim64 pr = prim64(U, a.gm1);
@@ -269,13 +304,16 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
 #pragma unroll
     for (int c = 0; c < 9; ++c) m[2 + c % 3] = max(m[2 + c % 3], fx_mag(Me[c * n3 + v]));
   }
-  unsigned* fin = red + F::W * L::Q;
-  fx_reduce<N, 5>(m, red, fin, t);
-  __syncthreads();
-  bool bad = false;
-#pragma unroll
-  for (int k = 0; k < 5; ++k) bad = bad || fx_bad(fin[k]);
-  const int eU = fx_exp(fin[0]), eT = fx_exp(fin[1]), eJ[3] = {fx_exp(fin[2]), fx_exp(fin[3]), fx_exp(fin[4])};
+}
+// The volume sums sum_d Dhat (Ja^d q) of the element in the W planes, from the
+// FP64 values in the q planes; a sum of variable k = 3 q + x has the scale
+// 2^(fxH_bits - 2 - e_q - eJ[x]) and is below 2^62
+template <int N>
+__device__ __forceinline__ void lift_sums_fx(const double* Me, long long* q, long long* J, long long* W, const Fx* sD,
+                                             int t, int eU, int eT, const int eJ[3]) {
+  using F = Fix<N>;
+  using L = LiftFix<N>;
+  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn, h = L::h;
   for (int v = t; v < n3; v += TPE) {
     const int pv = fx_pad<n>(v);
 #pragma unroll
@@ -349,6 +387,37 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
     __syncwarp();
     __syncthreads();
   }
+}
+
+template <int N>
+__global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_lift_fx(StageArgs a) {
+  using F = Fix<N>;
+  using L = LiftFix<N>;
+  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
+  Fx* sD = reinterpret_cast<Fx*>(smraw);
+  unsigned* red = reinterpret_cast<unsigned*>(smraw + 8 * L::ntab) + le * L::nred;
+  unsigned* fin = red + F::W * L::Q;
+  long long* q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::planes * Pn;
+  long long* J = q + 4 * Pn;   // [2][3][Pn]
+  long long* W = J + 6 * Pn;   // [12][Pn]
+  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
+  if (a.elem_case && __syncthreads_and(!er.busy)) return;
+  const int e = er.e;
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+  lift_table_fx<N>(a.ops, sD);
+  {
+    unsigned m[5];
+    lift_prims_fx<N>(a, e, q, m, t);
+    fx_reduce<N, 5>(m, red, fin, t);
+    __syncthreads();
+  }
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) bad = bad || fx_bad(fin[k]);
+  const int eU = fx_exp(fin[0]), eT = fx_exp(fin[1]), eJ[3] = {fx_exp(fin[2]), fx_exp(fin[3]), fx_exp(fin[4])};
+  lift_sums_fx<N>(Me, q, J, W, sD, t, eU, eT, eJ);
   if (!er.valid) return;
   const int pU = a.ops->fxH_bits - 2 - eU, pT = a.ops->fxH_bits - 2 - eT;
   const double* Lf = a.lflux;
@@ -938,39 +1007,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
 #pragma unroll
       for (int k = 0; k < 5; ++k) s[k] += sg * Fs[k * n2];
     }
-    // ---- ApplyJac, sources, Ut or the RK update ----
-    const double Ji = -Me[9 * n3 + v];
-    double Ut[5], U[5];
-    load_state64<n>(a, e, v, U);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) Ut[k] = s[k] * Ji;
-    if (a.sponge_sigma) {  // sponge source -sigma (U - U_base)
-      const double sg = a.sponge_sigma[(size_t)e * n3 + v];
-      const double* ub = a.sponge_base + (size_t)e * 5 * n3 + v;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) Ut[k] -= sg * (U[k] - ub[k * n3]);
-    }
-    if (a.source) {  // manufactured-solution source
-      double Q[5];
-      mms_source(a, a.xyzs + ((size_t)e * n3 + v) * 3, stage_time(a, MODE), Q);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) Ut[k] += Q[k];
-    }
-    if (MODE == 0) {
-      double* o = a.Ut + (size_t)e * 5 * n3 + v;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) o[k * n3] = Ut[k];
-    } else {
-      const double dt = case_dt(a, er.ce);
-      double* du = a.dU + (size_t)e * 5 * n3 + v;
-      double* uo = a.Urk + (size_t)e * 5 * n3 + v;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const double x = a.first_stage ? dt * Ut[k] : a.rkA * du[k * n3] + dt * Ut[k];
-        du[k * n3] = x;
-        uo[k * n3] = U[k] + a.rkB * x;
-      }
-    }
+    finish_node64<n, MODE>(a, e, er.ce, v, s);
   }
 }
 

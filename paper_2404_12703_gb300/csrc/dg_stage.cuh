@@ -1115,6 +1115,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
 #include "dg_stage_gl.cuh"
 #include "dg_fused32.cuh"
 #include "dg_fixed64.cuh"
+#include "dg_fixed64_gl.cuh"
 
 namespace dg {
 
@@ -1333,9 +1334,15 @@ cudaError_t stage_set_attrs() {
     lift(k_volume<N, 0, T, 0>, VolumeSmem<N, T, 0>::bytes);
   }
   lift(k_prolong_gl<N>, gl_prolong_smem<N>());
-  lift(k_lift_gl<N, T>, gl_lift_smem<N, T>());
-  lift(k_volume_gl<N, 0, T>, gl_volume_smem<N, T>());
-  lift(k_volume_gl<N, 1, T>, gl_volume_smem<N, T>());
+  if constexpr (V::fp64) {
+    lift(k_lift_gl_fx<N>, LiftGlFix<N>::bytes(V::D));
+    lift(k_volume_gl_fx<N, 0>, VolGlFix<N>::bytes(V::D));
+    lift(k_volume_gl_fx<N, 1>, VolGlFix<N>::bytes(V::D));
+  } else {
+    lift(k_lift_gl<N, T>, gl_lift_smem<N, T>());
+    lift(k_volume_gl<N, 0, T>, gl_volume_smem<N, T>());
+    lift(k_volume_gl<N, 1, T>, gl_volume_smem<N, T>());
+  }
   lift(k_volume<N, 1, T, 0>, VolumeSmem<N, T, 0>::bytes);
   if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D>, VolumeSmem<N, T, 2 * V::D>::bytes);
   if constexpr (!V::fp64) {
@@ -1523,6 +1530,9 @@ cudaError_t stage_launch_gl(dg_ctx* c, const double* U, int mode, double rkA, do
   a.first_stage = first;
   if (a.E == 0) return cudaSuccess;
   const unsigned nb = (unsigned)((a.E + S::EPB - 1) / S::EPB);
+  constexpr bool fx = sizeof(T) == sizeof(double);  // the fixed-point kernels
+  const int epb = fx_epb<N>(S::EPB, a.E);
+  const unsigned nbx = (unsigned)((a.E + epb - 1) / epb);
   const int sb = c->cfg.side_block;
   prof_begin(c, PK_SURF_PRIMS);
   k_prolong_gl<N><<<nb, S::THREADS, gl_prolong_smem<N>(), c->stream>>>(a);
@@ -1530,7 +1540,8 @@ cudaError_t stage_launch_gl(dg_ctx* c, const double* U, int mode, double rkA, do
   prof_end(c);
   if (c->prm.viscous) {
     prof_begin(c, PK_LIFT);
-    k_lift_gl<N, T><<<nb, S::THREADS, gl_lift_smem<N, T>(), c->stream>>>(a);
+    if constexpr (fx) k_lift_gl_fx<N><<<nbx, Fix<N>::TPE * epb, LiftGlFix<N>::bytes(epb), c->stream>>>(a);
+    else k_lift_gl<N, T><<<nb, S::THREADS, gl_lift_smem<N, T>(), c->stream>>>(a);
     prof_end(c);
     count_launch(2);
   }
@@ -1538,8 +1549,13 @@ cudaError_t stage_launch_gl(dg_ctx* c, const double* U, int mode, double rkA, do
   launch_side<N, T, true>(a, sb, c->stream, false);
   prof_end(c);
   prof_begin(c, PK_VOLUME);
-  if (mode == 0) k_volume_gl<N, 0, T><<<nb, S::THREADS, gl_volume_smem<N, T>(), c->stream>>>(a);
-  else k_volume_gl<N, 1, T><<<nb, S::THREADS, gl_volume_smem<N, T>(), c->stream>>>(a);
+  if constexpr (fx) {
+    if (mode == 0) k_volume_gl_fx<N, 0><<<nbx, Fix<N>::TPE * epb, VolGlFix<N>::bytes(epb), c->stream>>>(a);
+    else k_volume_gl_fx<N, 1><<<nbx, Fix<N>::TPE * epb, VolGlFix<N>::bytes(epb), c->stream>>>(a);
+  } else {
+    if (mode == 0) k_volume_gl<N, 0, T><<<nb, S::THREADS, gl_volume_smem<N, T>(), c->stream>>>(a);
+    else k_volume_gl<N, 1, T><<<nb, S::THREADS, gl_volume_smem<N, T>(), c->stream>>>(a);
+  }
   prof_end(c);
   count_launch(3);
   return cudaGetLastError();

@@ -2,7 +2,8 @@
 // Gauss-Legendre nodes (Eq. dgsem with lhat+-_i = l_i(+-1) / w_i; Sec. 5.1
 // runs this scheme's convergence test), templated on the arithmetic type T
 // like the LGL kernels (the side kernels are shared, reading the face states
-// from the arrays written here).
+// from the arrays written here).  FP64 runs k_lift_gl and k_volume_gl's work in
+// fixed point (dg_fixed64_gl.cuh); these two are FP32-bulk's.
 //
 // Per stage:
 //   k_prolong_gl   ProlongToFace: the state interpolated to the six faces

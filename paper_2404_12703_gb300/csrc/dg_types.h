@@ -32,6 +32,10 @@ struct Ops {
   long long fxS[NPMAX * NPMAX], fxH[NPMAX * NPMAX], fxW[NPMAX], fxHe[NPMAX * NPMAX / 4], fxHo[NPMAX * NPMAX / 4];
   int fxS_bits, fxH_bits, fxW_bits;
   float fxS_row;
+  // l_i(-1) and l_i(+1) (their absolute sums at most 2^62), and the same over
+  // w_i (at most 2^60): [2][n]
+  long long fxE[2 * NPMAX], fxL[2 * NPMAX];
+  int fxE_bits, fxL_bits;
   double Lp[NPMAX], Lm[NPMAX];   // l_i(+1), l_i(-1) (unit vectors on LGL)
   // geometry: the LGL derivative matrix (double-double) and the
   // interpolation from the LGL nodes to the solution nodes (double-double;
