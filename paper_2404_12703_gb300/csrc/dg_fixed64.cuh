@@ -175,18 +175,6 @@ __device__ __forceinline__ int fx_room(float b, int top) {
   return max(0, min(31, top - l));
 }
 
-// ConsToPrim in FP64 (the FP64 path's references are zero)
-struct Prim64 {
-  double rho, u, v, w, p, ri;
-};
-__device__ __forceinline__ Prim64 prim64(const double U[5], double gm1) {
-  Prim64 q;
-  q.rho = U[0];
-  q.ri = 1.0 / U[0];
-  q.u = U[1] * q.ri, q.v = U[2] * q.ri, q.w = U[3] * q.ri;
-  q.p = gm1 * (U[4] - 0.5 * (U[1] * q.u + U[2] * q.v + U[3] * q.w));
-  return q;
-}
 template <int n>
 __device__ __forceinline__ void load_state64(const StageArgs& a, int e, int v, double U[5]) {
   constexpr int n3 = n * n * n;
