@@ -187,10 +187,11 @@ __device__ __forceinline__ double case_dt(const StageArgs& a, int c) {
 //   H' = (d_E + p' - Hr d_rho) / rho,
 //   T' = (p' / R - Tr d_rho) / rho.
 // INTCVT: the FP32 conversions on the integer pipe (f32_rn / f64_of: the
-// same values as the hardware conversions, off the FP64 unit).  That pays
-// in the volume kernel, whose FP64 unit also carries the RK update; in the
-// lifting and surface kernels the extra integer instructions cost more than
-// the conversions they replace.
+// same values as the hardware conversions, off the FP64 unit, which the six
+// conversions of a state kept 80 % busy in the surface prolongation; 16 x 8 x
+// 16 channel, N = 7: k_surf_prims 20.1 -> 17.1 us, k_surf_flux 31.1 -> 29.8
+// us).  Not in the lifting, where the integer instructions cost more than the
+// conversions (71.4 -> 77.9 us).
 template <typename T, bool INTCVT = false>
 __device__ __forceinline__ SPrim<T> shifted_prim(const double U[5], double gm1, double Rinv, const CaseParams& cp,
                                                 double* p_full = nullptr) {
@@ -505,9 +506,8 @@ __global__ void __launch_bounds__(256) k_surf_prims(StageArgs a) {
   constexpr int ust = GL ? n2 : n3;
 #pragma unroll
   for (int k = 0; k < 5; ++k) UM[k] = uM[k * ust];
-  const SPrim<T> qM = shifted_prim<T>(UM, a.gm1, a.Rinv, cp);
+  const SPrim<T> qM = shifted_prim<T, true>(UM, a.gm1, a.Rinv, cp);
   T qa[4];
-  const int brow = a.side_bc ? a.side_bc[s] : -1;
   if (brow >= 0) {
     bc_lift_value<T>(a, cp, brow, UM, qM, nu, qa);  // boundary side: the condition's value
   } else {
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(256) k_surf_prims(StageArgs a) {
     const double* uS = GL ? a.Ufc + (size_t)s * 10 * n2 + 5 * n2 + pq : a.U + (size_t)ee.y * 5 * n3 + vS;
 #pragma unroll
     for (int k = 0; k < 5; ++k) US[k] = uS[k * ust];
-    const SPrim<T> qS = shifted_prim<T>(US, a.gm1, a.Rinv, cp);
+    const SPrim<T> qS = shifted_prim<T, true>(US, a.gm1, a.Rinv, cp);
     qa[0] = T(0.5) * (qM.u + qS.u), qa[1] = T(0.5) * (qM.v + qS.v), qa[2] = T(0.5) * (qM.w + qS.w);
     qa[3] = T(0.5) * (qM.Tt + qS.Tt);
   }
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
     const int qq = d == 2 ? idx[1] : idx[2];
     int pm = p, qm = qq;
     if (es_slave(es)) flip_to_master<n>(es_flip(es), p, qq, pm, qm);
-    const T sg = T(es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id]);
+    const T sg = from_f64<T>(es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id]);
     const T* L = Lf + (size_t)s * 12 * n2 + pm + n * qm;
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] += sg * L[k * n2];
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(256) k_surf_flux(StageArgs a) {
     const double* uS = GL ? a.Ufc + (size_t)s * 10 * n2 + 5 * n2 + pq : a.U + (size_t)ee.y * 5 * n3 + vS;
 #pragma unroll
     for (int k = 0; k < 5; ++k) US[k] = uS[k * ust];
-    const SPrim<T> qS = shifted_prim<T>(US, a.gm1, a.Rinv, cp);
+    const SPrim<T> qS = shifted_prim<T, true>(US, a.gm1, a.Rinv, cp);
     if (cp.riemann == DG_RIEMANN_ROE) roe_flux_s(qM, qS, nu, pick<T>(a.gm1, a.f_gm1), pick<T>(cp.Hr, cp.fHr), f);
     else lf_flux_s(qM, qS, nu, pick<T>(a.gamma, a.f_gamma), pick<T>(cp.pr, cp.fpr), f);
 #pragma unroll
@@ -878,13 +878,18 @@ struct VolumeSmem {
   // asynchronously (even count: the T arrays start 16-byte aligned)
   static constexpr int nUd = aos ? 10 * S::n3 : 0;
   static constexpr size_t n_dbl = (S::n2 + S::EPB * (2 * S::n3 + 4 * S::n2 + nUd) + 1) & ~size_t(1);
+  // a node plane: FP32 pads every line of n nodes by one, so that the four
+  // lines along the first direction that a warp holds at N = 7 fall in
+  // distinct banks (16 x 8 x 16 channel, N = 7: 125 -> 121 us per launch)
+  static constexpr int Pn = aos ? S::n3 + S::n2 : S::n3;
   // per-element stride of the primitives: a multiple of 4 floats in FP32, so
   // that every element's float4 view starts 16-byte aligned
-  static constexpr int pstride = aos ? 6 * ((S::n3 + 3) & ~3) : 6 * S::n3;
+  static constexpr int pstride = aos ? 6 * ((Pn + 3) & ~3) : 6 * Pn;
   // viscous / FV fluxes: FP32 keeps the four viscous components of a node in
   // one float4 (element stride padded like the primitives)
-  static constexpr int gstride = aos ? 5 * ((S::n3 + 3) & ~3) : 5 * S::n3;
-  static constexpr size_t n_t = 2 * n2p + S::EPB * (pstride + nJ * S::n3 + gstride);
+  static constexpr int gfv = 5 * ((S::n3 + 3) & ~3);
+  static constexpr int gstride = aos ? (gfv > 4 * Pn ? gfv : 4 * Pn) : 5 * S::n3;
+  static constexpr size_t n_t = 2 * n2p + S::EPB * (pstride + nJ * Pn + gstride);
   static constexpr size_t bytes = sizeof(double) * n_dbl + sizeof(T) * n_t;
 };
 
@@ -902,13 +907,15 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   extern __shared__ __align__(16) unsigned char smraw[];
   using L = VolumeSmem<N, T, EPB_>;
   constexpr bool aos = L::aos;
+  constexpr int Pn = L::Pn;
+  auto px = [](int node) { return aos ? node + node / n : node; };  // its plane index
   double* sVi = reinterpret_cast<double*>(smraw);  // [n2] Vinv (FP64)
   double* sX = sVi + n2;                           // [EPB][2 n3 + 4 n2] indicator scratch (FP64)
   T* sDs = reinterpret_cast<T*>(reinterpret_cast<double*>(smraw) + L::n_dbl);  // [n2] Dsplit
   T* sDh = sDs + L::n2p;                                                       // [n2] Dhat
   T* sP = sDh + L::n2p;                  // [EPB][6][n3] rho u v w p' H', halved (FP32: [n3] float4 + [n3] float2)
   T* sJ = sP + EPB * L::pstride;         // [EPB][9][n3] metrics, halved (FP32: [3][n3] float4)
-  T* sG = sJ + EPB * L::nJ * n3;         // [EPB][5][n3] viscous / FV fluxes (FP32 viscous: [n3] float4)
+  T* sG = sJ + EPB * L::nJ * Pn;         // [EPB][5][n3] viscous / FV fluxes (FP32 viscous: [n3] float4)
   const int le = threadIdx.x / n3, t = threadIdx.x % n3;
   double* sUd = sX + EPB * (2 * n3 + 4 * n2) + le * L::nUd;  // FP32: [2][5][n3] U and dU of the element
   // slots past the last element redo the last element, free slots of a
@@ -928,16 +935,16 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     sVi[k] = a.ops->Vinv[k];
   }
   T* P = sP + le * L::pstride;
-  T* Jm = sJ + le * L::nJ * n3;
+  T* Jm = sJ + le * L::nJ * Pn;
   T* G = sG + le * L::gstride;
   float4* G4 = reinterpret_cast<float4*>(G);
   // FP32 views of the same memory
   float4* P4 = reinterpret_cast<float4*>(P);
-  float2* P2 = reinterpret_cast<float2*>(P + 4 * n3);
+  float2* P2 = reinterpret_cast<float2*>(P + 4 * Pn);
   float4* J4 = reinterpret_cast<float4*>(Jm);
   // halved metric component c of direction d at a node
   auto Jc = [&](int d, int c, int node) -> T {
-    if constexpr (aos) return reinterpret_cast<const float*>(J4 + d * n3 + node)[c];
+    if constexpr (aos) return reinterpret_cast<const float*>(J4 + d * Pn + px(node))[c];
     else return Jm[(d * 3 + c) * n3 + node];
   };
   const double H_ref = cp.Hr;
@@ -969,11 +976,11 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     // halved values: every arithmetic mean of the two-point flux is then one
     // addition, bit-identical to (a + b) / 2
     if constexpr (aos) {
-      P4[t] = make_float4(0.5f * me.rho, 0.5f * me.u, 0.5f * me.v, 0.5f * me.w);
-      P2[t] = make_float2(0.5f * me.p, 0.5f * me.H);
+      P4[px(t)] = make_float4(0.5f * me.rho, 0.5f * me.u, 0.5f * me.v, 0.5f * me.w);
+      P2[px(t)] = make_float2(0.5f * me.p, 0.5f * me.H);
 #pragma unroll
       for (int d = 0; d < 3; ++d)
-        J4[d * n3 + t] = make_float4(0.5f * metric_at<T>(a, e, 3 * d, t, n3), 0.5f * metric_at<T>(a, e, 3 * d + 1, t, n3),
+        J4[d * Pn + px(t)] = make_float4(0.5f * metric_at<T>(a, e, 3 * d, t, n3), 0.5f * metric_at<T>(a, e, 3 * d + 1, t, n3),
                                      0.5f * metric_at<T>(a, e, 3 * d + 2, t, n3), 0.0f);
     } else {
       P[t] = T(0.5) * me.rho;
@@ -1009,17 +1016,17 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     // halved primitives and direction-d metrics of a node, either layout
     auto node = [&](int d, int v, T& r, T& u0, T& u1, T& u2, T& pp, T& H, T& j0, T& j1, T& j2) {
       if constexpr (aos) {
-        const float4 a4 = P4[v];
-        const float2 a2 = P2[v];
-        const float4 jj = J4[d * n3 + v];
+        const float4 a4 = P4[px(v)];
+        const float2 a2 = P2[px(v)];
+        const float4 jj = J4[d * Pn + px(v)];
         r = a4.x, u0 = a4.y, u1 = a4.z, u2 = a4.w, pp = a2.x, H = a2.y, j0 = jj.x, j1 = jj.y, j2 = jj.z;
       } else {
         r = P[v], u0 = P[n3 + v], u1 = P[2 * n3 + v], u2 = P[3 * n3 + v], pp = P[4 * n3 + v], H = P[5 * n3 + v];
         j0 = Jm[(d * 3) * n3 + v], j1 = Jm[(d * 3 + 1) * n3 + v], j2 = Jm[(d * 3 + 2) * n3 + v];
       }
     };
-#pragma unroll 1
-    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {  // (unrolled: the partners' padded offsets are then constants)
       const int id = idl[d], base = t - id * str[d];
       T ri, ui, vvi, wi, pi, Hi, j0, j1, j2;
       node(d, t, ri, ui, vvi, wi, pi, Hi, j0, j1, j2);
@@ -1059,7 +1066,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
         T fv[4];
         viscous_flux_n(tau, W, nv, fv);
         if constexpr (aos) {
-          G4[t] = make_float4(fv[0], fv[1], fv[2], fv[3]);
+          G4[px(t)] = make_float4(fv[0], fv[1], fv[2], fv[3]);
         } else {
 #pragma unroll
           for (int k = 0; k < 4; ++k) G[k * n3 + t] = fv[k];
@@ -1074,7 +1081,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
           const T c = sDh[id * n + al];
           const int nb = base + al * str[d];
           if constexpr (aos) {
-            const float4 gv = G4[nb];
+            const float4 gv = G4[px(nb)];
             acc[1] -= c * gv.x;
             acc[2] -= c * gv.y;
             acc[3] -= c * gv.z;
@@ -1174,7 +1181,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     const int qq = d == 2 ? idx[1] : idx[2];
     int pm = p, qm = qq;
     if (es_slave(es)) flip_to_master<n>(es_flip(es), p, qq, pm, qm);
-    const T sg = T(es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id]);
+    const T sg = from_f64<T>(es_slave(es) ? -a.ops->winv[id] : a.ops->winv[id]);
     const T* Fs = Fst + (size_t)s * 5 * n2 + pm + n * qm;
 #pragma unroll
     for (int k = 0; k < 5; ++k) acc[k] += sg * Fs[k * n2];
