@@ -780,7 +780,7 @@ int dg_set_params(dg_ctx* c, const dg_params* p) {
   c->prm = *p;
   destroy_graph(c);
   c->traces_valid = false;
-  if (c->state_set) {
+  if (c->state_set || p->precision == DG_FP64) {  // (FP64: back to zero)
     cudaError_t e = launch_refs(c);
     if (e != cudaSuccess) return cuda_fail(e, "dg_set_params");
   }
@@ -871,15 +871,17 @@ int dg_rhs(dg_ctx* c, const double* U_dev, double* Ut_dev) {
     e = launch_to_internal(c, U_dev, c->dU);
     Uin = c->dU;
   }
+  // FP32-bulk (in FP64 the references are zero: three launches less):
   // reference state of the shifted primitives taken from the evaluated state
   // (any constant is exact; this one keeps the FP32-bulk rounding small); the
   // context's own is kept and put back, so later steps are unchanged
-  if (e == cudaSuccess && U_dev && c->state_set) {
+  const bool refs = U_dev && c->prm.precision == DG_FP32_BULK;
+  if (e == cudaSuccess && refs && c->state_set) {
     k_keep_refs<<<1, 1, 0, c->stream>>>(c->scal, 0);
     count_launch();
     e = cudaGetLastError();
   }
-  if (U_dev) {  // the context's own state keeps the reference it was set with
+  if (refs) {  // the context's own state keeps the reference it was set with
     double* Ukeep = c->U;
     c->U = const_cast<double*>(Uin);
     if (e == cudaSuccess) e = launch_refs(c);
@@ -887,7 +889,7 @@ int dg_rhs(dg_ctx* c, const double* U_dev, double* Ut_dev) {
   }
   if (e == cudaSuccess) e = launch_rhs(c, Uin, 0, 0.0, 0.0, 0);
   if (e == cudaSuccess) e = launch_to_public(c, c->Ut, Ut_dev);
-  if (e == cudaSuccess && U_dev && c->state_set) {
+  if (e == cudaSuccess && refs && c->state_set) {
     k_keep_refs<<<1, 1, 0, c->stream>>>(c->scal, 1);
     count_launch();
     e = cudaGetLastError();
