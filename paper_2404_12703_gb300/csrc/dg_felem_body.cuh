@@ -364,7 +364,7 @@ do {
         __syncwarp();
         __syncthreads();  // the workspace is read by no thread any more
         face_epilogue<N>(a, cp, e, t, valid, mn, Jinv, J4, Qs, P4, Wk, sDr, sSn);  // P4, Q4 are free after the KEP sums
-        if (a.cfl_out && threadIdx.x == 0) cfl_block_finish(a, red, (int)(blockDim.x >> 5));
+        if (a.cfl_out && threadIdx.x == 0) cfl_block_finish(a, red, (int)((blockDim.x + 31) >> 5));
       }
     }
 } while (0);

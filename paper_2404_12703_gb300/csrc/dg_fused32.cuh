@@ -395,12 +395,15 @@ __device__ __forceinline__ void cfl_block_radii(const StageArgs& a, bool valid, 
   cfl_radii(Uv, M, a.f_gamma, a.f_gm1, a.f_Rinv, a.f_cflkv, a.sutherland, a.f_inv_Tref, aa, bb);
   const bool bad = valid && !(isfinite(aa) && isfinite(bb));
   if (!valid) aa = bb = 0.0f;
+  // a block's last warp may be a part of one (n^3 nodes per element)
+  const int lane = threadIdx.x & 31, lanes = min(32, (int)blockDim.x - (int)(threadIdx.x & ~31u));
+  const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    aa = fmaxf(aa, __shfl_xor_sync(0xffffffffu, aa, o));
-    bb = fmaxf(bb, __shfl_xor_sync(0xffffffffu, bb, o));
+    const float xa = __shfl_xor_sync(mask, aa, o), xb = __shfl_xor_sync(mask, bb, o);
+    if ((lane ^ o) < lanes) aa = fmaxf(aa, xa), bb = fmaxf(bb, xb);
   }
-  const bool wbad = __any_sync(0xffffffffu, bad);
+  const bool wbad = __any_sync(mask, bad);
   if ((threadIdx.x & 31) == 0) {
     const int w = threadIdx.x >> 5;
     red[2 * w] = aa;
@@ -473,7 +476,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS) k_fprep(StageArgs a) {
   __syncwarp();
   __syncthreads();
   face_epilogue<N>(a, cp, e, t, valid, me, Jinv, J4, Qs, R4, Wk, sDr, sSn);
-  if (a.cfl_out && threadIdx.x == 0) cfl_block_finish(a, red, (int)(blockDim.x >> 5));
+  if (a.cfl_out && threadIdx.x == 0) cfl_block_finish(a, red, (int)((blockDim.x + 31) >> 5));
 }
 
 // ---------------------------------------------------------------------------
