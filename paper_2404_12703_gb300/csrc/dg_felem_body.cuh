@@ -7,8 +7,8 @@
 // GPU), so that wave's loads find them in L2.
 //
 // This file is included inside the body of each kernel that runs this work
-// (k_felem, k_fpersist), with in scope: the template parameters N, MODE and
-// EPB_, the kernel's StageArgs parameter `a`, the element block `blk`, the
+// (k_felem, k_fpersist), with in scope: the template parameters N, MODE, EPB_
+// and EXTRA (shock capturing, sponge or source possible), the kernel's StageArgs parameter `a`, the element block `blk`, the
 // stage coefficients `sc` (A(), B(), C(), fA(), first()) and the dynamic
 // shared memory `smraw`.  It is text, not a function: behind a function that
 // takes the StageArgs by reference, the compiler holds the parameter fields
@@ -106,7 +106,7 @@ do {
     }
     cp_async_commit();
     // the FP64 pressure only for the indicator (one FP64 addition less otherwise)
-    const SPrim<float> me = shifted_prim<float, true>(U, a.gm1, a.Rinv, cp, a.shock ? &p_full : nullptr);
+    const SPrim<float> me = shifted_prim<float, true>(U, a.gm1, a.Rinv, cp, EXTRA && a.shock ? &p_full : nullptr);
     // halved values: every arithmetic mean of the two-point flux is one addition
     const int vp = pad_idx<n>(t);
     P4[vp] = make_float4(0.5f * me.rho, 0.5f * me.u, 0.5f * me.v, 0.5f * me.w);
@@ -227,7 +227,7 @@ do {
       }
     }
     // ---- shock capturing: indicator and FV sub-cell blending (Sec. 2.3) ----
-    if (a.shock) {
+    if (EXTRA && a.shock) {
       double al;
       if (a.alpha_force >= 0) {
         al = a.alpha_force;
@@ -300,7 +300,7 @@ do {
   #pragma unroll
     for (int k = 0; k < 5; ++k) ut32[k] = -(accC[k] + acc[k]) * Jinv;
     // the FP64 tendency: for dg_rhs, and in a stage with sources
-    const bool sources = a.sponge_sigma || a.source;
+    const bool sources = EXTRA && (a.sponge_sigma || a.source);
     double Ut[5];
     if (MODE == 0 || sources) {
   #pragma unroll

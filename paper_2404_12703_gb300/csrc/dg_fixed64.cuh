@@ -206,7 +206,7 @@ __device__ __forceinline__ ElemRef elem_ref(const StageArgs& a, int slot) {
 }
 
 // ApplyJac of a node's sums s, the sources, and Ut or the RK update
-template <int n, int MODE>
+template <int n, int MODE, bool EXTRA>
 __device__ __forceinline__ void finish_node64(const StageArgs& a, int e, int ce, int v, const double s[5]) {
   constexpr int n3 = n * n * n;
   const double Ji = -a.metric[((size_t)e * 10 + 9) * n3 + v];
@@ -214,13 +214,13 @@ __device__ __forceinline__ void finish_node64(const StageArgs& a, int e, int ce,
   load_state64<n>(a, e, v, U);
 #pragma unroll
   for (int k = 0; k < 5; ++k) Ut[k] = s[k] * Ji;
-  if (a.sponge_sigma) {  // sponge source -sigma (U - U_base)
+  if (EXTRA && a.sponge_sigma) {  // sponge source -sigma (U - U_base)
     const double sg = a.sponge_sigma[(size_t)e * n3 + v];
     const double* ub = a.sponge_base + (size_t)e * 5 * n3 + v;
 #pragma unroll
     for (int k = 0; k < 5; ++k) Ut[k] -= sg * (U[k] - ub[k * n3]);
   }
-  if (a.source) {  // manufactured-solution source
+  if (EXTRA && a.source) {  // manufactured-solution source
     double Q[5];
     mms_source(a, a.xyzs + ((size_t)e * n3 + v) * 3, stage_time(a, MODE), Q);
 #pragma unroll
@@ -674,7 +674,8 @@ __device__ void kep_f64(const double2* P, const double2* Jab, const double* Jc, 
   }
 }
 
-template <int N, int MODE>
+// EXTRA: a run with shock capturing, a sponge or a source
+template <int N, int MODE, bool EXTRA>
 __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_volume_fx(StageArgs a) {
   using F = Fix<N>;
   using L = VolFix<N>;
@@ -897,7 +898,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     }
   }
   // ---- shock capturing: indicator and FV sub-cell blending (Sec. 2.3) ----
-  if (a.shock) {
+  if (EXTRA && a.shock) {
     double al;
     if (a.alpha_force >= 0) {
       al = a.alpha_force;
@@ -995,7 +996,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
 #pragma unroll
       for (int k = 0; k < 5; ++k) s[k] += sg * Fs[k * n2];
     }
-    finish_node64<n, MODE>(a, e, er.ce, v, s);
+    finish_node64<n, MODE, EXTRA>(a, e, er.ce, v, s);
   }
 }
 

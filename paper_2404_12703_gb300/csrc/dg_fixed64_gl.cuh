@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
         sum[r][k] = fx_to((acc[r][k] >> min(pV - p, 63)) + (s.get() >> min(pS - p, 63)), p);
       }
     }
-    finish_node64<n, MODE>(a, e, er.ce, v, sum[r]);
+    finish_node64<n, MODE, true>(a, e, er.ce, v, sum[r]);
   }
 }
 

@@ -31,6 +31,7 @@
 #pragma once
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "dg_common.cuh"
 #include "dg_launch.h"
@@ -805,7 +806,7 @@ __global__ void __launch_bounds__(256) k_surf_flux(StageArgs a) {
 // 4 n2 doubles) may be reused after the caller's next barrier.
 // ---------------------------------------------------------------------------
 template <int n, int TPE = n * n * n>
-__device__ double element_alpha(double* sT1, double* sT2, double* sRow, const double* sVinv, const Ops* ops, int t,
+__device__ __noinline__ double element_alpha(double* sT1, double* sT2, double* sRow, const double* sVinv, const Ops* ops, int t,
                                 double amin, double amax) {
   constexpr int n2 = n * n, n3 = n2 * n, N = n - 1;
   __syncwarp();
@@ -1334,6 +1335,8 @@ struct Variants {
   static constexpr bool fp64 = sizeof(T) == sizeof(double);
 };
 
+// the kernels' code for shock capturing, a sponge or a source is needed
+inline bool extras(const StageArgs& a) { return a.shock || a.sponge_sigma || a.source; }
 // SMs of the current device
 inline int sm_count() {
   static int sms = 0;
@@ -1381,7 +1384,9 @@ inline void launch_vol(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
   if constexpr (FX) {
     const int epb = fx_epb<N>(S::EPB, a.E);
-    k_volume_fx<N, MODE><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(a);
+    const unsigned nb = (unsigned)((a.E + epb - 1) / epb);
+    if (extras(a)) k_volume_fx<N, MODE, true><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(a);
+    else k_volume_fx<N, MODE, false><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(a);
   } else {
     k_volume<N, MODE, T, E>
         <<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
@@ -1442,8 +1447,10 @@ cudaError_t stage_set_attrs() {
   if constexpr (V::fp64) {
     lift(k_lift_fx<N>, LiftFix<N>::bytes(V::lift2 ? 2 * V::D : V::D));
     const size_t vb = VolFix<N>::bytes(V::vol2 ? 2 * V::D : V::D);
-    lift(k_volume_fx<N, 0>, vb);
-    lift(k_volume_fx<N, 1>, vb);
+    lift(k_volume_fx<N, 0, false>, vb);
+    lift(k_volume_fx<N, 1, false>, vb);
+    lift(k_volume_fx<N, 0, true>, vb);
+    lift(k_volume_fx<N, 1, true>, vb);
   } else {
     lift(k_lift<N, T, 0>, lift_smem_bytes<N, T, 0>());
     if constexpr (V::lift2) lift(k_lift<N, T, 2 * V::D>, lift_smem_bytes<N, T, 2 * V::D>());
@@ -1463,9 +1470,14 @@ cudaError_t stage_set_attrs() {
   if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D>, VolumeSmem<N, T, 2 * V::D>::bytes);
   if constexpr (!V::fp64) {
     lift(k_fprep<N>, FusedSmem<N>::bytes);
-    lift(k_felem<N, 0, 0>, FusedSmem<N, 0>::bytes);
-    lift(k_felem<N, 1, 0>, FusedSmem<N, 0>::bytes);
-    if constexpr (V::vol2) lift(k_felem<N, 1, 2 * V::D>, FusedSmem<N, 2 * V::D>::bytes);
+    auto felem = [&](auto extra) {
+      constexpr bool X = decltype(extra)::value;
+      lift(k_felem<N, 0, 0, X>, FusedSmem<N, 0>::bytes);
+      lift(k_felem<N, 1, 0, X>, FusedSmem<N, 0>::bytes);
+      if constexpr (V::vol2) lift(k_felem<N, 1, 2 * V::D, X>, FusedSmem<N, 2 * V::D>::bytes);
+    };
+    felem(std::false_type());
+    felem(std::true_type());
     // the prefetch distances, queried here (context set-up) and not during
     // the capture of a step graph
     felem_wave<N, 0>();
@@ -1479,7 +1491,7 @@ cudaError_t stage_set_attrs() {
 // ---------------------------------------------------------------------------
 // The two-kernel FP32-bulk stage (dg_fused32.cuh)
 // ---------------------------------------------------------------------------
-// blocks of k_felem<N, 1, E> resident per SM times the SM count: the L2
+// blocks of k_felem<N, 1, E, false> resident per SM times the SM count: the L2
 // prefetch distance (one wave ahead)
 template <int N, int E>
 inline int felem_wave() {
@@ -1488,7 +1500,7 @@ inline int felem_wave() {
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_felem<N, 1, E>, Shape<N, E>::THREADS,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_felem<N, 1, E, false>, Shape<N, E>::THREADS,
                                                       FusedSmem<N, E>::bytes) == cudaSuccess &&
         sms > 0 && per > 0)
       wave = sms * per;
@@ -1563,7 +1575,9 @@ template <int N, int MODE, int E>
 inline void launch_felem(StageArgs a, int prefetch, cudaStream_t st) {
   using S = Shape<N, E>;
   a.prefetch = prefetch ? std::max(0, felem_wave<N, E>()) : 0;
-  k_felem<N, MODE, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, FusedSmem<N, E>::bytes, st>>>(a);
+  const unsigned nb = (unsigned)((a.E + S::EPB - 1) / S::EPB);
+  if (extras(a)) k_felem<N, MODE, E, true><<<nb, S::THREADS, FusedSmem<N, E>::bytes, st>>>(a);
+  else k_felem<N, MODE, E, false><<<nb, S::THREADS, FusedSmem<N, E>::bytes, st>>>(a);
 }
 template <int N>
 inline void launch_fflux(const StageArgs& a, int block, cudaStream_t st) {
