@@ -1435,6 +1435,8 @@ inline void vol_variant(const StageArgs& a, int epb, int pairs, cudaStream_t st)
 template <int N, int E>
 inline int felem_wave();
 template <int N>
+constexpr bool felem_single();
+template <int N>
 inline int persist_grid();
 
 template <int N, typename T>
@@ -1474,10 +1476,15 @@ cudaError_t stage_set_attrs() {
       constexpr bool X = decltype(extra)::value;
       lift(k_felem<N, 0, 0, X>, FusedSmem<N, 0>::bytes);
       lift(k_felem<N, 1, 0, X>, FusedSmem<N, 0>::bytes);
+      if constexpr (felem_single<N>()) {
+        lift(k_felem<N, 0, 1, X>, FusedSmem<N, 1>::bytes);
+        lift(k_felem<N, 1, 1, X>, FusedSmem<N, 1>::bytes);
+      }
       if constexpr (V::vol2) lift(k_felem<N, 1, 2 * V::D, X>, FusedSmem<N, 2 * V::D>::bytes);
     };
     felem(std::false_type());
     felem(std::true_type());
+    if constexpr (felem_single<N>()) felem_wave<N, 1>();
     // the prefetch distances, queried here (context set-up) and not during
     // the capture of a step graph
     felem_wave<N, 0>();
@@ -1602,9 +1609,19 @@ inline cudaError_t fprep_launch(dg_ctx* c, const double* U, int64_t e0 = 0, int6
   count_launch();
   return cudaGetLastError();
 }
+// One element per block on small meshes (N = 3, where a block holds four):
+// 4^3 elements then reach 64 SMs instead of 16 (ten steps of 4^3 elements 912 -> 780 us)
+template <int N>
+constexpr bool felem_single() {
+  return Shape<N>::EPB_DEFAULT > 1 && Shape<N>::n3 >= 64 && Shape<N>::n3 % 32 == 0;
+}
 template <int N>
 inline void felem_variant(const StageArgs& a, int mode, int epb, int prefetch, cudaStream_t st) {
   using V = Variants<N, float>;
+  if constexpr (felem_single<N>()) {
+    if ((a.E + V::D - 1) / V::D < sm_count())
+      return mode == 0 ? launch_felem<N, 0, 1>(a, 0, st) : launch_felem<N, 1, 1>(a, prefetch, st);
+  }
   if (mode == 0) return launch_felem<N, 0, 0>(a, 0, st);
   if constexpr (V::vol2) {
     if (epb == 2 * V::D) return launch_felem<N, 1, 2 * V::D>(a, prefetch, st);
