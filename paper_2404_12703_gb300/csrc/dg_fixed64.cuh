@@ -205,6 +205,31 @@ __device__ __forceinline__ ElemRef elem_ref(const StageArgs& a, int slot) {
   return r;
 }
 
+// Asks L2 for what an element block reads later on (its lifting fluxes or its
+// gradients, register and surface fluxes), and for the state and metrics of
+// the element a wave of blocks further on: each phase of a block then waits
+// on L2 instead of on memory.  One thread per side or array.
+template <int N>
+__device__ __forceinline__ void prefetch_sides64(const StageArgs& a, int e, const double* base, int comps, int t) {
+  constexpr int n2 = Fix<N>::n2;
+  if (t < 6) {
+    const size_t w = (size_t)comps * n2, s = (size_t)es_side(a.elem_side[(size_t)e * 6 + t]) * w;
+    prefetch_l2(base + s, 8 * w, base + s, base + s + w);
+  }
+}
+__device__ __forceinline__ void prefetch64(const double* base, size_t first, size_t count) {
+  prefetch_l2(base + first, 8 * count, base + first, base + first + count);
+}
+template <int N>
+__device__ __forceinline__ void prefetch_next64(const StageArgs& a, int slot, int t) {
+  constexpr int n3 = Fix<N>::n3;
+  if (slot < a.E && t >= 0 && t < 2) {
+    const size_t e = a.elem_list ? a.elem_list[slot] : slot;
+    if (t == 0) prefetch64(a.U, e * 5 * n3, 5 * n3);
+    else prefetch64(a.metric, e * 10 * n3, 10 * n3);
+  }
+}
+
 // ApplyJac of a node's sums s, the sources, and Ut or the RK update
 template <int n, int MODE, bool EXTRA>
 __device__ __forceinline__ void finish_node64(const StageArgs& a, int e, int ce, int v, const double s[5]) {
@@ -395,6 +420,8 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
   const int e = er.e;
   const double* Me = a.metric + (size_t)e * 10 * n3;
   lift_table_fx<N>(a.ops, sD);
+  prefetch_sides64<N>(a, e, a.lflux, 12, t);
+  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
   {
     unsigned m[5];
     lift_prims_fx<N>(a, e, q, m, t);
@@ -707,6 +734,10 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     sVi[k] = a.ops->Vinv[k];
     if (k < n) sW[k] = fx_split(a.ops->fxW[k]);
   }
+  prefetch_sides64<N>(a, e, a.fstar, 5, t);
+  if (t == 6 && a.viscous) prefetch64(a.g, (size_t)e * 12 * n3, 12 * n3);
+  if (t == 7 && MODE == 1 && !a.first_stage) prefetch64(a.dU, (size_t)e * 5 * n3, 5 * n3);
+  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
   // ---- primitives (FP64 in their planes until the scales are known), maxima ----
   {
     unsigned m[VQ_N];

@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
   const double* Me = a.metric + (size_t)e * 10 * n3;
   lift_table_fx<N>(a.ops, sD);
   for (int k = threadIdx.x; k < 2 * n; k += blockDim.x) sL[k] = fx_split(a.ops->fxL[k]), sE[k] = fx_split(a.ops->fxE[k]);
+  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
   {
     unsigned m[11];  // those of lift_prims_fx, then the faces' fluxes: velocity and temperature by Cartesian component
     lift_prims_fx<N>(a, e, q, m, t);
@@ -226,6 +227,8 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
     sDh[k] = fx_split(a.ops->fxH[k]);
     if (k < 2 * n) sL[k] = fx_split(a.ops->fxL[k]);
   }
+  if (t == 7 && MODE == 1 && !a.first_stage) prefetch64(a.dU, (size_t)e * 5 * n3, 5 * n3);
+  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
   {
     unsigned m[L::Q];
 #pragma unroll

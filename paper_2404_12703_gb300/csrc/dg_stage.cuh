@@ -1368,12 +1368,17 @@ inline int fx_epb(int E, int64_t elems) {
   while (E > least && (elems + E - 1) / E < 2 * sm_count()) E = std::max(least, E / 2 / least * least);
   return E;
 }
+// the prefetch distance in blocks: about the blocks the GPU holds at once
+// (128 registers per thread)
+inline int fx_wave(int threads) { return sm_count() * std::max(1, 512 / threads); }
 template <int N, typename T, int E>
 inline void launch_lift(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
   if constexpr (sizeof(T) == sizeof(double)) {
     const int epb = fx_epb<N>(S::EPB, a.E);
-    k_lift_fx<N><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, LiftFix<N>::bytes(epb), st>>>(a);
+    StageArgs b = a;
+    b.prefetch = fx_wave(Fix<N>::TPE * epb);
+    k_lift_fx<N><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, LiftFix<N>::bytes(epb), st>>>(b);
   } else {
     k_lift<N, T, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, lift_smem_bytes<N, T, E>(), st>>>(a);
   }
@@ -1385,8 +1390,10 @@ inline void launch_vol(const StageArgs& a, cudaStream_t st) {
   if constexpr (FX) {
     const int epb = fx_epb<N>(S::EPB, a.E);
     const unsigned nb = (unsigned)((a.E + epb - 1) / epb);
-    if (extras(a)) k_volume_fx<N, MODE, true><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(a);
-    else k_volume_fx<N, MODE, false><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(a);
+    StageArgs b = a;
+    b.prefetch = fx_wave(Fix<N>::TPE * epb);
+    if (extras(a)) k_volume_fx<N, MODE, true><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
+    else k_volume_fx<N, MODE, false><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
   } else {
     k_volume<N, MODE, T, E>
         <<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
@@ -1680,6 +1687,7 @@ cudaError_t stage_launch_gl(dg_ctx* c, const double* U, int mode, double rkA, do
   constexpr bool fx = sizeof(T) == sizeof(double);  // the fixed-point kernels
   const int epb = fx_epb<N>(S::EPB, a.E);
   const unsigned nbx = (unsigned)((a.E + epb - 1) / epb);
+  if (fx) a.prefetch = fx_wave(Fix<N>::TPE * epb);
   const int sb = c->cfg.side_block;
   prof_begin(c, PK_SURF_PRIMS);
   k_prolong_gl<N><<<nb, S::THREADS, gl_prolong_smem<N>(), c->stream>>>(a);
