@@ -237,6 +237,18 @@ __device__ __forceinline__ void finish_node64(const StageArgs& a, int e, int ce,
   const double Ji = -a.metric[((size_t)e * 10 + 9) * n3 + v];
   double Ut[5], U[5];
   load_state64<n>(a, e, v, U);
+  if constexpr (!EXTRA && MODE == 1) {  // (no sources: dt / J in one factor)
+    const double c = Ji * case_dt(a, ce);
+    double* du = a.dU + (size_t)e * 5 * n3 + v;
+    double* uo = a.Urk + (size_t)e * 5 * n3 + v;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const double x = a.first_stage ? s[k] * c : a.rkA * du[k * n3] + s[k] * c;
+      du[k * n3] = x;
+      uo[k * n3] = U[k] + a.rkB * x;
+    }
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < 5; ++k) Ut[k] = s[k] * Ji;
   if (EXTRA && a.sponge_sigma) {  // sponge source -sigma (U - U_base)
@@ -800,6 +812,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
   kep_fx<N>(P, Jab, Jc, A, sS, sW, sc, t, bad);
   double conv[R][5];  // convective DG volume term
   double visc[R][4];  // viscous volume term
+  long long vel[R][3];  // the velocity in fixed point (FP64 values in a bad element)
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int v = t + r * TPE, pv = fx_pad<n>(v < n3 ? v : 0);
@@ -818,29 +831,41 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) visc[r][k] = 0.0;
+    vel[r][0] = P[Pn + pv].x, vel[r][1] = P[Pn + pv].y, vel[r][2] = P[2 * Pn + pv].x;
   }
   __syncwarp();
   __syncthreads();  // the primitives' and sums' planes are free
   // ---- viscous volume term: collocated weak form, per direction ----
   if (a.viscous) {
-    long long* T = mine + L::offT;  // [9][n3]: tau, W; each thread reads back its own nodes only
+    // [9][n3]: tau and lambda grad T, then tau and W = tau u + lambda grad T
+    // (the work term in fixed point: 19 FP64 operations less per node); each
+    // thread reads back its own nodes only
+    long long* T = mine + L::offT;
     {
       unsigned mv[2] = {0, 0};
       for (int v = t; v < n3; v += TPE) {
-        double g[12], U[5];
+        double g[12];
         const double* pg = a.g + (size_t)e * 12 * n3 + v;
 #pragma unroll
         for (int k = 0; k < 12; ++k) g[k] = pg[k * n3];
-        load_state64<n>(a, e, v, U);
-        const Prim64 pr = prim64(U, a.gm1);
-        double tau[6], W[3], vmu, vlam;
-        visc_coeffs<double>(a, cp, a.sutherland ? pr.p * pr.ri * a.Rinv : 0.0, vmu, vlam);
-        viscous_parts(g, pr.u, pr.v, pr.w, vmu, vlam, tau, W);
+        double vmu, vlam, Tt = 0.0;
+        if (a.sutherland) {
+          double U[5];
+          load_state64<n>(a, e, v, U);
+          const Prim64 pr = prim64(U, a.gm1);
+          Tt = pr.p * pr.ri * a.Rinv;
+        }
+        visc_coeffs<double>(a, cp, Tt, vmu, vlam);
+        const double tw = (2.0 / 3.0) * (g[0] + g[4] + g[8]);
+        const double x[9] = {vmu * (2.0 * g[0] - tw), vmu * (2.0 * g[4] - tw), vmu * (2.0 * g[8] - tw),
+                             vmu * (g[1] + g[3]),     vmu * (g[2] + g[6]),     vmu * (g[5] + g[7]),
+                             vlam * g[9],             vlam * g[10],            vlam * g[11]};
         double* Td = reinterpret_cast<double*>(T) + v;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) Td[k * n3] = tau[k], mv[0] = max(mv[0], fx_mag(tau[k]));
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Td[(6 + k) * n3] = W[k], mv[1] = max(mv[1], fx_mag(W[k]));
+        for (int k = 0; k < 9; ++k) {
+          Td[k * n3] = x[k];
+          mv[k / 6] = max(mv[k / 6], fx_mag(x[k]));
+        }
       }
       fx_reduce<N, 2>(mv, red, fin, t);
       __syncthreads();
@@ -848,16 +873,51 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     // (an element that leaves the range only here has its metrics in fixed
     // point: the FP64 sums then read them from memory)
     const bool vbad = bad || fx_bad(fin[0]) || fx_bad(fin[1]);
-    const int eT = fx_exp(fin[0]), eW = fx_exp(fin[1]), eJm = max(max(sc->d[0].eJ, sc->d[1].eJ), sc->d[2].eJ);
+    const int eT = fx_exp(fin[0]), eL = fx_exp(fin[1]), eJm = max(max(sc->d[0].eJ, sc->d[1].eJ), sc->d[2].eJ);
+    const int eTU = eT + sc->eU, eW = max(eTU, eL) + 2;  // W: below 2^60 at 2^(60 - eW)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int v = t + r * TPE;
+      if (v >= n3) break;
+      if (vbad) {
+        double u[3];
+        if (bad) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) u[k] = __longlong_as_double(vel[r][k]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) u[k] = fx_to(vel[r][k], 60 - sc->eU);
+        }
+        double* Td = reinterpret_cast<double*>(T) + v;
+        const double t0 = Td[0], t1 = Td[n3], t2 = Td[2 * n3], t3 = Td[3 * n3], t4 = Td[4 * n3], t5 = Td[5 * n3];
+        Td[6 * n3] = t0 * u[0] + t3 * u[1] + t4 * u[2] + Td[6 * n3];
+        Td[7 * n3] = t3 * u[0] + t1 * u[1] + t5 * u[2] + Td[7 * n3];
+        Td[8 * n3] = t4 * u[0] + t5 * u[1] + t2 * u[2] + Td[8 * n3];
+      } else {
+        Fx x[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const long long q = fx_from<60>(__longlong_as_double(T[k * n3 + v]), eT);
+          T[k * n3 + v] = q;
+          x[k] = fx_split(q);
+        }
+        const Fx u = fx_split(vel[r][0]), w1 = fx_split(vel[r][1]), w2 = fx_split(vel[r][2]);
+        FxSum<2> w[3];  // 3 2^(60 + 60 - 64 + 2) < 2^59.6
+        w[0].add(x[0], u), w[0].add(x[3], w1), w[0].add(x[4], w2);
+        w[1].add(x[3], u), w[1].add(x[1], w1), w[1].add(x[5], w2);
+        w[2].add(x[4], u), w[2].add(x[5], w1), w[2].add(x[2], w2);
+        const int sU = min(eW - 2 - eTU, 63), sL = min(eW - 2 - eL, 63);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          T[(6 + k) * n3 + v] =
+              (w[k].get() >> sU) + (fx_from<58>(__longlong_as_double(T[(6 + k) * n3 + v]), eL) >> sL);
+      }
+    }
     long long acc[R][4];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[r][k] = 0;
-    if (!vbad)
-      for (int v = t; v < n3; v += TPE)
-#pragma unroll
-        for (int k = 0; k < 9; ++k) T[k * n3 + v] = fx_from<60>(__longlong_as_double(T[k * n3 + v]), k < 6 ? eT : eW);
 #pragma unroll 1
     for (int d = 0; d < 3; ++d) {
       for (int v = t; v < n3; v += TPE) {
