@@ -144,6 +144,29 @@ __device__ __forceinline__ int dir_stride(int d) {
   return d == 0 ? 1 : (d == 1 ? n : n * n);
 }
 
+// two FP32 operations in one instruction (each rounded as its scalar form)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void un2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 
@@ -600,8 +623,10 @@ __device__ __forceinline__ void fflux_body(const StageArgs& a, int64_t tid) {
   for (int k = 0; k < 5; ++k) out[k * n2] = f[k];
 }
 
+// four blocks per SM: it waits on gathered records (32^3 elements, N = 5, where
+// it took 77 registers and three blocks: 204 -> 177 us)
 template <int N>
-__global__ void __launch_bounds__(256) k_fflux(StageArgs a) {
+__global__ void __launch_bounds__(256, 4) k_fflux(StageArgs a) {
   fflux_body<N>(a, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
 }
 
