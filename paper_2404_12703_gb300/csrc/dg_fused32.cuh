@@ -199,7 +199,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes, const v
 // calls it (it holds barriers); W may be reused after the caller's next
 // barrier.
 // ---------------------------------------------------------------------------
-template <int n, int n4, bool READ = true>
+template <int n, int n4, bool READ>
 __device__ __forceinline__ void lift_volume(const float* Qs, const float4* J4, float* W, const float* sDr2, int t,
                                             float acc[12]) {
   constexpr int n2 = n * n, n3 = n2 * n, Pn = n3 + n2;

@@ -534,16 +534,23 @@ __global__ void __launch_bounds__(256) k_surf_prims(StageArgs a) {
 // Lifted gradients (weak form, Eq. lifting)
 // ---------------------------------------------------------------------------
 // (FP32-bulk; the FP64 lifting is k_lift_fx in dg_fixed64.cuh)
+template <int n, int n4, bool READ = true>
+__device__ __forceinline__ void lift_volume(const float* Qs, const float4* J4, float* W, const float* sDr2, int t,
+                                            float acc[12]);  // dg_fused32.cuh
+
 template <int N, typename T, int EPB_ = 0>
 __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
+  // line tasks as in the element kernel's epilogue (lift_volume): each loads a
+  // line's values once and keeps the products in registers (16 x 8 x 16
+  // channel, N = 7: 71 us with one node per thread over a product tile, now 66)
   using S = Shape<N, EPB_>;
-  constexpr int n = S::n, n2 = S::n2, n3 = S::n3, EPB = S::EPB;
-  constexpr int n2p = (n2 + 3) & ~3;  // keeps the arrays below 16-byte aligned
+  constexpr int n = S::n, n2 = S::n2, n3 = S::n3, EPB = S::EPB, Pn = n3 + n2, n4 = (n + 3) & ~3;
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* sDh = reinterpret_cast<T*>(smraw);  // [n2p]
-  T* sq = sDh + n2p;                     // [EPB][4][n3]
-  T* sF = sq + EPB * 4 * n3;             // [EPB][12][n3]
+  float* sDr = reinterpret_cast<float*>(smraw);  // [n][n4] 2 Dhat, rows padded
   const int le = threadIdx.x / n3, t = threadIdx.x % n3;
+  float* Qs = sDr + n * n4 + (size_t)le * 28 * Pn;       // [4][Pn] u, v, w, T', padded index
+  float4* J4 = reinterpret_cast<float4*>(Qs + 4 * Pn);   // [3][Pn] (Ja^d) / 2
+  float* Wk = Qs + 16 * Pn;                              // [12][Pn] the sums
   // Slots past the last element redo the last element in their own shared
   // memory slot, so that every thread of a block runs the same path through
   // the barriers; only the final global stores are masked.
@@ -558,88 +565,31 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
   const bool busy = valid && !(a.cases && a.cases[ce].dt == 0.0);
   if (a.elem_case && __syncthreads_and(!busy)) return;
   const CaseParams cp = case_params(a, ce);
-  for (int k = threadIdx.x; k < n2; k += blockDim.x) sDh[k] = T(a.ops->Dhat[k]);
-  T* q = sq + le * 4 * n3;
-  T* F = sF + le * 12 * n3;
-  // FP32: the node's ten metric values are loaded up front, so that their
-  // latency overlaps the state loads instead of following each barrier
-  constexpr bool pre = sizeof(T) == sizeof(float);
-  T Mpre[pre ? 10 : 1];
-  if constexpr (pre) {
-#pragma unroll
-    for (int c = 0; c < 10; ++c) Mpre[c] = metric_at<T>(a, e, c, t, n3);
+  for (int k = threadIdx.x; k < n * n4; k += blockDim.x) {
+    const int i = k / n4, al = k % n4;
+    sDr[k] = al < n ? 2.0f * (float)a.ops->Dhat[i * n + al] : 0.0f;
   }
-  auto Mv = [&](int c) -> T {
-    if constexpr (pre) return Mpre[c];
-    else return metric_at<T>(a, e, c, t, n3);
-  };
+  T mt[10];
+#pragma unroll
+  for (int c = 0; c < 10; ++c) mt[c] = metric_at<T>(a, e, c, t, n3);
+  const int vp = t + t / n;
   {
     double U[5];
     const double* u = a.U + (size_t)e * 5 * n3 + t;
 #pragma unroll
     for (int k = 0; k < 5; ++k) U[k] = u[k * n3];
     const SPrim<T> pr = shifted_prim<T>(U, a.gm1, a.Rinv, cp);
-    q[t] = pr.u;
-    q[n3 + t] = pr.v;
-    q[2 * n3 + t] = pr.w;
-    q[3 * n3 + t] = pr.Tt;
+    Qs[vp] = pr.u, Qs[Pn + vp] = pr.v, Qs[2 * Pn + vp] = pr.w, Qs[3 * Pn + vp] = pr.Tt;
   }
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    J4[d * Pn + vp] = make_float4(0.5f * mt[3 * d], 0.5f * mt[3 * d + 1], 0.5f * mt[3 * d + 2], 0.0f);
+  const T Ji = mt[9];
   __syncwarp();
   __syncthreads();
-  const int idx[3] = {t % n, (t / n) % n, t / n2};
-  constexpr int str[3] = {1, n, n2};
   T acc[12];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) acc[c] = T(0);
-  // FP32 (bound by shared-memory load instructions): the products are stored
-  // as six float2 planes, halving the loads of the line sums
-  constexpr bool pairs2 = sizeof(T) == sizeof(float);
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    {
-      const T J0 = Mv(d * 3 + 0), J1 = Mv(d * 3 + 1), J2 = Mv(d * 3 + 2);
-      T pr[12];
-#pragma unroll
-      for (int qv = 0; qv < 4; ++qv) {
-        const T qq = q[qv * n3 + t];
-        pr[qv * 3 + 0] = J0 * qq;
-        pr[qv * 3 + 1] = J1 * qq;
-        pr[qv * 3 + 2] = J2 * qq;
-      }
-      if constexpr (pairs2) {
-        float2* F2 = reinterpret_cast<float2*>(F);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) F2[k * n3 + t] = make_float2(pr[2 * k], pr[2 * k + 1]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) F[k * n3 + t] = pr[k];
-      }
-    }
-    __syncwarp();
-    __syncthreads();
-    {
-      const int id = idx[d], base = t - id * str[d];
-#pragma unroll
-      for (int al = 0; al < n; ++al) {
-        const T c = sDh[id * n + al];
-        const int nb = base + al * str[d];
-        if constexpr (pairs2) {
-          const float2* F2 = reinterpret_cast<const float2*>(F);
-#pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const float2 v = F2[k * n3 + nb];
-            acc[2 * k] += c * v.x;
-            acc[2 * k + 1] += c * v.y;
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 12; ++k) acc[k] += c * F[k * n3 + nb];
-        }
-      }
-    }
-    __syncwarp();
-    __syncthreads();
-  }
+  lift_volume<n, n4>(Qs, J4, Wk, sDr, t, acc);
+  const int idx[3] = {t % n, (t / n) % n, t / n2};
   if (!valid) return;
   // surface part: on LGL nodes only face nodes receive it
   const T* Lf = TBuf<T>::lflux(a);
@@ -659,7 +609,6 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] += sg * L[k * n2];
   }
-  const T Ji = Mv(9);
   T* g = TBuf<T>::g(a) + (size_t)e * 12 * n3 + t;
 #pragma unroll
   for (int k = 0; k < 12; ++k) g[k * n3] = acc[k] * Ji;
@@ -1320,7 +1269,7 @@ inline StageArgs make_stage_args(dg_ctx* c, const double* U) {
 template <int N, typename T, int E = 0>
 inline size_t lift_smem_bytes() {
   using S = Shape<N, E>;
-  return sizeof(T) * (((S::n2 + 3) & ~3) + S::EPB * 16 * S::n3);
+  return sizeof(T) * (S::n * ((S::n + 3) & ~3) + S::EPB * 28 * (S::n3 + S::n2));
 }
 
 // Launch variants the autotuner chooses among: the default elements per
