@@ -191,8 +191,7 @@ __device__ __forceinline__ double case_dt(const StageArgs& a, int c) {
 // same values as the hardware conversions, off the FP64 unit, which the six
 // conversions of a state kept 80 % busy in the surface prolongation; 16 x 8 x
 // 16 channel, N = 7: k_surf_prims 20.1 -> 17.1 us, k_surf_flux 31.1 -> 29.8
-// us).  Not in the lifting, where the integer instructions cost more than the
-// conversions (71.4 -> 77.9 us).
+// us; k_lift 65.6 -> 63.5 us).
 template <typename T, bool INTCVT = false>
 __device__ __forceinline__ SPrim<T> shifted_prim(const double U[5], double gm1, double Rinv, const CaseParams& cp,
                                                 double* p_full = nullptr) {
@@ -578,7 +577,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
     const double* u = a.U + (size_t)e * 5 * n3 + t;
 #pragma unroll
     for (int k = 0; k < 5; ++k) U[k] = u[k * n3];
-    const SPrim<T> pr = shifted_prim<T>(U, a.gm1, a.Rinv, cp);
+    const SPrim<T> pr = shifted_prim<T, true>(U, a.gm1, a.Rinv, cp);
     Qs[vp] = pr.u, Qs[Pn + vp] = pr.v, Qs[2 * Pn + vp] = pr.w, Qs[3 * Pn + vp] = pr.Tt;
   }
 #pragma unroll
@@ -849,7 +848,9 @@ struct VolumeSmem {
 // One node per thread, which sums over all its partners: FP32-bulk, and FP64's
 // other mapping (dg_set_config; the default FP64 kernel is k_volume_fx in
 // dg_fixed64.cuh).
-template <int N, int MODE, typename T, int EPB_ = 0>
+// EXTRA: a run with shock capturing, a sponge or a source; without their code
+// the FP32 kernel takes 114 instead of 117 us (16 x 8 x 16 channel, N = 7).
+template <int N, int MODE, typename T, int EPB_, bool EXTRA>
 __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::template vol_min_blocks<T>())
     k_volume(StageArgs a) {
   using S = Shape<N, EPB_>;
@@ -1050,7 +1051,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   __syncthreads();
 
   // ---- shock capturing: indicator and FV sub-cell blending (Sec. 2.3) ----
-  if (a.shock) {
+  if (EXTRA && a.shock) {
     double al;
     if (a.alpha_force >= 0) {
       al = a.alpha_force;
@@ -1144,13 +1145,13 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
 #pragma unroll
   for (int k = 0; k < 5; ++k) Ut[k] = to_f64<T>(-(accC[k] + acc[k]) * Ji);
   Ut[4] += H_ref * Ut[0];
-  if (a.sponge_sigma) {  // sponge source -sigma (U - U_base), FP64
+  if (EXTRA && a.sponge_sigma) {  // sponge source -sigma (U - U_base), FP64
     const double sg = a.sponge_sigma[(size_t)e * n3 + t];
     const double* ub = a.sponge_base + (size_t)e * 5 * n3 + t;
 #pragma unroll
     for (int k = 0; k < 5; ++k) Ut[k] -= sg * ((aos ? sUd[k * n3 + t] : U[k]) - ub[k * n3]);
   }
-  if (a.source) {  // manufactured-solution source, FP64
+  if (EXTRA && a.source) {  // manufactured-solution source, FP64
     double Q[5];
     mms_source(a, a.xyzs + ((size_t)e * n3 + t) * 3, stage_time(a, MODE), Q);
 #pragma unroll
@@ -1344,8 +1345,14 @@ inline void launch_vol(const StageArgs& a, cudaStream_t st) {
     if (extras(a)) k_volume_fx<N, MODE, true><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
     else k_volume_fx<N, MODE, false><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
   } else {
-    k_volume<N, MODE, T, E>
-        <<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
+    const unsigned nb = (unsigned)((a.E + S::EPB - 1) / S::EPB);
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (!extras(a)) {
+        k_volume<N, MODE, T, E, false><<<nb, S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
+        return;
+      }
+    }
+    k_volume<N, MODE, T, E, true><<<nb, S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
   }
 }
 template <int N, typename T, bool GL = false>
@@ -1412,7 +1419,10 @@ cudaError_t stage_set_attrs() {
   } else {
     lift(k_lift<N, T, 0>, lift_smem_bytes<N, T, 0>());
     if constexpr (V::lift2) lift(k_lift<N, T, 2 * V::D>, lift_smem_bytes<N, T, 2 * V::D>());
-    lift(k_volume<N, 0, T, 0>, VolumeSmem<N, T, 0>::bytes);
+    lift(k_volume<N, 0, T, 0, true>, VolumeSmem<N, T, 0>::bytes);
+    lift(k_volume<N, 0, T, 0, false>, VolumeSmem<N, T, 0>::bytes);
+    lift(k_volume<N, 1, T, 0, false>, VolumeSmem<N, T, 0>::bytes);
+    if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D, false>, VolumeSmem<N, T, 2 * V::D>::bytes);
   }
   lift(k_prolong_gl<N>, gl_prolong_smem<N>());
   if constexpr (V::fp64) {
@@ -1424,8 +1434,8 @@ cudaError_t stage_set_attrs() {
     lift(k_volume_gl<N, 0, T>, gl_volume_smem<N, T>());
     lift(k_volume_gl<N, 1, T>, gl_volume_smem<N, T>());
   }
-  lift(k_volume<N, 1, T, 0>, VolumeSmem<N, T, 0>::bytes);
-  if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D>, VolumeSmem<N, T, 2 * V::D>::bytes);
+  lift(k_volume<N, 1, T, 0, true>, VolumeSmem<N, T, 0>::bytes);
+  if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D, true>, VolumeSmem<N, T, 2 * V::D>::bytes);
   if constexpr (!V::fp64) {
     lift(k_fprep<N>, FusedSmem<N>::bytes);
     auto felem = [&](auto extra) {
