@@ -11,8 +11,58 @@ namespace dg {
 // ---------------------------------------------------------------------------
 // CFL reduction (the paper gives no rule; see dg_time_step in dg.h)
 // ---------------------------------------------------------------------------
-// T = float (FP32-bulk): the spectral radii in FP32, from the FP32 metrics alone
-template <int N, typename T>
+// Upper bounds of a node's FP64 radii, in FP32 and integer operations.  A
+// value's magnitude is cut to 20 fraction bits (lo) or raised above it (up);
+// out of FP32's range, not finite, or where the density or pressure may not be
+// positive (no sound speed, to be reported), the bounds are infinite or NaN.
+// Every product of bounds is raised by the smallest normal number, which
+// covers what underflows.
+__device__ __forceinline__ float mag_lo(double v) {
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  if (h < 897u << 20) return 0.0f;
+  if (h >= 1150u << 20) return __int_as_float(0x7f800000);
+  return __uint_as_float((h - (896u << 20)) << 3);
+}
+constexpr float kTiny = 1.2e-38f;  // above 2^-126
+__device__ __forceinline__ float mag_up(double v) { return __uint_as_float(__float_as_uint(mag_lo(v)) + 8u) + kTiny; }
+__device__ __forceinline__ float cut(double v) { return copysignf(mag_lo(v), __int_as_float(__double2hiint(v))); }
+__device__ __forceinline__ float mul_up(float a, float b) { return fmaf(a, b, kTiny); }
+__device__ __forceinline__ void radii_up(const double U[5], const double M[10], const double G[4], float gamma, float gm1,
+                                         float Rinv, float kv, int sutherland, float inv_Tref, float& aa, float& bb) {
+  constexpr float e = 1.0f + 1e-5f;  // covers the FP32 roundings of the few operations behind it
+  const float ri = e / mag_lo(U[0]) + kTiny;
+  const float m0 = cut(U[1]), m1 = cut(U[2]), m2 = cut(U[3]);
+  const float s2 = m0 * m0 + m1 * m1 + m2 * m2;
+  const float k2 = 0.5f * s2 * ri;  // the kinetic energy, at most 2e-5 of it above (or any amount below)
+  const float p = fmaf(e * gm1, mag_up(U[4]) - k2 * (1.0f - 5e-5f), kTiny);
+  const bool positive = U[0] > 0.0 && U[4] > 0.0 && mag_lo(U[4]) > e * mul_up(s2 + kTiny, ri);
+  const float c = positive ? e * sqrtf(mul_up(mul_up(e * gamma, p), ri)) : __int_as_float(0x7f800000);
+  float a = 0.0f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float j0 = cut(M[3 * d]), j1 = cut(M[3 * d + 1]), j2 = cut(M[3 * d + 2]);
+    // cutting a factor changes a product by less than 2^-18 of it, or (a
+    // factor or the product underflows) by kTiny times the other factor or 1
+    const float un = fabsf(m0 * j0 + m1 * j1 + m2 * j2) + 1e-5f * (fabsf(m0 * j0) + fabsf(m1 * j1) + fabsf(m2 * j2)) +
+                     kTiny * (6.0f + 2.0f * (fabsf(j0) + fabsf(j1) + fabsf(j2) + fabsf(m0) + fabsf(m1) + fabsf(m2)));
+    a += mul_up(un, ri) + mul_up(c, mag_up(G[d]));
+  }
+  const float Ji = mag_up(M[9]);
+  aa = e * mul_up(a, Ji);
+  float k = fmaf(e, kv, kTiny);
+  if (sutherland) {  // increasing in the temperature
+    const float th = e * mul_up(mul_up(mul_up(p, ri), Rinv + kTiny), inv_Tref + kTiny);
+    k = mul_up(k, e * 1.4042f * mul_up(th, sqrtf(th)) / (th + 0.4042f));
+  }
+  bb = e * mul_up(mul_up(mul_up(k, ri), mag_up(G[3])), mul_up(Ji, Ji));
+}
+
+// T = float (FP32-bulk): the spectral radii in FP32, from the FP32 metrics
+// alone.  T = double: bound by the FP64 unit (a division, a square root and
+// some thirty operations per node), so with PRUNE a node is evaluated only if
+// its upper bound exceeds the block's largest radius so far; the maximum is the
+// same (24^3 elements, N = 7: 610 -> 219 us per step).
+template <int N, typename T, bool PRUNE = false>
 __global__ void __launch_bounds__(256) k_cfl(int E, const double* __restrict__ U, const double* __restrict__ metric,
                                             const float* __restrict__ metric32, const double* __restrict__ geo,
                                             double gamma, double gm1, double Rinv, double kv, int viscous,
@@ -21,6 +71,11 @@ __global__ void __launch_bounds__(256) k_cfl(int E, const double* __restrict__ U
   constexpr bool f32 = sizeof(T) == sizeof(float);
   T lcT = T(0), lvT = T(0);  // per-thread maxima in the arithmetic type
   int bad = 0;
+  __shared__ int sc, sv;  // PRUNE: the block's maxima so far, rounded down to FP32 (bits)
+  if (PRUNE) {
+    if (threadIdx.x == 0) sc = sv = 0;
+    __syncthreads();
+  }
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < (int64_t)E * n3;
        x += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = x / n3;
@@ -39,7 +94,17 @@ __global__ void __launch_bounds__(256) k_cfl(int E, const double* __restrict__ U
       const double* Gm = geo + e * 4 * n3 + t;
 #pragma unroll
       for (int k = 0; k < 4; ++k) G[k] = Gm[k * n3];
+      if constexpr (PRUNE) {
+        float ua, ub;
+        radii_up(Uv, M, G, (float)gamma, (float)gm1, (float)Rinv, (float)kv, sutherland, (float)inv_Tref, ua, ub);
+        const float ca = __int_as_float(*(volatile int*)&sc), cb = __int_as_float(*(volatile int*)&sv);
+        if (ua < ca && (!viscous || ub < cb)) continue;
+      }
       cfl_radii(Uv, M, G, gamma, gm1, Rinv, kv, sutherland, inv_Tref, aa, bb);
+      if (PRUNE) {
+        if (aa > lcT) atomicMax(&sc, __float_as_int(__double2float_rd(aa)));
+        if (bb > lvT) atomicMax(&sv, __float_as_int(__double2float_rd(bb)));
+      }
     }
     if (!isfinite(aa) || !isfinite(bb)) bad = 1;
     lcT = fmax(lcT, aa);
@@ -409,22 +474,36 @@ cudaError_t launch_refs(dg_ctx* c) {
   return cudaGetLastError();
 }
 
-static int cfl_blocks(dg_ctx* c) {
+static int sm_count_of(const dg_ctx* c) {
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  return sms;
+}
+static int cfl_blocks(dg_ctx* c) {
   const int64_t need = (c->E * c->n3 + 255) / 256;
-  return (int)std::min<int64_t>(need, (int64_t)sms * 8);
+  return (int)std::min<int64_t>(need, (int64_t)sm_count_of(c) * 8);
 }
 
 cudaError_t launch_cfl(dg_ctx* c, bool report_only) {
   const double kv = std::max(4.0 / 3.0, c->prm.gamma / c->prm.Pr) * c->prm.mu;
   const int nb = cfl_blocks(c);
+  // FP64: two blocks per SM and PRUNE where a thread then meets two nodes or
+  // more, so that the block's maximum spares it most of them (24^3 elements,
+  // N = 7: one / two / eight blocks per SM 330 / 219 / 262 us; 12^3: 72 / 63 /
+  // 95).  Below that the bounds cost more than they spare (9 x 7 x 5, N = 6:
+  // 24 us without, 27 with).
+  const int nb2 = 2 * sm_count_of(c);
   prof_begin(c, PK_CFL);
   if (c->prm.precision == DG_FP32_BULK) {
     DG_DISPATCH(c->N, (k_cfl<NN, float><<<nb, 256, 0, c->stream>>>((int)c->E, c->U, c->metric, c->metric32, c->cflgeo,
                                                                  c->prm.gamma, c->prm.gamma - 1.0, 1.0 / c->prm.R, kv,
                                                                  c->prm.viscous, c->prm.sutherland,
                                                                  1.0 / c->prm.T_ref, c->scal)));
+  } else if (c->E * c->n3 > 2 * 256 * (int64_t)nb2) {
+    DG_DISPATCH(c->N, (k_cfl<NN, double, true><<<nb2, 256, 0, c->stream>>>((int)c->E, c->U, c->metric, c->metric32,
+                                                                        c->cflgeo, c->prm.gamma, c->prm.gamma - 1.0,
+                                                                        1.0 / c->prm.R, kv, c->prm.viscous,
+                                                                        c->prm.sutherland, 1.0 / c->prm.T_ref, c->scal)));
   } else {
     DG_DISPATCH(c->N, (k_cfl<NN, double><<<nb, 256, 0, c->stream>>>((int)c->E, c->U, c->metric, c->metric32,
                                                                   c->cflgeo, c->prm.gamma, c->prm.gamma - 1.0,
