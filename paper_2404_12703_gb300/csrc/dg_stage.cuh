@@ -616,9 +616,11 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
 // ---------------------------------------------------------------------------
 // FillFlux: Riemann flux + BR1 viscous flux, times the surface element
 // ---------------------------------------------------------------------------
-// GL: states and lifted gradients from the ProlongToFace arrays
+// GL: states and lifted gradients from the ProlongToFace arrays.  FP32 waits
+// on its gathers: 64 registers for four blocks of 256 per SM (it took 76 and
+// three; a few values spill) 29.0 -> 27.1 us on the 16 x 8 x 16 channel, N = 7.
 template <int N, typename T, bool GL = false>
-__global__ void __launch_bounds__(256) k_surf_flux(StageArgs a) {
+__global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_surf_flux(StageArgs a) {
   using S = Shape<N>;
   constexpr int n = S::n, n2 = S::n2, n3 = S::n3;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
