@@ -309,7 +309,7 @@ __device__ __forceinline__ void lf_flux_s(const SPrim<T>& L, const SPrim<T>& R, 
 // square from one reciprocal square root, the upwind terms collected by
 // direction, the stresses contracted with the normal before the work term,
 // and one scaling by s / 2.  k_surf_flux on 24^3 elements, N = 7: 1,373 -> 1,048
-// us per launch.
+// us per launch, 952 with 1 / rho and p from k_surf_prims.
 // ---------------------------------------------------------------------------
 // ConsToPrim in FP64 (the FP64 path's references are zero)
 struct Prim64 {
@@ -322,6 +322,10 @@ __device__ __forceinline__ Prim64 prim64(const double U[5], double gm1) {
   q.u = U[1] * q.ri, q.v = U[2] * q.ri, q.w = U[3] * q.ri;
   q.p = gm1 * (U[4] - 0.5 * (U[1] * q.u + U[2] * q.v + U[3] * q.w));
   return q;
+}
+// the same from 1 / rho and p as k_surf_prims left them
+__device__ __forceinline__ Prim64 prim64(const double U[5], double ri, double p) {
+  return {U[0], U[1] * ri, U[2] * ri, U[3] * ri, p, ri};
 }
 // twice Roe's flux through the unit normal n (no entropy fix)
 __device__ __forceinline__ void roe_flux64(const Prim64& L, const Prim64& R, double HL, double HR, const double n[3],
@@ -506,6 +510,33 @@ __global__ void __launch_bounds__(256) k_surf_prims(StageArgs a) {
   constexpr int ust = GL ? n2 : n3;
 #pragma unroll
   for (int k = 0; k < 5; ++k) UM[k] = uM[k * ust];
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (brow < 0) {  // inner side
+      int ps, qs;
+      flip_to_slave<n>(flip, p, q, ps, qs);
+      const int vS = face_vol_node<n>(fS, ps, qs);
+      double US[5];
+      const double* uS = GL ? a.Ufc + (size_t)s * 10 * n2 + 5 * n2 + pq : a.U + (size_t)ee.y * 5 * n3 + vS;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) US[k] = uS[k * ust];
+      const Prim64 L = prim64(UM, a.gm1), R = prim64(US, a.gm1);
+      const double qa[4] = {L.u + R.u, L.v + R.v, L.w + R.w,
+                            __dmul_rn(L.p * L.ri, a.Rinv) + __dmul_rn(R.p * R.ri, a.Rinv)};
+      double* out = a.lflux + (size_t)s * 12 * n2 + pq;
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        const double h = 0.5 * sn[x];
+#pragma unroll
+        for (int qv = 0; qv < 4; ++qv) out[(qv * 3 + x) * n2] = qa[qv] * h;
+      }
+      // for the same thread's side node in k_surf_flux, which overwrites them
+      // with the flux: two divisions and two pressures fewer there (24^3
+      // elements, N = 7: 1,047 -> 952 us, here 256 -> 253 us)
+      double* keep = a.fstar + (size_t)s * 5 * n2 + pq;
+      keep[0] = L.ri, keep[n2] = L.p, keep[2 * n2] = R.ri, keep[3 * n2] = R.p;
+      return;
+    }
+  }
   const SPrim<T> qM = shifted_prim<T, true>(UM, a.gm1, a.Rinv, cp);
   T qa[4];
   if (brow >= 0) {
@@ -619,7 +650,8 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS) k_lift(StageArgs a) {
 // GL: states and lifted gradients from the ProlongToFace arrays.  FP32 waits
 // on its gathers: 64 registers for four blocks of 256 per SM (it took 76 and
 // three; a few values spill) 29.0 -> 27.1 us on the 16 x 8 x 16 channel, N = 7.
-template <int N, typename T, bool GL = false>
+// VISC (FP64): a viscous run, in which k_surf_prims went before; FP32 asks a.viscous.
+template <int N, typename T, bool GL, bool VISC>
 __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_surf_flux(StageArgs a) {
   using S = Shape<N>;
   constexpr int n = S::n, n2 = S::n2, n3 = S::n3;
@@ -650,11 +682,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
       double UM[5], US[5], f[5];
 #pragma unroll
       for (int k = 0; k < 5; ++k) UM[k] = uM[k * ust], US[k] = uS[k * ust];
-      const Prim64 L = prim64(UM, a.gm1), R = prim64(US, a.gm1);
+      double* out = a.fstar + (size_t)s * 5 * n2 + pq;
+      const Prim64 L = VISC ? prim64(UM, out[0], out[n2]) : prim64(UM, a.gm1);
+      const Prim64 R = VISC ? prim64(US, out[2 * n2], out[3 * n2]) : prim64(US, a.gm1);
       const double HL = (UM[4] + L.p) * L.ri, HR = (US[4] + R.p) * R.ri;
       if (cp.riemann == DG_RIEMANN_ROE) roe_flux64(L, R, HL, HR, nu, a.gm1, f);
       else lf_flux64(L, R, HL, HR, UM, US, nu, a.gamma, f);
-      if (a.viscous) {
+      if constexpr (VISC) {
         double g[12];
         const double* pgM = GL ? a.gfc + (size_t)s * 24 * n2 + pq : a.g + (size_t)ee.x * 12 * n3 + vM;
         const double* pgS = GL ? a.gfc + (size_t)s * 24 * n2 + 12 * n2 + pq : a.g + (size_t)ee.y * 12 * n3 + vS;
@@ -665,7 +699,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
         for (int k = 0; k < 12; ++k) g[k] = pgS[k * ust];
         sub_viscous64(a, cp, R, g, nu, f);
       }
-      double* out = a.fstar + (size_t)s * 5 * n2 + pq;
       const double hs = 0.5 * sA;
 #pragma unroll
       for (int k = 0; k < 5; ++k) out[k * n2] = f[k] * hs;
@@ -697,7 +730,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
   T f[5];
   if (brow >= 0) {  // boundary side
     T gM[12];
-    if (a.viscous) {
+    if (VISC && a.viscous) {
       const T* pgM = GL ? Gf + (size_t)s * 24 * n2 + pq : G + (size_t)ee.x * 12 * n3 + vM;
 #pragma unroll
       for (int k = 0; k < 12; ++k) gM[k] = pgM[k * ust];
@@ -719,7 +752,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
     else lf_flux_s(qM, qS, nu, pick<T>(a.gamma, a.f_gamma), pick<T>(cp.pr, cp.fpr), f);
 #pragma unroll
     for (int k = 0; k < 5; ++k) f[k] *= sA;
-    if (a.viscous) {
+    if (VISC && a.viscous) {
       T gM[12], gS[12];
       const T* pgM = GL ? Gf + (size_t)s * 24 * n2 + pq : G + (size_t)ee.x * 12 * n3 + vM;
       const T* pgS = GL ? Gf + (size_t)s * 24 * n2 + 12 * n2 + pq : G + (size_t)ee.y * 12 * n3 + vS;
@@ -1363,7 +1396,8 @@ inline void launch_side(const StageArgs& a, int block, cudaStream_t st, bool pri
   const int b = side_threads(block, side_nodes);
   const unsigned g = (unsigned)((side_nodes + b - 1) / b);
   if (prims) k_surf_prims<N, T, GL><<<g, b, 0, st>>>(a);
-  else k_surf_flux<N, T, GL><<<g, b, 0, st>>>(a);
+  else if (sizeof(T) == sizeof(float) || a.viscous) k_surf_flux<N, T, GL, true><<<g, b, 0, st>>>(a);
+  else k_surf_flux<N, T, GL, sizeof(T) == sizeof(float)><<<g, b, 0, st>>>(a);
 }
 
 template <int N, typename T>
