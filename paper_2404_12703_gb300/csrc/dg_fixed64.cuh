@@ -9,9 +9,9 @@
 // FP64 multiplication, and with more bits.  The kernels here were bound by
 // the FP64 unit (84 - 96 % busy); what they keep on it is ConsToPrim, the
 // stress tensor and the Runge-Kutta update.  Measured per launch on 24^3
-// elements, N = 7 (7.08 M nodes): volume kernel 7.70 -> 2.89 ms, lifting
-// 4.12 -> 1.45 ms; now bound by latency at two blocks per SM (issue 44 % busy,
-// FP64 unit 42 %).
+// elements, N = 7 (7.08 M nodes): volume kernel 7.70 -> 2.46 ms, lifting
+// 4.12 -> 1.39 ms; now bound by latency at two blocks per SM (issue 45 - 49 %
+// busy, FP64 unit 30 - 41 %).
 //
 // Numbers.  Every element scales each group of quantities (density, velocity,
 // pressure, enthalpy, metrics, ...) by the power of two that brings the
@@ -23,7 +23,8 @@
 // the element alone, so results do not depend on the launch shape.
 // The bounds on every intermediate value stand beside it; none can overflow.
 // Error against the long-double oracle, N = 1 .. 7, Ma 0.1 - 1.25, viscous,
-// Roe and LF: 0.72 of the FP64 kernels' in the mean, at most 1.001.
+// Roe and LF: 0.67 of the FP64 kernels' in the mean, at most 1.12 (N = 1, where
+// both are near 1e-13).
 // An element with a non-finite value, or with a group whose largest value is
 // outside 2^-200 .. 2^200, is done in FP64 in the same kernels, with FP64's
 // own treatment of such values.

@@ -3,7 +3,7 @@
 // (see dg_fixed64.cuh for the numbers and why; the work is that of
 // k_lift_gl and k_volume_gl in dg_stage_gl.cuh, which FP32-bulk uses).
 // Measured per launch on 12^3 elements, N = 7 (0.88 M nodes): lifting
-// 864 -> 325 us, volume kernel 549 -> 269 us; error against the long-double
+// 864 -> 328 us, volume kernel 549 -> 265 us; error against the long-double
 // oracle 0.86 of the FP64 kernels' in the mean (N = 1 .. 7, Ma 0.1 - 1.25).
 #pragma once
 
