@@ -507,7 +507,10 @@ struct VolScale {
 };
 enum { VQ_RHO, VQ_U, VQ_V, VQ_W, VQ_P, VQ_H, VQ_RHOH, VQ_MOM, VQ_J, VQ_N = VQ_J + 9 };
 
-// threads 0 .. 2 of the element, one direction each; Q = maxima
+// Threads 0 .. 2 of the element form the shifts of one direction each
+// (vol_scale) and then align the directions' sums (vol_align), which reads the
+// other two threads' scales: the caller synchronises the whole warp between
+// the two, outside the branch on the thread (at N = 1 it holds four elements).
 __device__ __forceinline__ void vol_scale(VolScale& s, const unsigned* m, const Ops* o, int t) {
   const int eR = fx_exp(m[VQ_RHO]), eU = fx_exp(max(max(m[VQ_U], m[VQ_V]), m[VQ_W])), eP = fx_exp(m[VQ_P]),
             eH = fx_exp(m[VQ_H]);
@@ -546,14 +549,8 @@ __device__ __forceinline__ void vol_scale(VolScale& s, const unsigned* m, const 
   s.c[t][0] = a3 + 3 + w;
   s.c[t][1] = b3 - kp - eJ - 2 + d.s5 + w;
   s.c[t][2] = a3 - eH + 1 + d.s6 + w;
-  __syncwarp(__activemask());
-  int p[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) p[k] = min(min(s.c[0][k], s.c[1][k]), s.c[2][k]);
-  d.aM = min(s.c[t][0] - p[0], 63), d.aV = min(s.c[t][1] - p[1], 63), d.aE = min(s.c[t][2] - p[2], 63);
   if (t == 0) {
     s.eR = eR, s.eU = eU, s.eP = eP, s.eH = eH;
-    s.pM = p[0], s.pV = p[1], s.pE = p[2];
     // In FP64: groups out of range, and elements whose largest fluxes lie far
     // below the product of their groups' maxima (light and fast or hot fluid
     // beside dense fluid, ratios above four): their scale would leave the
@@ -566,6 +563,14 @@ __device__ __forceinline__ void vol_scale(VolScale& s, const unsigned* m, const 
     bad = bad || fR * fmaxf(u0, fmaxf(u1, u2)) * ldexpf(1.0f, lm) > 4.0f * fx_frac(m[VQ_MOM], eM);
     s.bad = bad;
   }
+}
+__device__ __forceinline__ void vol_align(VolScale& s, int t) {
+  int p[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) p[k] = min(min(s.c[0][k], s.c[1][k]), s.c[2][k]);
+  DirScale& d = s.d[t];
+  d.aM = min(s.c[t][0] - p[0], 63), d.aV = min(s.c[t][1] - p[1], 63), d.aE = min(s.c[t][2] - p[2], 63);
+  if (t == 0) s.pM = p[0], s.pV = p[1], s.pE = p[2];
 }
 
 // shared memory: S = w Dsplit, 1/w and Dhat split (Fx), Vinv, the reduction
@@ -778,6 +783,8 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     }
     fx_reduce<N, VQ_N>(m, red, fin, t);
     if (t < 3) vol_scale(*sc, fin, a.ops, t);
+    __syncwarp();
+    if (t < 3) vol_align(*sc, t);
     __syncwarp();
     __syncthreads();
   }
