@@ -327,7 +327,11 @@ __device__ __forceinline__ Prim64 prim64(const double U[5], double gm1) {
 __device__ __forceinline__ Prim64 prim64(const double U[5], double ri, double p) {
   return {U[0], U[1] * ri, U[2] * ri, U[3] * ri, p, ri};
 }
-// twice Roe's flux through the unit normal n (no entropy fix)
+// Both fluxes below are twice the flux without the pressure in the momentum:
+// that and the viscous flux come after them, the large terms last, so that
+// the sum is rounded at their size as seldom as may be (momentum error 0.95 of
+// the textbook form's in FP64; pressures first and one average 1.3).
+// Roe's flux through the unit normal n (no entropy fix)
 __device__ __forceinline__ void roe_flux64(const Prim64& L, const Prim64& R, double HL, double HR, const double n[3],
                                            double gm1, double f[5]) {
   const double z = sqrt(R.rho * L.ri), inv = 1.0 / (1.0 + z);
@@ -344,37 +348,35 @@ __device__ __forceinline__ void roe_flux64(const Prim64& L, const Prim64& R, dou
   const double S = w1 + w5, A = S + w2, B = (w5 - w1) * c - w3 * dun;
   const double mL = L.rho * (L.u * n[0] + L.v * n[1] + L.w * n[2]);
   const double mR = R.rho * (R.u * n[0] + R.v * n[1] + R.w * n[2]);
-  const double P = (L.p + R.p) - B;
-  f[0] = mL + mR - A;
-  f[1] = mL * L.u + mR * R.u + P * n[0] - A * u - w3 * du;
-  f[2] = mL * L.v + mR * R.v + P * n[1] - A * v - w3 * dv;
-  f[3] = mL * L.w + mR * R.w + P * n[2] - A * w - w3 * dw;
-  f[4] = mL * HL + mR * HR - S * H - w2 * hq - un * B - w3 * (u * du + v * dv + w * dw);
+  f[0] = mL + (mR - A);
+  f[1] = mL * L.u + (mR * R.u - (B * n[0] + (A * u + w3 * du)));
+  f[2] = mL * L.v + (mR * R.v - (B * n[1] + (A * v + w3 * dv)));
+  f[3] = mL * L.w + (mR * R.w - (B * n[2] + (A * w + w3 * dw)));
+  f[4] = mL * HL + (mR * HR - (S * H + (w2 * hq + (un * B + w3 * (u * du + v * dv + w * dw)))));
 }
-// twice the local Lax-Friedrichs flux
+// the local Lax-Friedrichs flux
 __device__ __forceinline__ void lf_flux64(const Prim64& L, const Prim64& R, double HL, double HR, const double UL[5],
                                           const double UR[5], const double n[3], double gamma, double f[5]) {
   const double uL = L.u * n[0] + L.v * n[1] + L.w * n[2], uR = R.u * n[0] + R.v * n[1] + R.w * n[2];
   const double lL = fabs(uL) + sqrt(gamma * L.p * L.ri), lR = fabs(uR) + sqrt(gamma * R.p * R.ri);
-  const double lm = lL > lR ? lL : lR, mL = L.rho * uL, mR = R.rho * uR, P = L.p + R.p;
-  f[0] = mL + mR - lm * (UR[0] - UL[0]);
-  f[1] = mL * L.u + mR * R.u + P * n[0] - lm * (UR[1] - UL[1]);
-  f[2] = mL * L.v + mR * R.v + P * n[1] - lm * (UR[2] - UL[2]);
-  f[3] = mL * L.w + mR * R.w + P * n[2] - lm * (UR[3] - UL[3]);
-  f[4] = mL * HL + mR * HR - lm * (UR[4] - UL[4]);
+  const double lm = lL > lR ? lL : lR, mL = L.rho * uL, mR = R.rho * uR;
+  f[0] = mL + (mR - lm * (UR[0] - UL[0]));
+  f[1] = mL * L.u + (mR * R.u - lm * (UR[1] - UL[1]));
+  f[2] = mL * L.v + (mR * R.v - lm * (UR[2] - UL[2]));
+  f[3] = mL * L.w + (mR * R.w - lm * (UR[3] - UL[3]));
+  f[4] = mL * HL + (mR * HR - lm * (UR[4] - UL[4]));
 }
-// f[1..4] -= F_v(q, g) . n
-__device__ __forceinline__ void sub_viscous64(const StageArgs& a, const CaseParams& cp, const Prim64& q,
-                                              const double g[12], const double n[3], double f[5]) {
+// F_v(q, g) . n, momentum and energy
+__device__ __forceinline__ void viscous_flux64(const StageArgs& a, const CaseParams& cp, const Prim64& q,
+                                               const double g[12], const double n[3], double v[4]) {
   double mu, lam;
   visc_coeffs<double>(a, cp, a.sutherland ? q.p * q.ri * a.Rinv : 0.0, mu, lam);
   const double tw = (2.0 / 3.0) * (g[0] + g[4] + g[8]);
   const double xy = g[1] + g[3], xz = g[2] + g[6], yz = g[5] + g[7];
-  const double fx = mu * ((2.0 * g[0] - tw) * n[0] + xy * n[1] + xz * n[2]);
-  const double fy = mu * (xy * n[0] + (2.0 * g[4] - tw) * n[1] + yz * n[2]);
-  const double fz = mu * (xz * n[0] + yz * n[1] + (2.0 * g[8] - tw) * n[2]);
-  f[1] -= fx, f[2] -= fy, f[3] -= fz;
-  f[4] -= q.u * fx + q.v * fy + q.w * fz + lam * (g[9] * n[0] + g[10] * n[1] + g[11] * n[2]);
+  v[0] = mu * ((2.0 * g[0] - tw) * n[0] + xy * n[1] + xz * n[2]);
+  v[1] = mu * (xy * n[0] + (2.0 * g[4] - tw) * n[1] + yz * n[2]);
+  v[2] = mu * (xz * n[0] + yz * n[1] + (2.0 * g[8] - tw) * n[2]);
+  v[3] = q.u * v[0] + q.v * v[1] + q.w * v[2] + lam * (g[9] * n[0] + g[10] * n[1] + g[11] * n[2]);
 }
 
 // ---------------------------------------------------------------------------
@@ -673,7 +675,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
     if (brow < 0) {  // inner side
       const double* nr = a.nrm + (size_t)s * 4 * n2 + pq;
       const double sA = nr[3 * n2], invd = 1.0 / sA;
-      const double nu[3] = {nr[0] * invd, nr[n2] * invd, nr[2 * n2] * invd};
+      const double sn[3] = {nr[0], nr[n2], nr[2 * n2]}, nu[3] = {sn[0] * invd, sn[1] * invd, sn[2] * invd};
       int ps, qs;
       flip_to_slave<n>(flip, p, q, ps, qs);
       const int vM = face_vol_node<n>(fM, p, q), vS = face_vol_node<n>(fS, ps, qs);
@@ -689,19 +691,26 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
       if (cp.riemann == DG_RIEMANN_ROE) roe_flux64(L, R, HL, HR, nu, a.gm1, f);
       else lf_flux64(L, R, HL, HR, UM, US, nu, a.gamma, f);
       if constexpr (VISC) {
-        double g[12];
+        double g[12], vL[4], vR[4];
         const double* pgM = GL ? a.gfc + (size_t)s * 24 * n2 + pq : a.g + (size_t)ee.x * 12 * n3 + vM;
         const double* pgS = GL ? a.gfc + (size_t)s * 24 * n2 + 12 * n2 + pq : a.g + (size_t)ee.y * 12 * n3 + vS;
 #pragma unroll
         for (int k = 0; k < 12; ++k) g[k] = pgM[k * ust];
-        sub_viscous64(a, cp, L, g, nu, f);
+        viscous_flux64(a, cp, L, g, nu, vL);
 #pragma unroll
         for (int k = 0; k < 12; ++k) g[k] = pgS[k * ust];
-        sub_viscous64(a, cp, R, g, nu, f);
+        viscous_flux64(a, cp, R, g, nu, vR);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) f[1 + k] -= vL[k] + vR[k];
       }
       const double hs = 0.5 * sA;
+      out[0] = f[0] * hs;
 #pragma unroll
-      for (int k = 0; k < 5; ++k) out[k * n2] = f[k] * hs;
+      for (int k = 0; k < 3; ++k) {
+        const double h = 0.5 * sn[k];
+        out[(1 + k) * n2] = L.p * h + (R.p * h + f[1 + k] * hs);
+      }
+      out[4 * n2] = f[4] * hs;
       return;
     }
   }
