@@ -6,28 +6,40 @@
 // 32 x 32 -> 64 bits with a 64-bit addition (mad.wide), 59 additions of 64-bit
 // integers (measured).  A product of two 62-bit fixed-point numbers, rounded
 // to 64 bits, is three mad.wide and a shift: eight times cheaper than one
-// FP64 multiplication, and with more bits.  The kernels here were bound by
-// the FP64 unit (84 - 96 % busy); what they keep on it is ConsToPrim, the
-// stress tensor and the Runge-Kutta update.  Measured per launch on 24^3
-// elements, N = 7 (7.08 M nodes): volume kernel 7.70 -> 2.46 ms, lifting
-// 4.12 -> 1.39 ms; now bound by latency at two blocks per SM (issue 45 - 49 %
-// busy, FP64 unit 30 - 41 %).
+// FP64 multiplication.  The kernels here were bound by the FP64 unit (84 - 96 %
+// busy); what they keep on it is ConsToPrim, the stress tensor and the
+// Runge-Kutta update.  Measured per launch on 24^3 elements, N = 7 (7.08 M
+// nodes): volume kernel 7.70 -> 2.57 ms, lifting 4.12 -> 1.42 ms; now bound by
+// latency at two blocks per SM.
 //
 // Numbers.  Every element scales each group of quantities (density, velocity,
-// pressure, enthalpy, metrics, ...) by the power of two that brings the
-// group's largest magnitude in the element below 2^60 or 2^61; a value is
-// that many bits of a two's complement 64-bit integer.  The error of a
-// conversion is below one unit, 2^-60 of the largest value, where FP64 rounds
-// each value to 2^-53 of itself; products keep 64 bits and are rounded, sums
-// are exact.  Results are rounded to FP64 once, at the end.  Scales depend on
-// the element alone, so results do not depend on the launch shape.
-// The bounds on every intermediate value stand beside it; none can overflow.
-// Error against the long-double oracle, N = 1 .. 7, Ma 0.1 - 1.25, viscous,
-// Roe and LF: 0.67 of the FP64 kernels' in the mean, at most 1.12 (N = 1, where
-// both are near 1e-13).
-// An element with a non-finite value, or with a group whose largest value is
-// outside 2^-200 .. 2^200, is done in FP64 in the same kernels, with FP64's
-// own treatment of such values.
+// pressure, enthalpy, metrics by Cartesian component, ...) by the power of two
+// that brings the group's largest magnitude in the element below 2^60 or 2^61;
+// a value is that many bits of a two's complement 64-bit integer.  A conversion
+// is off by less than one unit: 2^-59 of the group's largest value (2^-60 of
+// density, pressure, enthalpy and the lifted variables, 2^-57 of the heat flux
+// beside a large work term), where FP64 rounds each value to 2^-53 of itself.
+// Products keep 64 bits, sums are exact, results are rounded to FP64 once.
+// The largest values of a group so have more bits than FP64 gives them and
+// those below a sixty-fourth fewer.  What that may cost, and what is done:
+// - Different velocity components, metrics and stresses: groups or scalings by
+//   component (lifting, vol_scale, the rows of dg_fixed64_gl.cuh), so that a
+//   small cross-flow or a stretched element keeps its bits.
+// - Density, pressure, energy or temperature that span more than a factor of
+//   16 in an element: FP64 rounds a node's sums at the size of the largest
+//   values on the node's three lines.  Where they miss the element's large
+//   values (lines_quiet), the element is done in FP64.
+// - Light and fast or hot fluid beside dense fluid, small components beside
+//   hypersonic flow (vol_bad), stresses above the pressure: in FP64 too.
+// - A non-finite value, or a group whose largest value is outside 2^-200 ..
+//   2^200: in FP64, with its own treatment of such values.
+// FP64 sums cost what they did before (an all-FP64 step takes 0.76 - 1.0 of
+// the time it took with every element so, N = 1 .. 7).
+// Scales depend on the element alone, so results do not depend on the launch
+// shape.  The bounds on every intermediate value stand beside it; none can
+// overflow.  Error of the right-hand side against the long-double oracle over
+// that of the FP64 kernels, N = 1 .. 7, Ma 0.1 - 1.25, viscous, Roe and LF: 0.53
+// in the geometric mean, at most 0.999 in any variable (Gauss nodes 0.79, 0.999).
 #pragma once
 
 namespace dg {
@@ -43,7 +55,8 @@ __device__ __forceinline__ Fx fx_split(long long x) {
 // Sum of products a b 2^-64: h in units of 1, x in units of 2^-32 (the
 // products of the low words, below half a unit each, are left out).  get: the
 // sum times 2^S.  FxSum<S> rounds (x starts at half a unit of the result);
-// FxSumS takes S at run time and truncates.
+// FxSumS takes S at run time and truncates (the two nodes of a pair take the
+// same truncated flux, so that nothing is gained or lost).
 __device__ __forceinline__ long long fx_get(long long h, long long x, int S) {
   return (long long)((unsigned long long)h << S) + (x >> (32 - S));
 }
@@ -66,6 +79,8 @@ struct FxSumS {
   }
   __device__ __forceinline__ long long get(int S) const { return fx_get(h, x, S); }
 };
+// v 2^-k, rounded (k = 0 .. 62, |v| below 2^62)
+__device__ __forceinline__ long long fx_shr(long long v, int k) { return (v + (long long)((1ull << k) >> 1)) >> k; }
 
 // Biased FP64 exponent of the largest magnitude from the maximum of the high words
 __device__ __forceinline__ unsigned fx_field(unsigned hi_max) { return hi_max >> 20; }
@@ -170,10 +185,53 @@ __device__ __forceinline__ float fx_frac(unsigned hi, int e) {
   const int x = (int)fx_field(hi) - 1022 - e;
   return hi == 0u || x < -100 ? 0.0f : __uint_as_float(((unsigned)(126 + x) << 23) | ((hi & 0xfffffu) << 3)) * 1.00001f;
 }
+// b 2^k, b >= 0, from above (k clamped to +-126)
+__device__ __forceinline__ float fx_scale(float b, int k) { return b * __uint_as_float((unsigned)(127 + max(-126, min(126, k))) << 23); }
 // the largest S in 0 .. 31 with b 2^S <= 2^top
 __device__ __forceinline__ int fx_room(float b, int top) {
   const int l = (int)((__float_as_uint(b) + 0x7fffffu) >> 23) - 127;  // b <= 2^l
   return max(0, min(31, top - l));
+}
+
+// A magnitude's high word scaled by 2^-k (zero where it vanishes), the cut
+// below which a value of a group is quiet (a sixteenth of the largest), and
+// whether a node's three lines hold quiet values only.  Fixed point keeps a
+// quiet value's bits below FP64's; where a line through the node holds a
+// larger value, FP64 rounds the node's sums at that value's size anyway.
+__device__ __forceinline__ unsigned fx_down(unsigned mag, int k) {
+  return mag > (unsigned)k << 20 ? mag - ((unsigned)k << 20) : 0u;
+}
+__device__ __forceinline__ unsigned fx_cut(unsigned hi_max) { return fx_down(hi_max, 4); }
+template <int n, class Mag>
+__device__ __forceinline__ bool lines_quiet(int v, unsigned cut, Mag mag) {
+  for (int d = 0; d < 3; ++d) {
+    const int sd = dir_stride<n>(d), base = v - dir_index<n>(v, d) * sd;
+    for (int al = 0; al < n; ++al)
+      if (mag(base + al * sd) >= cut) return false;
+  }
+  return true;
+}
+// Which sums an element and its block take: direct (FP64), and whether any or
+// all elements of the block do
+struct SumForm {
+  bool direct, any, all;
+};
+// For a block that holds an element whose sums are taken in FP64 in any case
+// (bad) or that has a node with a quiet value (the groups' minima tell).
+// quiet(v): whether node v is quiet in a group on all its lines; flag: a word
+// of the element's shared memory, zero when called.
+template <int N, class Quiet>
+__device__ __noinline__ SumForm sum_form(bool bad, int t, unsigned* flag, Quiet quiet) {
+  constexpr int n3 = Fix<N>::n3, TPE = Fix<N>::TPE;
+  bool is = false;
+  if (!bad)
+    for (int v = t; v < n3; v += TPE) is = is || quiet(v);
+  if (is) *flag = 1u;
+  __syncwarp();
+  __syncthreads();
+  const bool direct = bad || *flag != 0u;
+  const bool any = __syncthreads_or(direct), all = __syncthreads_and(direct);
+  return {direct, any, all};
 }
 
 template <int n>
@@ -284,22 +342,19 @@ __device__ __forceinline__ void finish_node64(const StageArgs& a, int e, int ce,
 // ---------------------------------------------------------------------------
 // Lifted gradients (Eq. lifting)
 // ---------------------------------------------------------------------------
-// shared memory: the tables, the reduction words, then per element the q
-// planes (4), two buffers of one direction's metric planes (2 x 3) and the
-// sums (12), all padded node planes
+// shared memory: the tables (fixed point and FP64), the reduction words, then
+// per element the q planes (4), two buffers of one direction's metric planes
+// (2 x 3) and the sums (12), all padded node planes
 template <int N>
 struct LiftFix {
   using F = Fix<N>;
   static constexpr int h = F::n / 2;
   static constexpr int ntab = F::n % 2 == 0 ? 2 * h * h : F::n2;  // split table entries
   static constexpr int planes = 22;
-  static constexpr int Q = 5, nred = F::W * Q + Q;  // maxima: velocity, temperature, metrics by Cartesian component
-  static constexpr size_t head(int epb) { return (8 * ntab + 4 * (size_t)epb * nred + 15) & ~size_t(15); }
+  static constexpr int Q = 8, nred = F::W * Q + Q + 1;  // maxima: u, v, w, T, metrics by Cartesian component, ~T; flag
+  static constexpr size_t head(int epb) { return (16 * ntab + 4 * (size_t)epb * nred + 15) & ~size_t(15); }
   static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * planes * F::Pn; }
 };
-
-template <int n>
-__device__ void lift_direct(const StageArgs& a, int e, int v, double acc[12]);
 
 // Dhat split in shared memory: for even n its even and odd halves
 template <int N>
@@ -310,14 +365,15 @@ __device__ __forceinline__ void lift_table_fx(const Ops* o, Fx* sD) {
     sD[k] = Fix<N>::n % 2 == 0 ? fx_split(k < h * h ? o->fxHe[k] : o->fxHo[k - h * h]) : fx_split(o->fxH[k]);
 }
 // (u, v, w, T) of the element's nodes, in FP64, to the q planes, and the
-// maxima of velocity, temperature and the metrics by Cartesian component
+// maxima of their magnitudes, of the metrics by Cartesian component and of T's
+// complement (its minimum)
 template <int N>
-__device__ __forceinline__ void lift_prims_fx(const StageArgs& a, int e, long long* q, unsigned m[5], int t) {
+__device__ __forceinline__ void lift_prims_fx(const StageArgs& a, int e, long long* q, unsigned m[8], int t) {
   using F = Fix<N>;
   constexpr int n = F::n, n3 = F::n3, Pn = F::Pn;
   const double* Me = a.metric + (size_t)e * 10 * n3;
 #pragma unroll
-  for (int k = 0; k < 5; ++k) m[k] = 0;
+  for (int k = 0; k < 8; ++k) m[k] = 0;
   for (int v = t; v < n3; v += F::TPE) {
     double U[5];
     load_state64<n>(a, e, v, U);
@@ -325,30 +381,45 @@ __device__ __forceinline__ void lift_prims_fx(const StageArgs& a, int e, long lo
     const double T = pr.p * pr.ri * a.Rinv;
     double* qd = reinterpret_cast<double*>(q) + fx_pad<n>(v);
     qd[0] = pr.u, qd[Pn] = pr.v, qd[2 * Pn] = pr.w, qd[3 * Pn] = T;
-    m[0] = max(max(m[0], fx_mag(pr.u)), max(fx_mag(pr.v), fx_mag(pr.w)));
-    m[1] = max(m[1], fx_mag(T));
+    m[0] = max(m[0], fx_mag(pr.u)), m[1] = max(m[1], fx_mag(pr.v)), m[2] = max(m[2], fx_mag(pr.w));
+    m[3] = max(m[3], fx_mag(T)), m[7] = max(m[7], ~fx_mag(T));
 #pragma unroll
-    for (int c = 0; c < 9; ++c) m[2 + c % 3] = max(m[2 + c % 3], fx_mag(Me[c * n3 + v]));
+    for (int c = 0; c < 9; ++c) m[4 + c % 3] = max(m[4 + c % 3], fx_mag(Me[c * n3 + v]));
   }
+}
+// the temperature falls into quiet on a node's lines (sum_form); the velocity
+// needs no such test: an error of 2^-60 of the element's largest gradient of a
+// component is below FP64's rounding of the pressure in the momentum's sums
+template <int N>
+__device__ __forceinline__ SumForm lift_form(bool bad, const long long* q, const unsigned* fin, int t, unsigned* flag) {
+  constexpr int n = Fix<N>::n;
+  const unsigned cut = fx_cut(fin[3]);
+  const bool ask = bad || ~fin[7] < cut;
+  if (!(blockDim.x == Fix<N>::TPE ? ask : __syncthreads_or(ask))) return {false, false, false};
+  const double* T = reinterpret_cast<const double*>(q + 3 * Fix<N>::Pn);
+  auto mag = [=](int v) { return fx_mag(T[fx_pad<n>(v)]); };
+  return sum_form<N>(bad, t, flag, [=](int v) { return mag(v) < cut && lines_quiet<n>(v, cut, mag); });
 }
 // The volume sums sum_d Dhat (Ja^d q) of the element in the W planes, from the
 // FP64 values in the q planes; a sum of variable k = 3 q + x has the scale
-// 2^(fxH_bits - 2 - e_q - eJ[x]) and is below 2^62
+// 2^(fxH_bits - 2 - eq[q] - eJ[x]) and is below 2^62.  skip: an element whose
+// sums are taken in FP64 (lift_sums_f64).
 template <int N>
 __device__ __forceinline__ void lift_sums_fx(const double* Me, long long* q, long long* J, long long* W, const Fx* sD,
-                                             int t, int eU, int eT, const int eJ[3]) {
+                                             int t, const int eq[4], const int eJ[3], bool skip) {
   using F = Fix<N>;
   using L = LiftFix<N>;
-  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn, h = L::h;
+  constexpr int n = F::n, n2 = F::n2, TPE = F::TPE, Pn = F::Pn, h = L::h;
+  const int n3 = skip ? 0 : F::n3, tasks = skip ? 0 : 4 * n2;
   for (int v = t; v < n3; v += TPE) {
     const int pv = fx_pad<n>(v);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       long long* x = q + k * Pn + pv;
-      *x = fx_from<61>(__longlong_as_double(*x), k < 3 ? eU : eT);
+      *x = fx_from<61>(__longlong_as_double(*x), eq[k]);
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) J[c * Pn + pv] = fx_from<60>(Me[c * n3 + v], eJ[c]);
+    for (int c = 0; c < 3; ++c) J[c * Pn + pv] = fx_from<60>(Me[c * F::n3 + v], eJ[c]);
   }
   __syncwarp();
   __syncthreads();
@@ -356,7 +427,7 @@ __device__ __forceinline__ void lift_sums_fx(const double* Me, long long* q, lon
   for (int d = 0; d < 3; ++d) {
     const int sd = dir_stride<n>(d);
     const long long* Jd = J + (d & 1) * 3 * Pn;
-    for (int task = t; task < 4 * n2; task += TPE) {
+    for (int task = t; task < tasks; task += TPE) {
       const int qv = task / n2, bl = line_base<n>(d, task % n2);
       Fx ql[n];
 #pragma unroll
@@ -408,7 +479,76 @@ __device__ __forceinline__ void lift_sums_fx(const double* Me, long long* q, lon
       long long* Jn = J + ((d + 1) & 1) * 3 * Pn;
       for (int v = t; v < n3; v += TPE)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Jn[c * Pn + fx_pad<n>(v)] = fx_from<60>(Me[(3 * d + 3 + c) * n3 + v], eJ[c]);
+        for (int c = 0; c < 3; ++c) Jn[c * Pn + fx_pad<n>(v)] = fx_from<60>(Me[(3 * d + 3 + c) * F::n3 + v], eJ[c]);
+    }
+    __syncwarp();
+    __syncthreads();
+  }
+}
+// the same in FP64, all planes holding FP64 values; sD: Dhat, for even n its
+// even and odd halves
+template <int N>
+__device__ __forceinline__ void lift_sums_f64(const Ops* o, const double* Me, const double* q, double* J, double* W,
+                                           double* sD, int t, bool skip) {
+  using F = Fix<N>;
+  using L = LiftFix<N>;
+  constexpr int n = F::n, n2 = F::n2, TPE = F::TPE, Pn = F::Pn, h = L::h;
+  const int n3 = skip ? 0 : F::n3, tasks = skip ? 0 : 4 * n2;
+  for (int k = threadIdx.x; k < L::ntab; k += blockDim.x) {
+    if constexpr (n % 2 == 0) {
+      const double* D = o->Dhat + (k % (h * h)) / h * n;
+      const int j = k % h;
+      sD[k] = 0.5 * (k < h * h ? D[j] + D[n - 1 - j] : D[j] - D[n - 1 - j]);
+    } else {
+      sD[k] = o->Dhat[k];
+    }
+  }
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    double* Jd = J + (d & 1) * 3 * Pn;
+    for (int v = t; v < n3; v += TPE)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) Jd[c * Pn + fx_pad<n>(v)] = Me[(3 * d + c) * F::n3 + v];
+    __syncwarp();
+    __syncthreads();
+    const int sd = dir_stride<n>(d);
+    for (int task = t; task < tasks; task += TPE) {
+      const int qv = task / n2, bl = line_base<n>(d, task % n2);
+#pragma unroll 1
+      for (int x = 0; x < 3; ++x) {
+        double P[n];
+#pragma unroll
+        for (int al = 0; al < n; ++al) {
+          const int pa = fx_pad<n>(bl + al * sd);
+          P[al] = Jd[x * Pn + pa] * q[qv * Pn + pa];
+        }
+        double* w = W + (qv * 3 + x) * Pn;
+        auto put = [&](int i, double y) {
+          double* out = w + fx_pad<n>(bl + i * sd);
+          *out = d == 0 ? y : *out + y;
+        };
+        if constexpr (n % 2 == 0) {
+#pragma unroll
+          for (int i = 0; i < h; ++i) {
+            double ye = 0.0, yo = 0.0;
+#pragma unroll
+            for (int j = 0; j < h; ++j) {
+              ye += sD[i * h + j] * (P[j] + P[n - 1 - j]);
+              yo += sD[h * h + i * h + j] * (P[j] - P[n - 1 - j]);
+            }
+            put(i, yo + ye);
+            put(n - 1 - i, yo - ye);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < n; ++i) {
+            double y = 0.0;
+#pragma unroll
+            for (int j = 0; j < n; ++j) y += sD[i * n + j] * P[j];
+            put(i, y);
+          }
+        }
+      }
     }
     __syncwarp();
     __syncthreads();
@@ -423,8 +563,10 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
   extern __shared__ __align__(16) unsigned char smraw[];
   const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
   Fx* sD = reinterpret_cast<Fx*>(smraw);
-  unsigned* red = reinterpret_cast<unsigned*>(smraw + 8 * L::ntab) + le * L::nred;
+  double* sDd = reinterpret_cast<double*>(sD + L::ntab);  // (filled by lift_sums_f64)
+  unsigned* red = reinterpret_cast<unsigned*>(smraw + 16 * L::ntab) + le * L::nred;
   unsigned* fin = red + F::W * L::Q;
+  unsigned* flag = fin + L::Q;
   long long* q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::planes * Pn;
   long long* J = q + 4 * Pn;   // [2][3][Pn]
   long long* W = J + 6 * Pn;   // [12][Pn]
@@ -435,31 +577,33 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
   lift_table_fx<N>(a.ops, sD);
   prefetch_sides64<N>(a, e, a.lflux, 12, t);
   prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
+  if (t == 0) *flag = 0u;
   {
-    unsigned m[5];
+    unsigned m[8];
     lift_prims_fx<N>(a, e, q, m, t);
-    fx_reduce<N, 5>(m, red, fin, t);
+    fx_reduce<N, 8>(m, red, fin, t);
     __syncthreads();
   }
   bool bad = false;
 #pragma unroll
-  for (int k = 0; k < 5; ++k) bad = bad || fx_bad(fin[k]);
-  const int eU = fx_exp(fin[0]), eT = fx_exp(fin[1]), eJ[3] = {fx_exp(fin[2]), fx_exp(fin[3]), fx_exp(fin[4])};
-  lift_sums_fx<N>(Me, q, J, W, sD, t, eU, eT, eJ);
+  for (int k = 0; k < 7; ++k) bad = bad || fx_bad(fin[k]);
+  const int eq[4] = {fx_exp(fin[0]), fx_exp(fin[1]), fx_exp(fin[2]), fx_exp(fin[3])};
+  const int eJ[3] = {fx_exp(fin[4]), fx_exp(fin[5]), fx_exp(fin[6])};
+  const SumForm form = lift_form<N>(bad, q, fin, t, flag);
+  if (!form.all) lift_sums_fx<N>(Me, q, J, W, sD, t, eq, eJ, form.direct);
+  if (form.any)
+    lift_sums_f64<N>(a.ops, Me, reinterpret_cast<const double*>(q), reinterpret_cast<double*>(J),
+                     reinterpret_cast<double*>(W), sDd, t, !form.direct);
   if (!er.valid) return;
-  const int pU = a.ops->fxH_bits - 2 - eU, pT = a.ops->fxH_bits - 2 - eT;
+  const int pH = a.ops->fxH_bits - 2;
   const double* Lf = a.lflux;
   for (int v = t; v < n3; v += TPE) {
     const int pv = fx_pad<n>(v);
     double acc[12];
-    if (bad) {
-      double d12[12];
-      lift_direct<n>(a, e, v, d12);
 #pragma unroll
-      for (int k = 0; k < 12; ++k) acc[k] = d12[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 12; ++k) acc[k] = fx_to(W[k * Pn + pv], (k < 9 ? pU : pT) - eJ[k % 3]);
+    for (int k = 0; k < 12; ++k) {
+      const long long w = W[k * Pn + pv];
+      acc[k] = form.direct ? __longlong_as_double(w) : fx_to(w, pH - eq[k / 3] - eJ[k % 3]);
     }
     // surface part: on LGL nodes only face nodes receive it
     const int idx[3] = {v % n, (v / n) % n, v / n2};
@@ -488,89 +632,169 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
 // ---------------------------------------------------------------------------
 // Volume integral + SurfInt + ApplyJac (+ RK update)
 // ---------------------------------------------------------------------------
-// Scales of an element's two-point sums, from its groups' maxima.  For each
+// Scales of an element's two-point sums, from its groups' maxima.  The metrics
+// have an exponent eJ for each Cartesian component (over the three directions)
+// and the velocity's component i is held as u_i 2^(eJ_i) under one exponent, so
+// that the products u_i m_i of a stretched element meet in one scale.  For each
 // direction the shifts bring every product's bound (from the actual maxima,
-// component by component) next to 2^62, so that no bits go to loose bounds
-// or to anisotropic metrics; the directions' sums are aligned at the end.
+// component by component) next to 2^62, so that no bits go to loose bounds;
+// the directions' sums are aligned at the end.
 struct DirScale {
-  int eJ;                      // exponent of the direction's metrics
-  int s1, s2, s3, s4, s5, s6;  // shifts of un, fr, t, pressure, momentum, energy (kep_fx)
-  int kc;                      // right shift of t in the momentum flux (aligns it with the pressure)
-  int aM, aV, aE;              // right shifts of the direction's mass, momentum and energy sums
+  int s1, s2, s3, s6;  // shifts of un, fr, t and energy (kep_flux_fx)
+  // by momentum component: shift of the pressure (below zero: a right shift),
+  // right shift of t (aligns it with the pressure), shift of the flux
+  int s4[3], kc[3], s5[3];
+  int aM, aV[3], aE;  // right shifts of the direction's mass, momentum and energy sums
 };
 struct VolScale {
   DirScale d[3];
-  int eR, eU, eP, eH;
-  int pM, pV, pE;  // results: sums times 2^-p
-  int c[3][3];     // the directions' own scales
-  int bad;
+  int eR, eP, eH, eU;  // eU: of the scaled velocity
+  int eJ[3];
+  int pM, pV[3], pE;   // results: sums times 2^-p
+  int c[3][5];         // the directions' own scales
+  unsigned bad, quiet, iso;
 };
-enum { VQ_RHO, VQ_U, VQ_V, VQ_W, VQ_P, VQ_H, VQ_RHOH, VQ_MOM, VQ_J, VQ_N = VQ_J + 9 };
+// maxima of magnitudes; VQ_LO: of the complements of density, pressure and rho H
+// (their minima)
+enum { VQ_RHO, VQ_U, VQ_V, VQ_W, VQ_P, VQ_H, VQ_RHOH, VQ_MOM, VQ_J, VQ_LO = VQ_J + 9, VQ_N = VQ_LO + 3 };
+
+// Whether the predicate holds in any thread of the element's first warp (of
+// the element, at N = 1), called by all of them
+template <int N>
+__device__ __forceinline__ bool fx_any(bool x, int t) {
+  if constexpr (Fix<N>::TPE >= 32) return __any_sync(0xffffffffu, x);
+  else return (__ballot_sync(0xffffffffu, x) >> ((threadIdx.x & 31) - t) & ((1u << Fix<N>::TPE) - 1u)) != 0u;
+}
+// a magnitude's logarithm to base two in units of 2^-20, at most 0.09 too small
+// (its high word: exponent and fraction)
+__device__ __forceinline__ int fx_log(unsigned mag) { return (int)mag - (1023 << 20); }
+
+// Whether the element's two-point sums are in FP64 in any case: groups out of
+// range, and elements whose largest fluxes lie far below the product of their
+// groups' maxima (light and fast or hot fluid beside dense fluid, ratios above
+// about four): their scale would leave the fluxes fewer bits than FP64 gives
+// them.  Likewise a small velocity component beside fast flow: the error of
+// t u_i is that of the largest component, below FP64's rounding of p m_i unless
+// the dynamic pressure exceeds the pressure by far.  Threads of the first warp.
+template <int N>
+__device__ __forceinline__ bool vol_bad(const unsigned* m, int t) {
+  bool bad = false;
+  for (int k = t; k < VQ_LO; k += Fix<N>::TPE < 32 ? Fix<N>::TPE : 32) bad = bad || fx_bad(m[k]);
+  const unsigned mu = max(max(m[VQ_U], m[VQ_V]), m[VQ_W]);
+  const int r = fx_log(m[VQ_RHO]);
+  if (t == 0) bad = bad || r + fx_log(m[VQ_H]) - fx_log(m[VQ_RHOH]) > 2 << 20;
+  if (t == 1) bad = bad || (mu != 0u && r + fx_log(mu) - fx_log(m[VQ_MOM]) > 2 << 20);
+  if (t >= 2 && t < 5) {
+    const unsigned ui = m[VQ_U + t - 2];  // (unscaled: a stretched element's pressure terms differ as well)
+    bad = bad || (ui != 0u && ui < fx_down(mu, 4) && r + 2 * fx_log(mu) - fx_log(m[VQ_P]) > 4 << 20);
+  }
+  return fx_any<N>(bad, t);
+}
 
 // Threads 0 .. 2 of the element form the shifts of one direction each
 // (vol_scale) and then align the directions' sums (vol_align), which reads the
 // other two threads' scales: the caller synchronises the whole warp between
 // the two, outside the branch on the thread (at N = 1 it holds four elements).
-__device__ __forceinline__ void vol_scale(VolScale& s, const unsigned* m, const Ops* o, int t) {
-  const int eR = fx_exp(m[VQ_RHO]), eU = fx_exp(max(max(m[VQ_U], m[VQ_V]), m[VQ_W])), eP = fx_exp(m[VQ_P]),
-            eH = fx_exp(m[VQ_H]);
-  const unsigned* mj = m + VQ_J + 3 * t;
-  const int eJ = fx_exp(max(max(mj[0], mj[1]), mj[2]));
+// Returns whether the element is plain: the three components share their
+// shifts (kep_fx) and no value is quiet or out of range.
+__device__ __forceinline__ bool vol_scale(VolScale& s, const unsigned* m, const Ops* o, int t, bool bad) {
+  const int eR = fx_exp(m[VQ_RHO]), eP = fx_exp(m[VQ_P]), eH = fx_exp(m[VQ_H]);
+  int eJ[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) eJ[i] = fx_exp(max(max(m[VQ_J + i], m[VQ_J + 3 + i]), m[VQ_J + 6 + i]));
+  const int eJx = max(max(eJ[0], eJ[1]), eJ[2]);
+  // nearly equal components share the largest exponent (two bits at most)
+  const bool iso = eJx - min(min(eJ[0], eJ[1]), eJ[2]) <= 2;
+  if (iso) eJ[0] = eJ[1] = eJ[2] = eJx;
+  const int eU = max(max(fx_exp(m[VQ_U]) + eJ[0], fx_exp(m[VQ_V]) + eJ[1]), fx_exp(m[VQ_W]) + eJ[2]);
+  float uf[3], jf[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    uf[i] = fx_frac(m[VQ_U + i], eU - eJ[i]);
+    jf[i] = fx_frac(m[VQ_J + 3 * t + i], eJ[i]);
+  }
   const float fR = fx_frac(m[VQ_RHO], eR), fP = fx_frac(m[VQ_P], eP), fH = fx_frac(m[VQ_H], eH), fS = o->fxS_row;
-  const float u0 = fx_frac(m[VQ_U], eU), u1 = fx_frac(m[VQ_V], eU), u2 = fx_frac(m[VQ_W], eU);
-  const float j0 = fx_frac(mj[0], eJ), j1 = fx_frac(mj[1], eJ), j2 = fx_frac(mj[2], eJ);
   DirScale& d = s.d[t];
-  d.eJ = eJ;
   // bounds in units of 2^58 (un), 2^60 and 2^61 (the others)
-  float b = u0 * j0 + u1 * j1 + u2 * j2;
-  d.s1 = fx_room(b, 4);
-  b = fR * ldexpf(b, d.s1 - 4);  // fr / 2^60
-  d.s2 = fx_room(b, 2);
-  b = fS * ldexpf(b, d.s2 - 2);  // t / 2^60, summed over a row
-  d.s3 = fx_room(b, 1);
-  const float bt = ldexpf(b, d.s3 - 1);  // t / 2^61
+  float b = uf[0] * jf[0] + uf[1] * jf[1] + uf[2] * jf[2];
+  const int s1 = fx_room(b, 4);
+  b = fR * fx_scale(b, s1 - 4);  // fr / 2^60
+  const int s2 = fx_room(b, 2);
+  b = fS * fx_scale(b, s2 - 2);  // t / 2^60, summed over a row
+  const int s3 = fx_room(b, 1);
+  const float bt = fx_scale(b, s3 - 1);  // t / 2^61
   const float bp0 = fS * fP;             // pressure / 2^60
-  d.s4 = fx_room(bp0, 2);
-  // scales: value times 2^a
-  const int a3 = o->fxS_bits + 61 - eR + 56 - eU - eJ + d.s1 - 128 + d.s2 + d.s3;
-  const int b3 = o->fxS_bits + 61 - eP - 64 + d.s4;
-  const int delta = (a3 - eU + 2) - (b3 - eJ);
-  d.kc = min(max(delta, 0), 62);
-  const int kp = max(-delta, 0);
-  float bp = ldexpf(bp0, d.s4 - 1);  // pressure / 2^61
-  bp = ldexpf(bp, -kp);
-  d.s4 -= kp;  // (below zero: a right shift, see kep_fx)
-  const float bm = ldexpf(bt, -d.kc) * fmaxf(u0, fmaxf(u1, u2)) + bp * fmaxf(j0, fmaxf(j1, j2));  // momentum / 2^58
-  d.s5 = fx_room(bm, 3);
-  const float be = bt * fH;  // energy / 2^59
-  d.s6 = fx_room(be, 2);
-  // the means' factors 1/8 (mass), 1/4 (pressure) and 1/16 (energy) included; 1/w (fxW)
+  const int s4 = fx_room(bp0, 2);
+  d.s1 = s1, d.s2 = s2, d.s3 = s3;
+  // scales: value times 2^a; the means' factors 1/8 (mass), 1/4 (pressure) and 1/16 (energy); 1/w (fxW)
+  const int a3 = o->fxS_bits + 61 - eR + 56 - eU + s1 - 128 + s2 + s3;
+  const int b3 = o->fxS_bits + 61 - eP - 64 + s4;
   const int w = o->fxW_bits - 62;
   s.c[t][0] = a3 + 3 + w;
-  s.c[t][1] = b3 - kp - eJ - 2 + d.s5 + w;
-  s.c[t][2] = a3 - eH + 1 + d.s6 + w;
+  if (iso) uf[0] = fmaxf(uf[0], fmaxf(uf[1], uf[2])), jf[0] = fmaxf(jf[0], fmaxf(jf[1], jf[2]));
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (iso && i > 0) {  // as the first
+      d.kc[i] = d.kc[0], d.s4[i] = d.s4[0], d.s5[i] = d.s5[0], s.c[t][1 + i] = s.c[t][1];
+      continue;
+    }
+    // t u_i against p m_i; a component whose metric (or velocity) is zero has the other's scale
+    const int at = a3 - (eU - eJ[i]) + 2, ap = b3 - eJ[i];
+    const bool of_t = jf[i] == 0.0f || (at < ap && uf[i] != 0.0f);
+    const int kc = of_t ? 0 : min(max(at - ap, 0), 62), kp = of_t ? min(max(ap - at, 0), 90) : 0;
+    const float bp = jf[i] == 0.0f ? 0.0f : fx_scale(bp0, s4 - 1 - kp);  // pressure / 2^61
+    const int s5 = fx_room(fx_scale(bt, -kc) * uf[i] + bp * jf[i], 3);  // momentum / 2^58
+    d.kc[i] = kc;
+    d.s4[i] = s4 - (jf[i] == 0.0f ? 90 : kp);
+    d.s5[i] = s5;
+    s.c[t][1 + i] = (of_t ? at : ap) - 2 + s5 + w;
+  }
+  d.s6 = fx_room(bt * fH, 2);  // energy / 2^59
+  s.c[t][4] = a3 - eH + 1 + d.s6 + w;
   if (t == 0) {
     s.eR = eR, s.eU = eU, s.eP = eP, s.eH = eH;
-    // In FP64: groups out of range, and elements whose largest fluxes lie far
-    // below the product of their groups' maxima (light and fast or hot fluid
-    // beside dense fluid, ratios above four): their scale would leave the
-    // fluxes fewer bits than FP64 gives them.
-    bool bad = false;
-    for (int k = 0; k < VQ_N; ++k) bad = bad || fx_bad(m[k]);
-    const int eX = fx_exp(m[VQ_RHOH]), eM = fx_exp(m[VQ_MOM]);
-    const int lh = min(max(eR + eH - eX, -60), 60), lm = min(max(eR + eU - eM, -60), 60);
-    bad = bad || fR * fH * ldexpf(1.0f, lh) > 4.0f * fx_frac(m[VQ_RHOH], eX);
-    bad = bad || fR * fmaxf(u0, fmaxf(u1, u2)) * ldexpf(1.0f, lm) > 4.0f * fx_frac(m[VQ_MOM], eM);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s.eJ[i] = eJ[i];
     s.bad = bad;
+    s.quiet = 0u;
+    s.iso = iso;
   }
+  return iso && !bad && ~m[VQ_LO] >= fx_cut(m[VQ_RHO]) && ~m[VQ_LO + 1] >= fx_cut(m[VQ_P]) &&
+         ~m[VQ_LO + 2] >= fx_cut(m[VQ_RHOH]);
 }
 __device__ __forceinline__ void vol_align(VolScale& s, int t) {
-  int p[3];
+  int p[5];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) p[k] = min(min(s.c[0][k], s.c[1][k]), s.c[2][k]);
+  for (int k = 0; k < 5; ++k) p[k] = min(min(s.c[0][k], s.c[1][k]), s.c[2][k]);
   DirScale& d = s.d[t];
-  d.aM = min(s.c[t][0] - p[0], 63), d.aV = min(s.c[t][1] - p[1], 63), d.aE = min(s.c[t][2] - p[2], 63);
-  if (t == 0) s.pM = p[0], s.pV = p[1], s.pE = p[2];
+  d.aM = min(s.c[t][0] - p[0], 62), d.aE = min(s.c[t][4] - p[4], 62);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) d.aV[i] = min(s.c[t][1 + i] - p[1 + i], 62);
+  if (t == 0) {
+    s.pM = p[0], s.pE = p[4];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s.pV[i] = p[1 + i];
+  }
+}
+// The form of the element's two-point sums: in FP64 where the scales ask for
+// it or where density, pressure or rho H are quiet on a node's lines (a corner
+// of an element that a strong front just enters).  The velocity needs no such
+// test: within a stable time step an error of 2^-59 of the element's largest
+// mass or energy flux changes a node's density and energy by less than FP64's
+// rounding of them (unless those are quiet), the momentum's by less than that
+// of the pressure terms.
+template <int N>
+__device__ __forceinline__ SumForm vol_form(VolScale* sc, const unsigned* m, const longlong2* P, int t) {
+  constexpr int n = Fix<N>::n, Pn = Fix<N>::Pn;
+  const double2* Pd = reinterpret_cast<const double2*>(P);
+  auto rho = [=](int v) { return fx_mag(Pd[fx_pad<n>(v)].x); };
+  auto prs = [=](int v) { return fx_mag(Pd[fx_pad<n>(v)].y); };
+  auto rhoH = [=](int v) { return fx_mag(Pd[fx_pad<n>(v)].x * Pd[2 * Pn + fx_pad<n>(v)].y); };
+  const unsigned cR = fx_cut(m[VQ_RHO]), cP = fx_cut(m[VQ_P]), cH = fx_cut(m[VQ_RHOH]);
+  return sum_form<N>(sc->bad != 0u, t, &sc->quiet, [=](int v) {
+    return (rho(v) < cR && lines_quiet<n>(v, cR, rho)) || (prs(v) < cP && lines_quiet<n>(v, cP, prs)) ||
+           (rhoH(v) < cH && lines_quiet<n>(v, cH, rhoH));
+  });
 }
 
 // shared memory: S = w Dsplit, 1/w and Dhat split (Fx), Vinv, the reduction
@@ -597,7 +821,8 @@ struct VolFix {
   static_assert(offP % 2 == 0 && per_elem % 2 == 0 && (6 * F::Pn) % 2 == 0, "16-byte alignment of the pair planes");
 };
 
-// One two-point flux of KEP type, times S: (t, f1, f2, f3, f4)
+// One two-point flux of KEP type, times S: (t, f1, f2, f3, f4).  ISO: the
+// momentum components share their shifts.
 struct KepNode {
   longlong2 a0, a1, a2, j0;  // (rho, p), (u, v), (w, H), (m0, m1)
   long long j1;              // m2
@@ -607,23 +832,32 @@ __device__ __forceinline__ KepNode kep_load(const longlong2* P, const longlong2*
   constexpr int Pn = fx_plane<n>();
   return {P[pv], P[Pn + pv], P[2 * Pn + pv], Jab[pv], Jc[pv]};
 }
+template <bool ISO>
 __device__ __forceinline__ void kep_flux_fx(const KepNode& x, const KepNode& y, Fx S, const DirScale& d, long long f[5]) {
   // sums of two values: u and m below 2^61, rho, p and H below 2^62; every
   // result below 2^62 by the choice of its shift
-  const Fx m0 = fx_split(x.j0.x + y.j0.x), m1 = fx_split(x.j0.y + y.j0.y), m2 = fx_split(x.j1 + y.j1);
-  const Fx u0 = fx_split(x.a1.x + y.a1.x), u1 = fx_split(x.a1.y + y.a1.y), u2 = fx_split(x.a2.x + y.a2.x);
-  FxSumS un, fr, tt, pd, f1, f2, f3, f4;
-  un.add(u0, m0), un.add(u1, m1), un.add(u2, m2);
+  const Fx m[3] = {fx_split(x.j0.x + y.j0.x), fx_split(x.j0.y + y.j0.y), fx_split(x.j1 + y.j1)};
+  const Fx u[3] = {fx_split(x.a1.x + y.a1.x), fx_split(x.a1.y + y.a1.y), fx_split(x.a2.x + y.a2.x)};
+  FxSumS un, fr, tt, f4;
+  un.add(u[0], m[0]), un.add(u[1], m[1]), un.add(u[2], m[2]);
   fr.add(fx_split(x.a0.x + y.a0.x), fx_split(un.get(d.s1)));
   tt.add(S, fx_split(fr.get(d.s2)));
   f[0] = tt.get(d.s3);
-  const Fx tk = fx_split(f[0] >> d.kc);
-  pd.add(S, fx_split(x.a0.y + y.a0.y));
-  const Fx ps = fx_split(d.s4 >= 0 ? pd.get(d.s4) : pd.get(0) >> min(-d.s4, 63));
-  f1.add(tk, u0), f1.add(ps, m0);
-  f2.add(tk, u1), f2.add(ps, m1);
-  f3.add(tk, u2), f3.add(ps, m2);
-  f[1] = f1.get(d.s5), f[2] = f2.get(d.s5), f[3] = f3.get(d.s5);
+  const Fx p = fx_split(x.a0.y + y.a0.y);
+  Fx tk, ps;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (!ISO || i == 0) {
+      const int s4 = d.s4[i];
+      FxSumS pd;
+      pd.add(S, p);
+      tk = fx_split(f[0] >> d.kc[i]);
+      ps = fx_split(s4 >= 0 ? pd.get(s4) : pd.get(0) >> min(-s4, 62));
+    }
+    FxSumS fi;
+    fi.add(tk, u[i]), fi.add(ps, m[i]);
+    f[1 + i] = fi.get(d.s5[ISO ? 0 : i]);
+  }
   f4.add(fx_split(f[0]), fx_split(x.a2.y + y.a2.y));
   f[4] = f4.get(d.s6);
 }
@@ -635,7 +869,7 @@ __device__ __forceinline__ void kep_flux_fx(const KepNode& x, const KepNode& y, 
 // even n the partner n / 2 places on is taken from both sides.  That is 3 + 1
 // fluxes per node and direction at n = 8 where every node summing over all
 // its partners takes 7.
-template <int N>
+template <int N, bool ISO>
 __device__ __forceinline__ void kep_fx(const longlong2* P, const longlong2* Jab, const long long* Jc, long long* A,
                                        const Fx* sS, const Fx* sW, const VolScale* sc, int t, bool skip) {
   using F = Fix<N>;
@@ -660,17 +894,18 @@ __device__ __forceinline__ void kep_fx(const longlong2* P, const longlong2* Jab,
       for (int k = 1; k <= (n - 1) / 2; ++k) {
         const int al = id + k < n ? id + k : id + k - n, from = id >= k ? id - k : id - k + n;
         long long f[5];
-        kep_flux_fx(me, kep_load<n>(P, Jd, Jcd, fx_pad<n>(base + al * sd)), sS[id * n + al], ds, f);
+        kep_flux_fx<ISO>(me, kep_load<n>(P, Jd, Jcd, fx_pad<n>(base + al * sd)), sS[id * n + al], ds, f);
         const int src = min(lane0 + lane - id + from, 31);
 #pragma unroll
         for (int c = 0; c < 5; ++c) acc[c] += f[c] - __shfl_sync(0xffffffffu, f[c], src);
       }
       if constexpr (n % 2 == 0) {
-        const int al = id < n / 2 ? id + n / 2 : id - n / 2;
+        const bool low = id < n / 2;  // (S of the lower node, so that both take the same flux)
+        const int al = low ? id + n / 2 : id - n / 2;
         long long f[5];
-        kep_flux_fx(me, kep_load<n>(P, Jd, Jcd, fx_pad<n>(base + al * sd)), sS[id * n + al], ds, f);
+        kep_flux_fx<ISO>(me, kep_load<n>(P, Jd, Jcd, fx_pad<n>(base + al * sd)), sS[min(id, al) * n + max(id, al)], ds, f);
 #pragma unroll
-        for (int c = 0; c < 5; ++c) acc[c] += f[c];
+        for (int c = 0; c < 5; ++c) acc[c] += low ? f[c] : -f[c];
       }
       if (on) {
         const Fx wi = sW[id];
@@ -678,7 +913,7 @@ __device__ __forceinline__ void kep_fx(const longlong2* P, const longlong2* Jab,
         for (int c = 0; c < 5; ++c) {
           FxSum<2> y;  // 2^(61 + 62 - 64 + 2)
           y.add(wi, fx_split(acc[c]));
-          const long long z = y.get() >> (c == 0 ? ds.aM : c == 4 ? ds.aE : ds.aV);
+          const long long z = fx_shr(y.get(), c == 0 ? ds.aM : c == 4 ? ds.aE : ds.aV[ISO ? 0 : c - 1]);
           A[c * Pn + pv] = d == 0 ? z : A[c * Pn + pv] + z;
         }
       }
@@ -687,35 +922,62 @@ __device__ __forceinline__ void kep_fx(const longlong2* P, const longlong2* Jab,
     __syncthreads();
   }
 }
-// the same in FP64, one node: P and J hold FP64 values
-template <int n>
-__device__ void kep_f64(const double2* P, const double2* Jab, const double* Jc, const double* Dsplit, int v,
-                        double conv[5]) {
-  constexpr int Pn = fx_plane<n>();
-  const int pv = fx_pad<n>(v);
-#pragma unroll
-  for (int k = 0; k < 5; ++k) conv[k] = 0.0;
-  const double2 a0 = P[pv], a1 = P[Pn + pv], a2 = P[2 * Pn + pv];
+// the same in FP64 (P, J and A hold FP64 values), with the same exchange of
+// fluxes, so that an element whose sums are taken here costs the FP64 unit as
+// many of them
+template <int N>
+__device__ __noinline__ void kep_f64(const double2* P, const double2* Jab, const double* Jc, double* A,
+                                     const double* Dsplit, int t, bool skip) {
+  using F = Fix<N>;
+  constexpr int n = F::n, n3 = F::n3, Pn = F::Pn, LW = F::LW;
+  const int lane = F::TPE >= 32 ? t & 31 : t;
+  const int lane0 = F::TPE >= 32 ? 0 : (threadIdx.x & 31) - t;
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
-    const int id = dir_index<n>(v, d), sd = dir_stride<n>(d), base = v - id * sd;
-    const double2 j0 = Jab[d * Pn + pv];
-    const double j1 = Jc[d * Pn + pv];
+    const int sd = dir_stride<n>(d);
+    const double2* Jd = Jab + d * Pn;
+    const double* Jcd = Jc + d * Pn;
 #pragma unroll 1
-    for (int al = 0; al < n; ++al) {
-      if (al == id) continue;
-      const int pa = fx_pad<n>(base + al * sd);
-      const double2 b0 = P[pa], b1 = P[Pn + pa], b2 = P[2 * Pn + pa], c0 = Jab[d * Pn + pa];
-      const double m0 = j0.x + c0.x, m1 = j0.y + c0.y, m2 = j1 + Jc[d * Pn + pa];  // twice the means
-      const double u0 = a1.x + b1.x, u1 = a1.y + b1.y, u2 = a2.x + b2.x;
-      const double D = 0.125 * Dsplit[id * n + al], p = 2.0 * (a0.y + b0.y);
-      const double fr = (a0.x + b0.x) * (u0 * m0 + u1 * m1 + u2 * m2), hf = 0.5 * fr;
-      conv[0] += D * fr;
-      conv[1] += D * (hf * u0 + p * m0);
-      conv[2] += D * (hf * u1 + p * m1);
-      conv[3] += D * (hf * u2 + p * m2);
-      conv[4] += D * (hf * (a2.y + b2.y));
+    for (int r = 0; r < F::RL; ++r) {
+      const int slot = ((t / 32) + r * F::W) * LW + lane;
+      const bool on = lane < LW && slot < n3 && !skip;
+      const int line = on ? slot / n : 0, id = lane % n, base = line_base<n>(d, line);
+      const int pv = fx_pad<n>(base + id * sd);
+      const double2 a0 = P[pv], a1 = P[Pn + pv], a2 = P[2 * Pn + pv], j0 = Jd[pv];
+      const double j1 = Jcd[pv];
+      double acc[5] = {0, 0, 0, 0, 0};
+      auto flux = [&](int al, double f[5]) {  // eight times the flux's mass part, and so on
+        const int pa = fx_pad<n>(base + al * sd);
+        const double2 b0 = P[pa], b1 = P[Pn + pa], b2 = P[2 * Pn + pa], c0 = Jd[pa];
+        const double m0 = j0.x + c0.x, m1 = j0.y + c0.y, m2 = j1 + Jcd[pa];  // twice the means
+        const double u0 = a1.x + b1.x, u1 = a1.y + b1.y, u2 = a2.x + b2.x, p = 2.0 * (a0.y + b0.y);
+        const double fr = (a0.x + b0.x) * (u0 * m0 + u1 * m1 + u2 * m2), hf = 0.5 * fr;
+        f[0] = fr, f[1] = hf * u0 + p * m0, f[2] = hf * u1 + p * m1, f[3] = hf * u2 + p * m2, f[4] = hf * (a2.y + b2.y);
+      };
+      double f[5];
+#pragma unroll
+      for (int k = 1; k <= (n - 1) / 2; ++k) {
+        const int al = id + k < n ? id + k : id + k - n, from = id >= k ? id - k : id - k + n;
+        flux(al, f);
+        const int src = min(lane0 + lane - id + from, 31);
+        const double D = 0.125 * Dsplit[id * n + al], Df = 0.125 * Dsplit[id * n + from];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[c] += D * f[c] + Df * __shfl_sync(0xffffffffu, f[c], src);
+      }
+      if constexpr (n % 2 == 0) {
+        const int al = id < n / 2 ? id + n / 2 : id - n / 2;
+        const double D = 0.125 * Dsplit[id * n + al];
+        flux(al, f);
+#pragma unroll
+        for (int c = 0; c < 5; ++c) acc[c] += D * f[c];
+      }
+      if (on) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) A[c * Pn + pv] = d == 0 ? acc[c] : A[c * Pn + pv] + acc[c];
+      }
     }
+    __syncwarp();
+    __syncthreads();
   }
 }
 
@@ -757,6 +1019,8 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
   if (t == 7 && MODE == 1 && !a.first_stage) prefetch64(a.dU, (size_t)e * 5 * n3, 5 * n3);
   prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
   // ---- primitives (FP64 in their planes until the scales are known), maxima ----
+  bool iso = true;
+  SumForm form = {false, false, false};
   {
     unsigned m[VQ_N];
 #pragma unroll
@@ -770,25 +1034,30 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
       Pd[0] = make_double2(pr.rho, pr.p);
       Pd[Pn] = make_double2(pr.u, pr.v);
       Pd[2 * Pn] = make_double2(pr.w, H);
-      m[VQ_RHO] = max(m[VQ_RHO], fx_mag(pr.rho));
+      m[VQ_RHO] = max(m[VQ_RHO], fx_mag(pr.rho)), m[VQ_LO] = max(m[VQ_LO], ~fx_mag(pr.rho));
       m[VQ_U] = max(m[VQ_U], fx_mag(pr.u));
       m[VQ_V] = max(m[VQ_V], fx_mag(pr.v));
       m[VQ_W] = max(m[VQ_W], fx_mag(pr.w));
-      m[VQ_P] = max(m[VQ_P], fx_mag(pr.p));
+      m[VQ_P] = max(m[VQ_P], fx_mag(pr.p)), m[VQ_LO + 1] = max(m[VQ_LO + 1], ~fx_mag(pr.p));
       m[VQ_H] = max(m[VQ_H], fx_mag(H));
-      m[VQ_RHOH] = max(m[VQ_RHOH], fx_mag(rH));
+      m[VQ_RHOH] = max(m[VQ_RHOH], fx_mag(rH)), m[VQ_LO + 2] = max(m[VQ_LO + 2], ~fx_mag(rH));
       m[VQ_MOM] = max(max(m[VQ_MOM], fx_mag(U[1])), max(fx_mag(U[2]), fx_mag(U[3])));
 #pragma unroll
       for (int c = 0; c < 9; ++c) m[VQ_J + c] = max(m[VQ_J + c], fx_mag(Me[c * n3 + v]));
     }
     fx_reduce<N, VQ_N>(m, red, fin, t);
-    if (t < 3) vol_scale(*sc, fin, a.ops, t);
+    bool plain = true, out = false;
+    if (t < 32) out = vol_bad<N>(fin, t);
+    if (t < 3) plain = vol_scale(*sc, fin, a.ops, t, out);
     __syncwarp();
     if (t < 3) vol_align(*sc, t);
     __syncwarp();
-    __syncthreads();
+    if (!__syncthreads_and(plain)) {  // (all of the block's elements)
+      iso = __syncthreads_and(sc->iso != 0u);
+      form = vol_form<N>(sc, fin, P, t);
+    }
   }
-  const bool bad = sc->bad != 0;
+  const bool bad = form.direct;
   for (int v = t; v < n3; v += TPE) {
     const int pv = fx_pad<n>(v);
     double mt[9];
@@ -804,38 +1073,36 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
       const double2* Pd = reinterpret_cast<const double2*>(P) + pv;
       const double2 x0 = Pd[0], x1 = Pd[Pn], x2 = Pd[2 * Pn];
       P[pv] = make_longlong2(fx_from<61>(x0.x, sc->eR), fx_from<61>(x0.y, sc->eP));
-      P[Pn + pv] = make_longlong2(fx_from<60>(x1.x, sc->eU), fx_from<60>(x1.y, sc->eU));
-      P[2 * Pn + pv] = make_longlong2(fx_from<60>(x2.x, sc->eU), fx_from<61>(x2.y, sc->eH));
+      const int e0 = sc->eJ[0], e1 = sc->eJ[1], e2 = sc->eJ[2], eU = sc->eU;
+      P[Pn + pv] = make_longlong2(fx_from<60>(x1.x, eU - e0), fx_from<60>(x1.y, eU - e1));
+      P[2 * Pn + pv] = make_longlong2(fx_from<60>(x2.x, eU - e2), fx_from<61>(x2.y, sc->eH));
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        const int eJ = sc->d[d].eJ;
-        Jab[d * Pn + pv] = make_longlong2(fx_from<60>(mt[3 * d], eJ), fx_from<60>(mt[3 * d + 1], eJ));
-        Jc[d * Pn + pv] = fx_from<60>(mt[3 * d + 2], eJ);
+        Jab[d * Pn + pv] = make_longlong2(fx_from<60>(mt[3 * d], e0), fx_from<60>(mt[3 * d + 1], e1));
+        Jc[d * Pn + pv] = fx_from<60>(mt[3 * d + 2], e2);
       }
     }
   }
   __syncwarp();
   __syncthreads();
   // ---- split-form KEP volume integral ----
-  kep_fx<N>(P, Jab, Jc, A, sS, sW, sc, t, bad);
+  if (!form.all) {
+    if (iso) kep_fx<N, true>(P, Jab, Jc, A, sS, sW, sc, t, bad);
+    else kep_fx<N, false>(P, Jab, Jc, A, sS, sW, sc, t, bad);
+  }
+  if (form.any)
+    kep_f64<N>(reinterpret_cast<const double2*>(P), reinterpret_cast<const double2*>(Jab),
+               reinterpret_cast<const double*>(Jc), reinterpret_cast<double*>(A), a.ops->Dsplit, t, !bad);
   double conv[R][5];  // convective DG volume term
   double visc[R][4];  // viscous volume term
   long long vel[R][3];  // the velocity in fixed point (FP64 values in a bad element)
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int v = t + r * TPE, pv = fx_pad<n>(v < n3 ? v : 0);
-    if (bad) {
-      double c5[5] = {0, 0, 0, 0, 0};
-      if (v < n3)
-        kep_f64<n>(reinterpret_cast<const double2*>(P), reinterpret_cast<const double2*>(Jab),
-                   reinterpret_cast<const double*>(Jc), a.ops->Dsplit, v, c5);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) conv[r][k] = c5[k];
-    } else {
-      conv[r][0] = fx_to(A[pv], sc->pM);
-#pragma unroll
-      for (int k = 1; k < 4; ++k) conv[r][k] = fx_to(A[k * Pn + pv], sc->pV);
-      conv[r][4] = fx_to(A[4 * Pn + pv], sc->pE);
+    for (int k = 0; k < 5; ++k) {
+      const long long y = A[k * Pn + pv];
+      conv[r][k] = bad ? __longlong_as_double(y) : fx_to(y, k == 0 ? sc->pM : k == 4 ? sc->pE : sc->pV[k - 1]);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) visc[r][k] = 0.0;
@@ -850,7 +1117,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     // thread reads back its own nodes only
     long long* T = mine + L::offT;
     {
-      unsigned mv[2] = {0, 0};
+      unsigned mv[4] = {0, 0, 0, 0};
       for (int v = t; v < n3; v += TPE) {
         double g[12];
         const double* pg = a.g + (size_t)e * 12 * n3 + v;
@@ -872,17 +1139,26 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
           Td[k * n3] = x[k];
-          mv[k / 6] = max(mv[k / 6], fx_mag(x[k]));
+          mv[k < 6 ? 0 : k - 5] = max(mv[k < 6 ? 0 : k - 5], fx_mag(x[k]));
         }
       }
-      fx_reduce<N, 2>(mv, red, fin, t);
+      fx_reduce<N, 4>(mv, red, fin, t);
       __syncthreads();
     }
-    // (an element that leaves the range only here has its metrics in fixed
-    // point: the FP64 sums then read them from memory)
-    const bool vbad = bad || fx_bad(fin[0]) || fx_bad(fin[1]);
-    const int eT = fx_exp(fin[0]), eL = fx_exp(fin[1]), eJm = max(max(sc->d[0].eJ, sc->d[1].eJ), sc->d[2].eJ);
-    const int eTU = eT + sc->eU, eW = max(eTU, eL) + 2;  // W: below 2^60 at 2^(60 - eW)
+    // The six stresses share an exponent and are contracted with the metrics
+    // at their largest component's: an error below FP64's rounding of the
+    // pressure terms of the same sums while the stresses stay below the
+    // pressure by the element's stretching.  W_j is held as W_j 2^(eJ_j), like
+    // the velocity.  (An element that leaves the range only here has its
+    // metrics in fixed point: the FP64 sums then read them from memory.)
+    const int eJ[3] = {sc->eJ[0], sc->eJ[1], sc->eJ[2]};
+    const int eJm = max(max(eJ[0], eJ[1]), eJ[2]), eJn = min(min(eJ[0], eJ[1]), eJ[2]);
+    const int eT = fx_exp(fin[0]), eL[3] = {fx_exp(fin[1]), fx_exp(fin[2]), fx_exp(fin[3])};
+    const bool vbad = bad || fx_bad(fin[0]) || fx_bad(fin[1]) || fx_bad(fin[2]) || fx_bad(fin[3]) ||
+                      eT + eJm - eJn > sc->eP + 1;
+    const int eUm = sc->eU - eJn, eTU = eT + eUm;
+    // W_j: below 2^60 at 2^(60 - eW + eJ_j)
+    const int eW = max(max(max(eTU, eL[0]) + eJ[0], max(eTU, eL[1]) + eJ[1]), max(eTU, eL[2]) + eJ[2]) + 2;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int v = t + r * TPE;
@@ -894,7 +1170,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
           for (int k = 0; k < 3; ++k) u[k] = __longlong_as_double(vel[r][k]);
         } else {
 #pragma unroll
-          for (int k = 0; k < 3; ++k) u[k] = fx_to(vel[r][k], 60 - sc->eU);
+          for (int k = 0; k < 3; ++k) u[k] = fx_to(vel[r][k], 60 - sc->eU + eJ[k]);
         }
         double* Td = reinterpret_cast<double*>(T) + v;
         const double t0 = Td[0], t1 = Td[n3], t2 = Td[2 * n3], t3 = Td[3 * n3], t4 = Td[4 * n3], t5 = Td[5 * n3];
@@ -909,16 +1185,16 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
           T[k * n3 + v] = q;
           x[k] = fx_split(q);
         }
-        const Fx u = fx_split(vel[r][0]), w1 = fx_split(vel[r][1]), w2 = fx_split(vel[r][2]);
+        const Fx u = fx_split(fx_shr(vel[r][0], min(eJ[0] - eJn, 62))), w1 = fx_split(fx_shr(vel[r][1], min(eJ[1] - eJn, 62))),
+                 w2 = fx_split(fx_shr(vel[r][2], min(eJ[2] - eJn, 62)));
         FxSum<2> w[3];  // 3 2^(60 + 60 - 64 + 2) < 2^59.6
         w[0].add(x[0], u), w[0].add(x[3], w1), w[0].add(x[4], w2);
         w[1].add(x[3], u), w[1].add(x[1], w1), w[1].add(x[5], w2);
         w[2].add(x[4], u), w[2].add(x[5], w1), w[2].add(x[2], w2);
-        const int sU = min(eW - 2 - eTU, 63), sL = min(eW - 2 - eL, 63);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-          T[(6 + k) * n3 + v] =
-              (w[k].get() >> sU) + (fx_from<58>(__longlong_as_double(T[(6 + k) * n3 + v]), eL) >> sL);
+          T[(6 + k) * n3 + v] = fx_shr(w[k].get(), min(eW - eJ[k] - 2 - eTU, 62)) +
+                                fx_shr(fx_from<58>(__longlong_as_double(T[(6 + k) * n3 + v]), eL[k]), min(eW - eJ[k] - 2 - eL[k], 62));
       }
     }
     long long acc[R][4];
@@ -943,7 +1219,12 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
           reinterpret_cast<double2*>(G)[Pn + pv] = make_double2(fv[2], fv[3]);
         } else {
           const longlong2 jab = Jab[d * Pn + pv];
-          const Fx j0 = fx_split(jab.x), j1 = fx_split(jab.y), j2 = fx_split(Jc[d * Pn + pv]);
+          const long long jc = Jc[d * Pn + pv];
+          const Fx c0 = fx_split(jab.x), c1 = fx_split(jab.y), c2 = fx_split(jc);  // by component, for W
+          Fx j0 = c0, j1 = c1, j2 = c2;                                           // at the largest's exponent
+          if (!iso)
+            j0 = fx_split(fx_shr(jab.x, min(eJm - eJ[0], 62))), j1 = fx_split(fx_shr(jab.y, min(eJm - eJ[1], 62))),
+            j2 = fx_split(fx_shr(jc, min(eJm - eJ[2], 62)));
           Fx x[9];
 #pragma unroll
           for (int k = 0; k < 9; ++k) x[k] = fx_split(T[k * n3 + v]);
@@ -951,7 +1232,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
           f1.add(x[0], j0), f1.add(x[3], j1), f1.add(x[4], j2);
           f2.add(x[3], j0), f2.add(x[1], j1), f2.add(x[5], j2);
           f3.add(x[4], j0), f3.add(x[5], j1), f3.add(x[2], j2);
-          f4.add(x[6], j0), f4.add(x[7], j1), f4.add(x[8], j2);
+          f4.add(x[6], c0), f4.add(x[7], c1), f4.add(x[8], c2);
           G[pv] = make_longlong2(f1.get(), f2.get());
           G[Pn + pv] = make_longlong2(f3.get(), f4.get());
         }
@@ -980,15 +1261,14 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
               const Fx c = sDh[id * n + al];
               s1.add(c, fx_split(g0.x)), s2.add(c, fx_split(g0.y)), s3.add(c, fx_split(g1.x)), s4.add(c, fx_split(g1.y));
             }
-            const int sh = min(eJm - sc->d[d].eJ, 63);  // the directions' metrics have their own exponents
-            acc[r][0] += s1.get() >> sh, acc[r][1] += s2.get() >> sh, acc[r][2] += s3.get() >> sh, acc[r][3] += s4.get() >> sh;
+            acc[r][0] += s1.get(), acc[r][1] += s2.get(), acc[r][2] += s3.get(), acc[r][3] += s4.get();
           }
         }
       }
       __syncwarp();
       __syncthreads();
     }
-    const int pT = a.ops->fxH_bits - 3 - eT - eJm, pW = a.ops->fxH_bits - 3 - eW - eJm;
+    const int pT = a.ops->fxH_bits - 3 - eT - eJm, pW = a.ops->fxH_bits - 3 - eW;
     if (!vbad) {
 #pragma unroll
       for (int r = 0; r < R; ++r)
@@ -1096,28 +1376,6 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
       for (int k = 0; k < 5; ++k) s[k] += sg * Fs[k * n2];
     }
     finish_node64<n, MODE, EXTRA>(a, e, er.ce, v, s);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The lifting's sums of one node in FP64, for elements outside the fixed-point range
-// ---------------------------------------------------------------------------
-template <int n>
-__device__ __noinline__ void lift_direct(const StageArgs& a, int e, int v, double acc[12]) {
-  constexpr int n3 = n * n * n;
-  const double* Me = a.metric + (size_t)e * 10 * n3;
-  for (int k = 0; k < 12; ++k) acc[k] = 0.0;
-  for (int d = 0; d < 3; ++d) {
-    const int id = dir_index<n>(v, d), sd = dir_stride<n>(d);
-    for (int al = 0; al < n; ++al) {
-      const int va = v + (al - id) * sd;
-      double U[5];
-      load_state64<n>(a, e, va, U);
-      const Prim64 pr = prim64(U, a.gm1);
-      const double q[4] = {pr.u, pr.v, pr.w, pr.p * pr.ri * a.Rinv}, c = a.ops->Dhat[id * n + al];
-      for (int k = 0; k < 4; ++k)
-        for (int x = 0; x < 3; ++x) acc[3 * k + x] += c * (Me[(3 * d + x) * n3 + va] * q[k]);
-    }
   }
 }
 

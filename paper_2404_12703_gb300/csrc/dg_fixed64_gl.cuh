@@ -19,8 +19,8 @@ __device__ __forceinline__ FaceRef slot_ref(const StageArgs& a, int e, int slot)
 // ---------------------------------------------------------------------------
 // Lifted gradients and their ProlongToFace
 // ---------------------------------------------------------------------------
-// shared memory: Dhat's table, l / w and l at the ends, the reduction words,
-// then per element the planes of k_lift_fx (q and J planes: also the six
+// shared memory: Dhat's table, l / w and l at the ends, Dhat's table in FP64,
+// the reduction words, then per element the planes of k_lift_fx (q and J planes: also the six
 // faces' lifting fluxes [12][6 n2]; W planes: also the gradients)
 template <int N>
 struct LiftGlFix {
@@ -28,10 +28,17 @@ struct LiftGlFix {
   static constexpr int ntab = LiftFix<N>::ntab + 4 * F::n;
   static constexpr int nqj = 10 * F::Pn > 72 * F::n2 ? 10 * F::Pn : 72 * F::n2;
   static constexpr int per_elem = nqj + 12 * F::Pn;
-  static constexpr int Q = 12, nred = F::W * Q + 11 + 12;
-  static constexpr size_t head(int epb) { return (8 * ntab + 4 * (size_t)epb * nred + 15) & ~size_t(15); }
+  static constexpr int Q = 20, nred = F::W * Q + 20 + 12 + 1;
+  static constexpr size_t head(int epb) { return (8 * (ntab + LiftFix<N>::ntab) + 4 * (size_t)epb * nred + 15) & ~size_t(15); }
   static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * per_elem; }
 };
+
+// (out of line here, where its registers cost the fixed-point path more than a call: 337 against 347 us)
+template <int N>
+__device__ __noinline__ void lift_sums_f64_call(const Ops* o, const double* Me, const double* q, double* J, double* W,
+                                                double* sD, int t, bool skip) {
+  lift_sums_f64<N>(o, Me, q, J, W, sD, t, skip);
+}
 
 template <int N>
 __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fix<N>::TPE * Fix<N>::D))
@@ -44,9 +51,11 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
   Fx* sD = reinterpret_cast<Fx*>(smraw);
   Fx* sL = sD + LiftFix<N>::ntab;  // [2][n] l(-1) / w, l(+1) / w
   Fx* sE = sL + 2 * n;             // [2][n] l(-1), l(+1)
-  unsigned* red = reinterpret_cast<unsigned*>(sE + 2 * n) + le * L::nred;
-  unsigned* fin = red + F::W * L::Q;  // [11] maxima of the lifting
-  unsigned* fing = fin + 11;          // [12] of the gradients
+  double* sDd = reinterpret_cast<double*>(sE + 2 * n);  // (filled by lift_sums_f64)
+  unsigned* red = reinterpret_cast<unsigned*>(sDd + LiftFix<N>::ntab) + le * L::nred;
+  unsigned* fin = red + F::W * L::Q;  // [20] maxima of the lifting
+  unsigned* fing = fin + 20;          // [12] of the gradients
+  unsigned* flag = fing + 12;
   long long* q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::per_elem;
   long long* J = q + 4 * Pn;
   long long* Fl = q;           // [12][6 n2] the faces' lifting fluxes (after the volume sums)
@@ -57,28 +66,32 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
   lift_table_fx<N>(a.ops, sD);
   for (int k = threadIdx.x; k < 2 * n; k += blockDim.x) sL[k] = fx_split(a.ops->fxL[k]), sE[k] = fx_split(a.ops->fxE[k]);
   prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
+  if (t == 0) *flag = 0u;
   {
-    unsigned m[11];  // those of lift_prims_fx, then the faces' fluxes: velocity and temperature by Cartesian component
+    unsigned m[20];  // those of lift_prims_fx, then the faces' fluxes, each of the 12 by itself
     lift_prims_fx<N>(a, e, q, m, t);
 #pragma unroll
-    for (int k = 5; k < 11; ++k) m[k] = 0;
+    for (int k = 8; k < 20; ++k) m[k] = 0;
     for (int s = t; s < 6 * n2; s += TPE) {
       const FaceRef r = slot_ref<n>(a, e, s);
       const double* Lr = a.lflux + (size_t)r.s * 12 * n2 + r.pqm;
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        const int g = (k < 9 ? 5 : 8) + k % 3;
-        m[g] = max(m[g], fx_mag(Lr[k * n2]));
-      }
+      for (int k = 0; k < 12; ++k) m[8 + k] = max(m[8 + k], fx_mag(Lr[k * n2]));
     }
-    fx_reduce<N, 11>(m, red, fin, t);
+    fx_reduce<N, 20>(m, red, fin, t);
     __syncthreads();
   }
   bool bad = false;
 #pragma unroll
-  for (int k = 0; k < 11; ++k) bad = bad || fx_bad(fin[k]);
-  const int eU = fx_exp(fin[0]), eT = fx_exp(fin[1]), eJ[3] = {fx_exp(fin[2]), fx_exp(fin[3]), fx_exp(fin[4])};
-  lift_sums_fx<N>(Me, q, J, W, sD, t, eU, eT, eJ);
+  for (int k = 0; k < 20; ++k) bad = bad || (k != 7 && fx_bad(fin[k]));
+  const int eq[4] = {fx_exp(fin[0]), fx_exp(fin[1]), fx_exp(fin[2]), fx_exp(fin[3])};
+  const int eJ[3] = {fx_exp(fin[4]), fx_exp(fin[5]), fx_exp(fin[6])};
+  const SumForm form = lift_form<N>(bad, q, fin, t, flag);
+  bad = form.direct;
+  if (!form.all) lift_sums_fx<N>(Me, q, J, W, sD, t, eq, eJ, bad);
+  if (form.any)
+    lift_sums_f64_call<N>(a.ops, Me, reinterpret_cast<const double*>(q), reinterpret_cast<double*>(J),
+                          reinterpret_cast<double*>(W), sDd, t, !bad);
   // the six faces' lifting fluxes q* (s n), signed for this element (the
   // slave's outward normal is minus the master's), in its face frames
   for (int s = t; s < 6 * n2; s += TPE) {
@@ -87,7 +100,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       const double x = r.slave ? -Lr[k * n2] : Lr[k * n2];
-      Fl[k * 6 * n2 + s] = bad ? __double_as_longlong(x) : fx_from<60>(x, fx_exp(fin[(k < 9 ? 5 : 8) + k % 3]));
+      Fl[k * 6 * n2 + s] = bad ? __double_as_longlong(x) : fx_from<60>(x, fx_exp(fin[8 + k]));
     }
   }
   __syncwarp();
@@ -100,10 +113,8 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
     const int idx[3] = {v % n, (v / n) % n, v / n2};
     double acc[12];
     if (bad) {
-      double d12[12];
-      lift_direct<n>(a, e, v, d12);
 #pragma unroll
-      for (int k = 0; k < 12; ++k) acc[k] = d12[k];
+      for (int k = 0; k < 12; ++k) acc[k] = __longlong_as_double(W[k * Pn + pv]);
       const double* Fd = reinterpret_cast<const double*>(Fl);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -127,10 +138,10 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
         FxSum<2> s;
 #pragma unroll
         for (int f = 0; f < 6; ++f) s.add(c[f], fx_split(Fl[k * 6 * n2 + at[f]]));
-        const int pV = a.ops->fxH_bits - 2 - (k < 9 ? eU : eT) - eJ[k % 3];
-        const int pS = a.ops->fxL_bits + 60 - 64 + 2 - fx_exp(fin[(k < 9 ? 5 : 8) + k % 3]);
+        const int pV = a.ops->fxH_bits - 2 - eq[k / 3] - eJ[k % 3];
+        const int pS = a.ops->fxL_bits + 60 - 64 + 2 - fx_exp(fin[8 + k]);
         const int p = min(pV, pS);
-        acc[k] = fx_to((W[k * Pn + pv] >> min(pV - p, 63)) + (s.get() >> min(pS - p, 63)), p);
+        acc[k] = fx_to(fx_shr(W[k * Pn + pv], min(pV - p, 62)) + fx_shr(s.get(), min(pS - p, 62)), p);
       }
     }
     const double Ji = Me[9 * n3 + v];
@@ -190,16 +201,26 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
 // Volume integral (collocated flux divergence) + SurfInt + ApplyJac (+ RK)
 // ---------------------------------------------------------------------------
 // A node's fluxes are a tensor T (rho u; rho u u + p - tau, symmetric; rho u H
-// - W: 12 numbers), contracted with each direction's metrics.
+// - W: 12 numbers in FP64), contracted with each direction's metrics.  The
+// metrics have an exponent eJ for each Cartesian component (over the three
+// directions), each of T's five rows one exponent for its three values scaled
+// by 2^(eJ_j), so that the products of a row meet in one scale whatever the
+// element's stretching (15 numbers).
 // shared memory: Dhat, l / w at the ends, the reduction words, then per
-// element the fluxes of one direction (5 planes), the tensor (12 planes, each
-// thread's own nodes only) and the six faces' surface fluxes [5][6 n2]
+// element the fluxes of one direction (5 planes), the tensor (15 planes) and
+// the six faces' surface fluxes [5][6 n2]
+// the place of row r, column j among the 12 numbers
+__device__ __forceinline__ constexpr int gl_at(int r, int j) {
+  return r == 0 ? j : r == 4 ? 9 + j : r - 1 == j ? 3 + j : 4 + r + j;  // xx, yy, zz, xy, xz, yz from 3 on
+}
+
 template <int N>
 struct VolGlFix {
   using F = Fix<N>;
   static constexpr int ntab = F::n2 + 2 * F::n;
-  static constexpr int offT = 5 * F::Pn, offS = offT + 12 * F::n3, per_elem = offS + 30 * F::n2;
-  static constexpr int Q = 9, nred = F::W * Q + Q;  // maxima: mass, momentum, energy rows; metrics by direction; f* of the three
+  static constexpr int offT = 5 * F::Pn, offS = offT + 15 * F::n3, per_elem = offS + 30 * F::n2;
+  // maxima: T; metrics by component; the five f*; density, pressure and rho H and their complements (minima); flag
+  static constexpr int Q = 26, nred = F::W * Q + Q + 1;
   static constexpr size_t head(int epb) { return (8 * ntab + 4 * (size_t)epb * nred + 15) & ~size_t(15); }
   static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * per_elem; }
 };
@@ -216,8 +237,9 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
   Fx* sL = sDh + n2;
   unsigned* red = reinterpret_cast<unsigned*>(sL + 2 * n) + le * L::nred;
   unsigned* fin = red + F::W * L::Q;
+  unsigned* flag = fin + L::Q;
   long long* G = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::per_elem;  // [5][Pn]
-  long long* T = G + L::offT;   // [12][n3]
+  long long* T = G + L::offT;   // [15][n3] (in FP64 the first 12)
   long long* Fs = G + L::offS;  // [5][6 n2]
   const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
   const int e = er.e;
@@ -229,6 +251,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
   }
   if (t == 7 && MODE == 1 && !a.first_stage) prefetch64(a.dU, (size_t)e * 5 * n3, 5 * n3);
   prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
+  if (t == 0) *flag = 0u;
   {
     unsigned m[L::Q];
 #pragma unroll
@@ -256,35 +279,68 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
       double* Td = reinterpret_cast<double*>(T) + v;
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
-        const int g = k < 3 ? 0 : k < 9 ? 1 : 2;
         Td[k * n3] = x[k];
-        m[g] = max(m[g], fx_mag(x[k]));
+        m[k] = max(m[k], fx_mag(x[k]));
       }
+      const unsigned lev[3] = {fx_mag(U[0]), fx_mag(pr.p), fx_mag(rH)};
 #pragma unroll
-      for (int c = 0; c < 9; ++c) m[3 + c / 3] = max(m[3 + c / 3], fx_mag(Me[c * n3 + v]));
+      for (int k = 0; k < 3; ++k) m[20 + k] = max(m[20 + k], lev[k]), m[23 + k] = max(m[23 + k], ~lev[k]);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) m[12 + c % 3] = max(m[12 + c % 3], fx_mag(Me[c * n3 + v]));
     }
     for (int s = t; s < 6 * n2; s += TPE) {
       const FaceRef r = slot_ref<n>(a, e, s);
       const double* src = a.fstar + (size_t)r.s * 5 * n2 + r.pqm;
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const int g = 6 + (k == 0 ? 0 : k < 4 ? 1 : 2);
-        m[g] = max(m[g], fx_mag(src[k * n2]));
-      }
+      for (int k = 0; k < 5; ++k) m[15 + k] = max(m[15 + k], fx_mag(src[k * n2]));
     }
     fx_reduce<N, L::Q>(m, red, fin, t);
     __syncthreads();
   }
   bool bad = false;
 #pragma unroll
-  for (int k = 0; k < L::Q; ++k) bad = bad || fx_bad(fin[k]);
-  const int eM = fx_exp(fin[0]), eV = fx_exp(fin[1]), eE = fx_exp(fin[2]);
-  const int eJm = max(max(fx_exp(fin[3]), fx_exp(fin[4])), fx_exp(fin[5]));
-  if (!bad)
-    for (int v = t; v < n3; v += TPE)
+  for (int k = 0; k < 20; ++k) bad = bad || fx_bad(fin[k]);
+  const int eJ[3] = {fx_exp(fin[12]), fx_exp(fin[13]), fx_exp(fin[14])};
+  int eR[5];  // the rows' exponents
 #pragma unroll
-      for (int k = 0; k < 12; ++k)
-        T[k * n3 + v] = fx_from<60>(__longlong_as_double(T[k * n3 + v]), k < 3 ? eM : k < 9 ? eV : eE);
+  for (int r = 0; r < 5; ++r) {
+    eR[r] = -4000;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) eR[r] = max(eR[r], fx_exp(fin[gl_at(r, j)]) + eJ[j]);
+  }
+  {
+    // FP64 sums where density, pressure or rho H are quiet on a node's lines (vol_form)
+    bool ask = bad;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ask = ask || ~fin[23 + k] < fx_cut(fin[20 + k]);
+    if (blockDim.x == TPE ? ask : __syncthreads_or(ask)) {
+      const double* u = a.U + (size_t)e * 5 * n3;
+      const double gm1 = a.gm1;
+      const unsigned cR = fx_cut(fin[20]), cP = fx_cut(fin[21]), cH = fx_cut(fin[22]);
+      auto level = [=](int v, int k) {
+        double U[5];
+        for (int i = 0; i < 5; ++i) U[i] = u[i * n3 + v];
+        const double p = prim64(U, gm1).p;
+        return fx_mag(k == 0 ? U[0] : k == 1 ? p : U[4] + p);
+      };
+      auto rho = [=](int v) { return level(v, 0); };
+      auto prs = [=](int v) { return level(v, 1); };
+      auto rhoH = [=](int v) { return level(v, 2); };
+      const SumForm form = sum_form<N>(bad, t, flag, [=](int v) {
+        return (rho(v) < cR && lines_quiet<n>(v, cR, rho)) || (prs(v) < cP && lines_quiet<n>(v, cP, prs)) ||
+               (rhoH(v) < cH && lines_quiet<n>(v, cH, rhoH));
+      });
+      bad = form.direct;
+    }
+  }
+  if (!bad)
+    for (int v = t; v < n3; v += TPE) {
+      double x[12];
+#pragma unroll
+      for (int k = 0; k < 12; ++k) x[k] = __longlong_as_double(T[k * n3 + v]);
+#pragma unroll
+      for (int k = 0; k < 15; ++k) T[k * n3 + v] = fx_from<60>(x[gl_at(k / 3, k % 3)], eR[k / 3] - eJ[k % 3]);
+    }
   // the six faces' fluxes f* s, signed for this element
   for (int s = t; s < 6 * n2; s += TPE) {
     const FaceRef r = slot_ref<n>(a, e, s);
@@ -292,7 +348,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       const double x = r.slave ? -src[k * n2] : src[k * n2];
-      Fs[k * 6 * n2 + s] = bad ? __double_as_longlong(x) : fx_from<60>(x, fx_exp(fin[6 + (k == 0 ? 0 : k < 4 ? 1 : 2)]));
+      Fs[k * 6 * n2 + s] = bad ? __double_as_longlong(x) : fx_from<60>(x, fx_exp(fin[15 + k]));
     }
   }
   long long acc[R][5];
@@ -303,7 +359,6 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
     for (int k = 0; k < 5; ++k) acc[r][k] = 0, sum[r][k] = 0.0;
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
-    const int eJ = fx_exp(fin[3 + d]);
     for (int v = t; v < n3; v += TPE) {
       const int pv = fx_pad<n>(v);
       const double nv[3] = {Me[3 * d * n3 + v], Me[(3 * d + 1) * n3 + v], Me[(3 * d + 2) * n3 + v]};
@@ -316,18 +371,15 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
         Gd[3 * Pn] = Td[7 * n3] * nv[0] + Td[8 * n3] * nv[1] + Td[5 * n3] * nv[2];
         Gd[4 * Pn] = Td[9 * n3] * nv[0] + Td[10 * n3] * nv[1] + Td[11 * n3] * nv[2];
       } else {
-        const Fx j0 = fx_split(fx_from<60>(nv[0], eJ)), j1 = fx_split(fx_from<60>(nv[1], eJ)),
-                 j2 = fx_split(fx_from<60>(nv[2], eJ));
-        auto row = [&](int x, int y, int z) {
+        const Fx j0 = fx_split(fx_from<60>(nv[0], eJ[0])), j1 = fx_split(fx_from<60>(nv[1], eJ[1])),
+                 j2 = fx_split(fx_from<60>(nv[2], eJ[2]));
+#pragma unroll
+        for (int r = 0; r < 5; ++r) {
+          const long long* x = T + 3 * r * n3 + v;
           FxSum<2> s;  // 3 2^(60 + 60 - 64 + 2) < 2^59.6
-          s.add(fx_split(T[x * n3 + v]), j0), s.add(fx_split(T[y * n3 + v]), j1), s.add(fx_split(T[z * n3 + v]), j2);
-          return s.get();
-        };
-        G[pv] = row(0, 1, 2);
-        G[Pn + pv] = row(3, 6, 7);
-        G[2 * Pn + pv] = row(6, 4, 8);
-        G[3 * Pn + pv] = row(7, 8, 5);
-        G[4 * Pn + pv] = row(9, 10, 11);
+          s.add(fx_split(x[0]), j0), s.add(fx_split(x[n3]), j1), s.add(fx_split(x[2 * n3]), j2);
+          G[r * Pn + pv] = s.get();
+        }
       }
     }
     __syncwarp();
@@ -353,7 +405,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
             for (int k = 0; k < 5; ++k) s[k].add(c, fx_split(G[k * Pn + pa]));
           }
 #pragma unroll
-          for (int k = 0; k < 5; ++k) acc[r][k] += s[k].get() >> min(eJm - eJ, 63);
+          for (int k = 0; k < 5; ++k) acc[r][k] += s[k].get();
         }
       }
     }
@@ -390,10 +442,10 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
         FxSum<2> s;  // 6 2^(60 + 60 - 64 + 2) < 2^60.6
 #pragma unroll
         for (int f = 0; f < 6; ++f) s.add(c[f], fx_split(Fs[k * 6 * n2 + at[f]]));
-        const int pV = a.ops->fxH_bits - 3 - (k == 0 ? eM : k < 4 ? eV : eE) - eJm;
-        const int pS = a.ops->fxL_bits + 60 - 64 + 2 - fx_exp(fin[6 + (k == 0 ? 0 : k < 4 ? 1 : 2)]);
+        const int pV = a.ops->fxH_bits - 3 - eR[k];
+        const int pS = a.ops->fxL_bits + 60 - 64 + 2 - fx_exp(fin[15 + k]);
         const int p = min(pV, pS);
-        sum[r][k] = fx_to((acc[r][k] >> min(pV - p, 63)) + (s.get() >> min(pS - p, 63)), p);
+        sum[r][k] = fx_to(fx_shr(acc[r][k], min(pV - p, 62)) + fx_shr(s.get(), min(pS - p, 62)), p);
       }
     }
     finish_node64<n, MODE, true>(a, e, er.ce, v, sum[r]);
