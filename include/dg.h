@@ -259,13 +259,14 @@ int dg_set_sponge(dg_ctx* ctx, const double* sigma, const double* U_base);
 /* Autotuner of the stage kernels' launch configuration (the paper plans
    launch-configuration tuning, Sec. 3.3; this is the library's own).  Times
    every launch variant on the context's current state and keeps the fastest:
-   elements per thread block of the lifting and volume kernels (the default,
-   about 256 threads, or twice as many elements), the volume kernel's thread
-   form of the line sums (FP64: 64-bit fixed point, or FP64 sums per
-   node) and the side kernels' block size (128 or 256 threads).  In the
+   elements per thread block of the lifting and volume kernels (the default D,
+   about 256 threads and fewer elements on meshes that would leave
+   multiprocessors idle, or always 2 D), the form of the volume kernel's line
+   sums (FP64: 64-bit fixed point, or FP64 sums per node) and the side kernels'
+   block size (128, or 256 with fewer threads on such meshes).  In the
    two-kernel FP32-bulk stage (see dg_stage_form) the volume entries apply to
    its element kernel and the side entry to its side kernel.  Only scratch
-   arrays are written; the state is unchanged.  config (may be NULL, 6 ints,
+   arrays are written; the state is unchanged.  config (may be NULL, 7 ints,
    as in dg_set_config).  ms (may be NULL, 8 doubles): mean time per launch
    of each variant (-1 where a variant does not exist), in the order lift D,
    lift 2D, volume D default mapping, volume D other mapping, volume 2D
@@ -277,8 +278,12 @@ int dg_set_sponge(dg_ctx* ctx, const double* sigma, const double* U_base);
 int dg_autotune(dg_ctx* ctx, int* config, double* ms);
 
 /* Sets or reads back the launch configuration, 7 ints: lift elements per
-   block, volume elements per block, FP64's fixed-point sums (1) or FP64 sums per node (0), side
-   block size (0 / -1 entries select the defaults), the FP32-bulk stage form
+   block, volume elements per block, FP64's fixed-point sums (1) or FP64 sums
+   per node (0), side block size (0 / -1 entries select the defaults, which
+   read back as D, D, 1 in FP64 and 0 in FP32-bulk, and 256).  The default
+   sizes D and 256 are upper limits: kernels that gain by it launch smaller
+   blocks on meshes that would leave multiprocessors idle; 2 D and 128 are
+   launched as given on every mesh.  Then the FP32-bulk stage form
    (0: the two-kernel stage where it applies, else four kernels; 1: always
    the four-kernel stage), the two-kernel stage's L2 prefetch of the next
    wave's element data (1 on, the default; 0 off) and its launch form (0:

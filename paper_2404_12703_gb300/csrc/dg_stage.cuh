@@ -1318,7 +1318,7 @@ inline size_t lift_smem_bytes() {
 }
 
 // Launch variants the autotuner chooses among: the default elements per
-// block D and 2D (lifting up to 1024 nodes, volume up to 512), and for FP64
+// block D (fewer on small meshes: fx_epb, felem_variant) and 2D (lifting up to 1024 nodes, volume up to 512), and for FP64
 // the volume kernel's two forms (fixed point, or FP64 sums per node).
 template <int N, typename T>
 struct Variants {
@@ -1342,17 +1342,19 @@ inline int sm_count() {
   }
   return sms;
 }
-// Threads per block of the side kernels: the configured 128 or 256, halved
-// while the grid would leave SMs without two blocks.  A block's side nodes
+// Threads per block of the side kernels: 128 where that is configured, else
+// 256, halved while the grid would leave SMs without two blocks.  A block's side nodes
 // share one SM's units: at 4^3 elements, N = 3, 256-thread blocks put the
 // 3,072 side nodes on 12 of 152 SMs (FP64 flux kernel 26.3 us, 32-thread
 // blocks 16.4 us).
 inline int side_threads(int block, int64_t nodes) {
-  int b = block == 128 ? 128 : 256;
+  if (block == 128) return 128;
+  int b = 256;
   while (b > 32 && (nodes + b - 1) / b < 2 * sm_count()) b /= 2;
   return b;
 }
-// Elements per block of the fixed-point kernels: E, fewer while the grid
+// Elements per block of the fixed-point kernels where none are configured (or
+// the default D is): E = D, fewer while the grid
 // would leave SMs without two blocks (the elements of a block share one
 // SM's units; 4^3 elements at N = 3 in blocks of four used 16 of 152 SMs).
 // At N = 1 four elements share a warp.
@@ -1369,7 +1371,7 @@ template <int N, typename T, int E>
 inline void launch_lift(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
   if constexpr (sizeof(T) == sizeof(double)) {
-    const int epb = fx_epb<N>(S::EPB, a.E);
+    const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E) : S::EPB;
     StageArgs b = a;
     b.prefetch = fx_wave(Fix<N>::TPE * epb);
     k_lift_fx<N><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, LiftFix<N>::bytes(epb), st>>>(b);
@@ -1377,12 +1379,12 @@ inline void launch_lift(const StageArgs& a, cudaStream_t st) {
     k_lift<N, T, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, lift_smem_bytes<N, T, E>(), st>>>(a);
   }
 }
-// FX: the fixed-point form (FP64)
+// FX: the fixed-point form (FP64); E = 0: the default elements per block
 template <int N, int MODE, typename T, int E, bool FX>
 inline void launch_vol(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
   if constexpr (FX) {
-    const int epb = fx_epb<N>(S::EPB, a.E);
+    const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E) : S::EPB;
     const unsigned nb = (unsigned)((a.E + epb - 1) / epb);
     StageArgs b = a;
     b.prefetch = fx_wave(Fix<N>::TPE * epb);
@@ -1629,14 +1631,14 @@ constexpr bool felem_single() {
 template <int N>
 inline void felem_variant(const StageArgs& a, int mode, int epb, int prefetch, cudaStream_t st) {
   using V = Variants<N, float>;
+  if constexpr (V::vol2) {
+    if (mode != 0 && epb == 2 * V::D) return launch_felem<N, 1, 2 * V::D>(a, prefetch, st);
+  }
   if constexpr (felem_single<N>()) {
     if ((a.E + V::D - 1) / V::D < sm_count())
       return mode == 0 ? launch_felem<N, 0, 1>(a, 0, st) : launch_felem<N, 1, 1>(a, prefetch, st);
   }
   if (mode == 0) return launch_felem<N, 0, 0>(a, 0, st);
-  if constexpr (V::vol2) {
-    if (epb == 2 * V::D) return launch_felem<N, 1, 2 * V::D>(a, prefetch, st);
-  }
   launch_felem<N, 1, 0>(a, prefetch, st);
 }
 
@@ -1806,10 +1808,10 @@ cudaError_t stage_autotune_fused(dg_ctx* c, double* ms) {
     ms[6] = timed([&] { launch_fflux<N>(a, 256, st); });
     ms[7] = timed([&] { launch_fflux<N>(a, 128, st); });
     best.side_block = ms[7] < ms[6] ? 128 : 256;
-    ms[2] = timed([&] { launch_felem<N, 1, 0>(a, pf, st); });
+    ms[2] = timed([&] { felem_variant<N>(a, 1, V::D, pf, st); });  // (what a step launches)
     best.vol_epb = V::D;
     if constexpr (V::vol2) {
-      ms[4] = timed([&] { launch_felem<N, 1, 2 * V::D>(a, pf, st); });
+      ms[4] = timed([&] { felem_variant<N>(a, 1, 2 * V::D, pf, st); });
       if (ms[4] < ms[2]) best.vol_epb = 2 * V::D;
     }
     e = cudaGetLastError();
