@@ -33,9 +33,13 @@ __device__ __forceinline__ void radii_up(const double U[5], const double M[10], 
   const float ri = e / mag_lo(U[0]) + kTiny;
   const float m0 = cut(U[1]), m1 = cut(U[2]), m2 = cut(U[3]);
   const float s2 = m0 * m0 + m1 * m1 + m2 * m2;
-  const float k2 = 0.5f * s2 * ri;  // the kinetic energy, at most 2e-5 of it above (or any amount below)
+  // The kinetic energy, at most 2e-5 of it above (or any amount below): 3e-5 of
+  // it are left for the rounding of the difference, 6e-8 of the energy where
+  // that is not the larger by far, and else within e of the difference.
+  const float k2 = 0.5f * s2 * ri;
   const float p = fmaf(e * gm1, mag_up(U[4]) - k2 * (1.0f - 5e-5f), kTiny);
-  const bool positive = U[0] > 0.0 && U[4] > 0.0 && mag_lo(U[4]) > e * mul_up(s2 + kTiny, ri);
+  // cutting the momentum takes 2e-6 of its square, e in 1 / rho adds 1e-5
+  const bool positive = U[0] > 0.0 && U[4] > 0.0 && mag_lo(U[4]) > 0.5f * e * mul_up(s2 + kTiny, ri);
   const float c = positive ? e * sqrtf(mul_up(mul_up(e * gamma, p), ri)) : __int_as_float(0x7f800000);
   float a = 0.0f;
 #pragma unroll
@@ -61,7 +65,10 @@ __device__ __forceinline__ void radii_up(const double U[5], const double M[10], 
 // alone.  T = double: bound by the FP64 unit (a division, a square root and
 // some thirty operations per node), so with PRUNE a node is evaluated only if
 // its upper bound exceeds the block's largest radius so far; the maximum is the
-// same (24^3 elements, N = 7: 610 -> 219 us per step).
+// same (24^3 elements, N = 7: 616 -> 223 us per call, 346 at Ma = 3; where all
+// radii are equal to 1e-5, uniform flow on a uniform mesh, 708: letting the
+// bound rest after eight nodes it did not spare takes 657 there but 235 and 390
+// on the flows).
 template <int N, typename T, bool PRUNE = false>
 __global__ void __launch_bounds__(256) k_cfl(int E, const double* __restrict__ U, const double* __restrict__ metric,
                                             const float* __restrict__ metric32, const double* __restrict__ geo,
@@ -98,7 +105,7 @@ __global__ void __launch_bounds__(256) k_cfl(int E, const double* __restrict__ U
         float ua, ub;
         radii_up(Uv, M, G, (float)gamma, (float)gm1, (float)Rinv, (float)kv, sutherland, (float)inv_Tref, ua, ub);
         const float ca = __int_as_float(*(volatile int*)&sc), cb = __int_as_float(*(volatile int*)&sv);
-        if (ua < ca && (!viscous || ub < cb)) continue;
+        if (ua < ca && (!viscous || kv == 0.0 || ub < cb)) continue;  // (kv = 0: every bb is zero)
       }
       cfl_radii(Uv, M, G, gamma, gm1, Rinv, kv, sutherland, inv_Tref, aa, bb);
       if (PRUNE) {
