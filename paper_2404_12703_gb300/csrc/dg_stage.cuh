@@ -334,7 +334,8 @@ __device__ __forceinline__ Prim64 prim64(const double U[5], double ri, double p)
 // Roe's flux through the unit normal n (no entropy fix)
 __device__ __forceinline__ void roe_flux64(const Prim64& L, const Prim64& R, double HL, double HR, const double n[3],
                                            double gm1, double f[5]) {
-  const double z = sqrt(R.rho * L.ri), inv = 1.0 / (1.0 + z);
+  // (NaN for a negative density on either side, as from the square roots of both)
+  const double z = __double2hiint(L.rho) < 0 ? __longlong_as_double(-1LL) : sqrt(R.rho * L.ri), inv = 1.0 / (1.0 + z);
   const double u = (L.u + z * R.u) * inv, v = (L.v + z * R.v) * inv, w = (L.w + z * R.w) * inv;
   const double H = (HL + z * HR) * inv, hq = 0.5 * (u * u + v * v + w * w), c2 = gm1 * (H - hq);
   const double y = rsqrt(c2), c = c2 * y, c2i = y * y;
