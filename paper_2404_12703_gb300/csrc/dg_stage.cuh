@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(256) k_surf_prims(StageArgs a) {
   T qa[4];
   if (brow >= 0) {
     bc_lift_value<T>(a, cp, brow, UM, qM, nu, qa);  // boundary side: the condition's value
-  } else {
+  } else if constexpr (sizeof(T) == sizeof(float)) {
     int ps, qs;
     flip_to_slave<n>(flip, p, q, ps, qs);
     const int vS = face_vol_node<n>(fS, ps, qs);
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == sizeof(float) ? 4 : 1) k_sur
       for (int k = 0; k < 12; ++k) gM[k] = T(0);
     }
     bc_flux<T>(a, cp, brow, UM, qM, gM, nu, sA, sn, f);
-  } else {
+  } else if constexpr (sizeof(T) == sizeof(float)) {
     int ps, qs;
     flip_to_slave<n>(flip, p, q, ps, qs);
     const int vS = face_vol_node<n>(fS, ps, qs);
