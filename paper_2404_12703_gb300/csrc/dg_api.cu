@@ -548,6 +548,13 @@ void dg_destroy(dg_ctx* c) {
 
 }  // extern "C"
 
+// the current device and its number of multiprocessors
+static void set_device(dg_ctx* c) {
+  cudaGetDevice(&c->device);
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess && sms > 0) c->sms = sms;
+}
+
 namespace dg {
 
 // A serving pool: the arrays of a context sized for capE elements and 3 capE
@@ -556,7 +563,7 @@ int create_pool_ctx(dg_ctx** out, int N, int64_t capE, const dg_params* params, 
                     std::string& msg) {
   *out = nullptr;
   dg_ctx* c = new dg_ctx();
-  cudaGetDevice(&c->device);
+  set_device(c);
   c->stream = stream;
   c->prm = *params;
   c->N = N;
@@ -657,7 +664,7 @@ int init_mesh_impl(dg_ctx** out, const dg_mesh_desc* mesh, const dg_params* para
   if (mesh->nodes == DG_NODES_GAUSS && params->shock_capturing)
     return fail(DG_ERR_ARG, "shock capturing needs LGL nodes (the sub-cell FV scheme lives on the LGL sub-cells)");
   dg_ctx* c = new dg_ctx();
-  cudaGetDevice(&c->device);
+  set_device(c);
   c->stream = stream;
   c->pool_stream = pool_stream;
   c->gauss = mesh->nodes == DG_NODES_GAUSS;

@@ -481,14 +481,9 @@ cudaError_t launch_refs(dg_ctx* c) {
   return cudaGetLastError();
 }
 
-static int sm_count_of(const dg_ctx* c) {
-  int sms = 148;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  return sms;
-}
 static int cfl_blocks(dg_ctx* c) {
   const int64_t need = (c->E * c->n3 + 255) / 256;
-  return (int)std::min<int64_t>(need, (int64_t)sm_count_of(c) * 8);
+  return (int)std::min<int64_t>(need, (int64_t)c->sms * 8);
 }
 
 cudaError_t launch_cfl(dg_ctx* c, bool report_only) {
@@ -499,7 +494,7 @@ cudaError_t launch_cfl(dg_ctx* c, bool report_only) {
   // N = 7: one / two / eight blocks per SM 330 / 219 / 262 us; 12^3: 72 / 63 /
   // 95).  Below that the bounds cost more than they spare (9 x 7 x 5, N = 6:
   // 24 us without, 27 with).
-  const int nb2 = 2 * sm_count_of(c);
+  const int nb2 = 2 * c->sms;
   prof_begin(c, PK_CFL);
   if (c->prm.precision == DG_FP32_BULK) {
     DG_DISPATCH(c->N, (k_cfl<NN, float><<<nb, 256, 0, c->stream>>>((int)c->E, c->U, c->metric, c->metric32, c->cflgeo,

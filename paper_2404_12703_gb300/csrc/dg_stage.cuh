@@ -1236,6 +1236,7 @@ namespace dg {
 // ---------------------------------------------------------------------------
 inline StageArgs make_stage_args(dg_ctx* c, const double* U) {
   StageArgs a{};
+  a.sms = c->sms;
   a.E = (int)c->E;
   a.S = (int)c->S;
   a.U = U;
@@ -1332,26 +1333,15 @@ struct Variants {
 
 // the kernels' code for shock capturing, a sponge or a source is needed
 inline bool extras(const StageArgs& a) { return a.shock || a.sponge_sigma || a.source; }
-// SMs of the current device
-inline int sm_count() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms <= 0)
-      sms = 152;
-  }
-  return sms;
-}
 // Threads per block of the side kernels: 128 where that is configured, else
 // 256, halved while the grid would leave SMs without two blocks.  A block's side nodes
 // share one SM's units: at 4^3 elements, N = 3, 256-thread blocks put the
 // 3,072 side nodes on 12 of 152 SMs (FP64 flux kernel 26.3 us, 32-thread
 // blocks 16.4 us).
-inline int side_threads(int block, int64_t nodes) {
+inline int side_threads(int block, int64_t nodes, int sms) {
   if (block == 128) return 128;
   int b = 256;
-  while (b > 32 && (nodes + b - 1) / b < 2 * sm_count()) b /= 2;
+  while (b > 32 && (nodes + b - 1) / b < 2 * sms) b /= 2;
   return b;
 }
 // Elements per block of the fixed-point kernels where none are configured (or
@@ -1360,21 +1350,21 @@ inline int side_threads(int block, int64_t nodes) {
 // SM's units; 4^3 elements at N = 3 in blocks of four used 16 of 152 SMs).
 // At N = 1 four elements share a warp.
 template <int N>
-inline int fx_epb(int E, int64_t elems) {
+inline int fx_epb(int E, int64_t elems, int sms) {
   const int least = Fix<N>::TPE < 32 ? 32 / Fix<N>::TPE : 1;
-  while (E > least && (elems + E - 1) / E < 2 * sm_count()) E = std::max(least, E / 2 / least * least);
+  while (E > least && (elems + E - 1) / E < 2 * sms) E = std::max(least, E / 2 / least * least);
   return E;
 }
 // the prefetch distance in blocks: about the blocks the GPU holds at once
 // (128 registers per thread)
-inline int fx_wave(int threads) { return sm_count() * std::max(1, 512 / threads); }
+inline int fx_wave(int threads, int sms) { return sms * std::max(1, 512 / threads); }
 template <int N, typename T, int E>
 inline void launch_lift(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
   if constexpr (sizeof(T) == sizeof(double)) {
-    const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E) : S::EPB;
+    const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E, a.sms) : S::EPB;
     StageArgs b = a;
-    b.prefetch = fx_wave(Fix<N>::TPE * epb);
+    b.prefetch = fx_wave(Fix<N>::TPE * epb, a.sms);
     k_lift_fx<N><<<(unsigned)((a.E + epb - 1) / epb), Fix<N>::TPE * epb, LiftFix<N>::bytes(epb), st>>>(b);
   } else {
     k_lift<N, T, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, lift_smem_bytes<N, T, E>(), st>>>(a);
@@ -1385,10 +1375,10 @@ template <int N, int MODE, typename T, int E, bool FX>
 inline void launch_vol(const StageArgs& a, cudaStream_t st) {
   using S = Shape<N, E>;
   if constexpr (FX) {
-    const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E) : S::EPB;
+    const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E, a.sms) : S::EPB;
     const unsigned nb = (unsigned)((a.E + epb - 1) / epb);
     StageArgs b = a;
-    b.prefetch = fx_wave(Fix<N>::TPE * epb);
+    b.prefetch = fx_wave(Fix<N>::TPE * epb, a.sms);
     if (extras(a)) k_volume_fx<N, MODE, true><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
     else k_volume_fx<N, MODE, false><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
   } else {
@@ -1405,7 +1395,7 @@ inline void launch_vol(const StageArgs& a, cudaStream_t st) {
 template <int N, typename T, bool GL = false>
 inline void launch_side(const StageArgs& a, int block, cudaStream_t st, bool prims) {
   const int64_t side_nodes = (int64_t)a.S * Shape<N>::n2;
-  const int b = side_threads(block, side_nodes);
+  const int b = side_threads(block, side_nodes, a.sms);
   const unsigned g = (unsigned)((side_nodes + b - 1) / b);
   if (prims) k_surf_prims<N, T, GL><<<g, b, 0, st>>>(a);
   else if (sizeof(T) == sizeof(float) || a.viscous) k_surf_flux<N, T, GL, true><<<g, b, 0, st>>>(a);
@@ -1603,7 +1593,7 @@ inline void launch_felem(StageArgs a, int prefetch, cudaStream_t st) {
 template <int N>
 inline void launch_fflux(const StageArgs& a, int block, cudaStream_t st) {
   const int64_t side_nodes = (int64_t)a.S * Shape<N>::n2;
-  const int b = side_threads(block, side_nodes);
+  const int b = side_threads(block, side_nodes, a.sms);
   k_fflux<N><<<(unsigned)((side_nodes + b - 1) / b), b, 0, st>>>(a);
 }
 // face data of state U: every element of the context (a serving pool: its
@@ -1636,7 +1626,7 @@ inline void felem_variant(const StageArgs& a, int mode, int epb, int prefetch, c
     if (mode != 0 && epb == 2 * V::D) return launch_felem<N, 1, 2 * V::D>(a, prefetch, st);
   }
   if constexpr (felem_single<N>()) {
-    if ((a.E + V::D - 1) / V::D < sm_count())
+    if ((a.E + V::D - 1) / V::D < a.sms)
       return mode == 0 ? launch_felem<N, 0, 1>(a, 0, st) : launch_felem<N, 1, 1>(a, prefetch, st);
   }
   if (mode == 0) return launch_felem<N, 0, 0>(a, 0, st);
@@ -1692,9 +1682,9 @@ cudaError_t stage_launch_gl(dg_ctx* c, const double* U, int mode, double rkA, do
   if (a.E == 0) return cudaSuccess;
   const unsigned nb = (unsigned)((a.E + S::EPB - 1) / S::EPB);
   constexpr bool fx = sizeof(T) == sizeof(double);  // the fixed-point kernels
-  const int epb = fx_epb<N>(S::EPB, a.E);
+  const int epb = fx_epb<N>(S::EPB, a.E, a.sms);
   const unsigned nbx = (unsigned)((a.E + epb - 1) / epb);
-  if (fx) a.prefetch = fx_wave(Fix<N>::TPE * epb);
+  if (fx) a.prefetch = fx_wave(Fix<N>::TPE * epb, a.sms);
   const int sb = c->cfg.side_block;
   prof_begin(c, PK_SURF_PRIMS);
   k_prolong_gl<N><<<nb, S::THREADS, gl_prolong_smem<N>(), c->stream>>>(a);

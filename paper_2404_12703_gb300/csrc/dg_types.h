@@ -109,6 +109,7 @@ struct StageConfig {
 // Per-stage launch parameters of the RHS kernels.
 struct StageArgs {
   int E, S;
+  int sms;               // multiprocessors of the context's device (launch shapes; host only)
   const double* U;       // [E][5][n3] internal state
   const double* metric;  // [E][10][n3]: J a^d_c at d*3+c, then 1/J
   const float* metric32;  // the same, rounded to FP32 (FP32-bulk)
@@ -190,7 +191,7 @@ struct StageArgs {
 }  // namespace dg
 
 struct dg_ctx {
-  int device = 0;
+  int device = 0, sms = 152;  // and its multiprocessors
   cudaStream_t stream = nullptr;      // user stream: all work is ordered on it
   cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
   cudaStream_t pool_stream = nullptr;  // non-null: arrays from the library pool, in this stream's order
