@@ -262,24 +262,24 @@ int dg_set_sponge(dg_ctx* ctx, const double* sigma, const double* U_base);
    elements per thread block of the lifting and volume kernels (the default D,
    about 256 threads and fewer elements on meshes that would leave
    multiprocessors idle, or always 2 D), the form of the volume kernel's line
-   sums (FP64: 64-bit fixed point, or FP64 sums per node) and the side kernels'
+   sums (FP64: 64-bit fixed point, or FP64 sums) and the side kernels'
    block size (128, or 256 with fewer threads on such meshes).  In the
    two-kernel FP32-bulk stage (see dg_stage_form) the volume entries apply to
    its element kernel and the side entry to its side kernel.  Only scratch
    arrays are written; the state is unchanged.  config (may be NULL, 7 ints,
    as in dg_set_config).  ms (may be NULL, 8 doubles): mean time per launch
    of each variant (-1 where a variant does not exist), in the order lift D,
-   lift 2D, volume D default mapping, volume D other mapping, volume 2D
+   lift 2D, volume D default form, volume D other form, volume 2D
    default, volume 2D other, side kernels at 256, at 128.  Synchronises.
-   Elements per block change no arithmetic; the volume mapping changes the
-   summation order of the split-form sums (both within the FP64 parity).
+   Elements per block change no arithmetic; the form of the sums changes their
+   rounding (both within the FP64 parity).
    DG_ERR_STATE on Gauss-Legendre nodes (their kernels have one launch
    configuration). */
 int dg_autotune(dg_ctx* ctx, int* config, double* ms);
 
 /* Sets or reads back the launch configuration, 7 ints: lift elements per
-   block, volume elements per block, FP64's fixed-point sums (1) or FP64 sums
-   per node (0), side block size (0 / -1 entries select the defaults, which
+   block, volume elements per block, the FP64 volume kernel's sums in fixed
+   point (1) or in FP64 (0), side block size (0 / -1 entries select the defaults, which
    read back as D, D, 1 in FP64 and 0 in FP32-bulk, and 256).  The default
    sizes D and 256 are upper limits: kernels that gain by it launch smaller
    blocks on meshes that would leave multiprocessors idle; 2 D and 128 are

@@ -1206,8 +1206,8 @@ int dg_set_config(dg_ctx* c, const int* config) {
   const int ps = config[6];
   if (!(le == 0 || le == D || (lift2 && le == 2 * D))) return fail(DG_ERR_ARG, "lift elements per block");
   if (!(ve == 0 || ve == D || (vol2 && ve == 2 * D))) return fail(DG_ERR_ARG, "volume elements per block");
-  if (!(pr == -1 || pr == 0 || pr == 1)) return fail(DG_ERR_ARG, "volume mapping");
-  if (pr == 1 && c->prm.precision == DG_FP32_BULK) return fail(DG_ERR_ARG, "line pairs are an FP64 mapping");
+  if (!(pr == -1 || pr == 0 || pr == 1)) return fail(DG_ERR_ARG, "form of the volume kernel's sums (-1, 0 or 1)");
+  if (pr == 1 && c->prm.precision == DG_FP32_BULK) return fail(DG_ERR_ARG, "the form of the volume kernel's sums is an FP64 choice");
   if (!(sb == 0 || sb == 128 || sb == 256)) return fail(DG_ERR_ARG, "side block size");
   if (!(sf == 0 || sf == 1)) return fail(DG_ERR_ARG, "stage form (0: default, 1: four kernels)");
   if (!(pf == 0 || pf == 1)) return fail(DG_ERR_ARG, "prefetch (0 or 1)");

@@ -1047,7 +1047,7 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     }
     fx_reduce<N, VQ_N>(m, red, fin, t);
     bool plain = true, out = false;
-    if (t < 32) out = vol_bad<N>(fin, t);
+    if (t < 32) out = a.sums64 || vol_bad<N>(fin, t);
     if (t < 3) plain = vol_scale(*sc, fin, a.ops, t, out);
     __syncwarp();
     if (t < 3) vol_align(*sc, t);

@@ -650,7 +650,7 @@ struct CoefOfStage {
 // the kernel keeps its registers: k_felem<7, 1> spills 8 bytes instead of 80,
 // k_felem<5, 1> none instead of 40 (24^3 elements, N = 7: 995 -> 939 us per launch).
 template <int N, int MODE, int EPB_, bool EXTRA>
-__global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::template vol_min_blocks<float>())
+__global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::vol_min_blocks())
     k_felem(StageArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const unsigned blk = blockIdx.x;
@@ -728,7 +728,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned expected, i
 }
 
 template <int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS, Shape<N>::template vol_min_blocks<float>())
+__global__ void __launch_bounds__(Shape<N>::THREADS, Shape<N>::vol_min_blocks())
     k_fpersist(StageArgs a, PersistArgs p) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const unsigned expected = gridDim.x + p.expect_extra;

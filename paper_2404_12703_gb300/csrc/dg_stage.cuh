@@ -47,12 +47,9 @@ struct Shape {
   static constexpr int EPB_DEFAULT = n3 >= 256 ? 1 : 256 / n3;
   static constexpr int EPB = EPB_ > 0 ? EPB_ : EPB_DEFAULT;  // elements per block
   static constexpr int THREADS = EPB * n3;
-  // FP32-bulk volume kernel: at least 1024 resident threads per SM (it is
-  // latency-bound); the FP64 one is bound by the FP64 pipe at one block
-  template <typename T>
-  static constexpr int vol_min_blocks() {
-    return sizeof(T) == sizeof(float) && THREADS <= 512 ? 1024 / THREADS : 1;
-  }
+  // FP32-bulk volume and element kernels: at least 1024 resident threads per
+  // SM (they are latency-bound)
+  static constexpr int vol_min_blocks() { return THREADS <= 512 ? 1024 / THREADS : 1; }
 };
 
 // buffers of the arithmetic type T
@@ -859,61 +856,59 @@ __device__ __noinline__ double element_alpha(double* sT1, double* sT2, double* s
   return sT2[0];
 }
 
-// shared-memory layout of k_volume: FP64 part first, then the T arrays
-template <int N, typename T, int EPB_ = 0>
+// shared-memory layout of k_volume: FP64 part first, then the FP32 arrays:
+// node-major primitives (float4 + float2) and metrics (one float4 per
+// direction), so a partner is read with three loads
+template <int N, int EPB_ = 0>
 struct VolumeSmem {
   using S = Shape<N, EPB_>;
-  // FP32: node-major primitives (float4 + float2) and metrics (one float4 per
-  // direction), so a partner is read with three loads
-  static constexpr bool aos = sizeof(T) == sizeof(float);
   static constexpr int n2p = (S::n2 + 3) & ~3;
-  static constexpr int nJ = aos ? 12 : 9;
-  // Vinv, indicator scratch, FP32: the node's state and RK register copied in
-  // asynchronously (even count: the T arrays start 16-byte aligned)
-  static constexpr int nUd = aos ? 10 * S::n3 : 0;
+  static constexpr int nJ = 12;
+  // Vinv, indicator scratch, the node's state and RK register copied in
+  // asynchronously (even count: the FP32 arrays start 16-byte aligned)
+  static constexpr int nUd = 10 * S::n3;
   static constexpr size_t n_dbl = (S::n2 + S::EPB * (2 * S::n3 + 4 * S::n2 + nUd) + 1) & ~size_t(1);
-  // a node plane: FP32 pads every line of n nodes by one, so that the four
-  // lines along the first direction that a warp holds at N = 7 fall in
-  // distinct banks (16 x 8 x 16 channel, N = 7: 125 -> 121 us per launch)
-  static constexpr int Pn = aos ? S::n3 + S::n2 : S::n3;
-  // per-element stride of the primitives: a multiple of 4 floats in FP32, so
-  // that every element's float4 view starts 16-byte aligned
-  static constexpr int pstride = aos ? 6 * ((Pn + 3) & ~3) : 6 * Pn;
-  // viscous / FV fluxes: FP32 keeps the four viscous components of a node in
-  // one float4 (element stride padded like the primitives)
+  // a node plane: every line of n nodes padded by one, so that the four lines
+  // along the first direction that a warp holds at N = 7 fall in distinct
+  // banks (16 x 8 x 16 channel, N = 7: 125 -> 121 us per launch)
+  static constexpr int Pn = S::n3 + S::n2;
+  // per-element stride of the primitives: a multiple of 4 floats, so that
+  // every element's float4 view starts 16-byte aligned
+  static constexpr int pstride = 6 * ((Pn + 3) & ~3);
+  // viscous / FV fluxes: the four viscous components of a node in one float4
+  // (element stride padded like the primitives)
   static constexpr int gfv = 5 * ((S::n3 + 3) & ~3);
-  static constexpr int gstride = aos ? (gfv > 4 * Pn ? gfv : 4 * Pn) : 5 * S::n3;
+  static constexpr int gstride = gfv > 4 * Pn ? gfv : 4 * Pn;
   static constexpr size_t n_t = 2 * n2p + S::EPB * (pstride + nJ * Pn + gstride);
-  static constexpr size_t bytes = sizeof(double) * n_dbl + sizeof(T) * n_t;
+  static constexpr size_t bytes = sizeof(double) * n_dbl + sizeof(float) * n_t;
 };
 
 // ---------------------------------------------------------------------------
 // Volume integral + SurfInt + ApplyJac (+ RK update)
 // ---------------------------------------------------------------------------
-// One node per thread, which sums over all its partners: FP32-bulk, and FP64's
-// other mapping (dg_set_config; the default FP64 kernel is k_volume_fx in
-// dg_fixed64.cuh).
+// FP32-bulk (FP64: k_volume_fx in dg_fixed64.cuh): one node per thread, which
+// sums over all its partners.
 // EXTRA: a run with shock capturing, a sponge or a source; without their code
 // the FP32 kernel takes 114 instead of 117 us (16 x 8 x 16 channel, N = 7).
-template <int N, int MODE, typename T, int EPB_, bool EXTRA>
-__global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::template vol_min_blocks<T>())
+template <int N, int MODE, int EPB_, bool EXTRA>
+__global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::vol_min_blocks())
     k_volume(StageArgs a) {
   using S = Shape<N, EPB_>;
+  using T = float;
   constexpr int n = S::n, n2 = S::n2, n3 = S::n3, EPB = S::EPB;
   extern __shared__ __align__(16) unsigned char smraw[];
-  using L = VolumeSmem<N, T, EPB_>;
-  constexpr bool aos = L::aos;
+  using L = VolumeSmem<N, EPB_>;
   constexpr int Pn = L::Pn;
-  auto px = [](int node) { return aos ? node + node / n : node; };  // its plane index
+  auto px = [](int node) { return node + node / n; };  // its plane index
   double* sVi = reinterpret_cast<double*>(smraw);  // [n2] Vinv (FP64)
   double* sX = sVi + n2;                           // [EPB][2 n3 + 4 n2] indicator scratch (FP64)
   T* sDs = reinterpret_cast<T*>(reinterpret_cast<double*>(smraw) + L::n_dbl);  // [n2] Dsplit
   T* sDh = sDs + L::n2p;                                                       // [n2] Dhat
-  T* sP = sDh + L::n2p;                  // [EPB][6][n3] rho u v w p' H', halved (FP32: [n3] float4 + [n3] float2)
-  T* sJ = sP + EPB * L::pstride;         // [EPB][9][n3] metrics, halved (FP32: [3][n3] float4)
-  T* sG = sJ + EPB * L::nJ * Pn;         // [EPB][5][n3] viscous / FV fluxes (FP32 viscous: [n3] float4)
+  T* sP = sDh + L::n2p;                  // [EPB] rho u v w p' H', halved ([Pn] float4 + [Pn] float2)
+  T* sJ = sP + EPB * L::pstride;         // [EPB] metrics, halved ([3][Pn] float4)
+  T* sG = sJ + EPB * L::nJ * Pn;         // [EPB] viscous ([Pn] float4) / FV fluxes ([5][n3])
   const int le = threadIdx.x / n3, t = threadIdx.x % n3;
-  double* sUd = sX + EPB * (2 * n3 + 4 * n2) + le * L::nUd;  // FP32: [2][5][n3] U and dU of the element
+  double* sUd = sX + EPB * (2 * n3 + 4 * n2) + le * L::nUd;  // [2][5][n3] U and dU of the element
   // slots past the last element redo the last element, free slots of a
   // serving pool compute on what they hold; neither stores (see k_lift)
   const int ei = blockIdx.x * EPB + le < a.E ? blockIdx.x * EPB + le : a.E - 1;
@@ -934,15 +929,11 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   T* Jm = sJ + le * L::nJ * Pn;
   T* G = sG + le * L::gstride;
   float4* G4 = reinterpret_cast<float4*>(G);
-  // FP32 views of the same memory
   float4* P4 = reinterpret_cast<float4*>(P);
   float2* P2 = reinterpret_cast<float2*>(P + 4 * Pn);
   float4* J4 = reinterpret_cast<float4*>(Jm);
   // halved metric component c of direction d at a node
-  auto Jc = [&](int d, int c, int node) -> T {
-    if constexpr (aos) return reinterpret_cast<const float*>(J4 + d * Pn + px(node))[c];
-    else return Jm[(d * 3 + c) * n3 + node];
-  };
+  auto Jc = [&](int d, int c, int node) -> T { return reinterpret_cast<const float*>(J4 + d * Pn + px(node))[c]; };
   const double H_ref = cp.Hr;
   double U[5];
   double p_full;
@@ -950,44 +941,28 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   T g[12];
   {
     const double* u = a.U + (size_t)e * 5 * n3 + t;
-    if constexpr (aos) {
-      // the state now, the RK register (read only at the end) in a second group
+    // the state now, the RK register (read only at the end) in a second group
 #pragma unroll
-      for (int k = 0; k < 5; ++k) cp_async8(sUd + k * n3 + t, u + k * n3);
-      cp_async_commit();
-      if (MODE == 1 && !a.first_stage) {
-        const double* du = a.dU + (size_t)e * 5 * n3 + t;
+    for (int k = 0; k < 5; ++k) cp_async8(sUd + k * n3 + t, u + k * n3);
+    cp_async_commit();
+    if (MODE == 1 && !a.first_stage) {
+      const double* du = a.dU + (size_t)e * 5 * n3 + t;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) cp_async8(sUd + (5 + k) * n3 + t, du + k * n3);
-      }
-      cp_async_commit();
-      cp_async_wait<1>();
-#pragma unroll
-      for (int k = 0; k < 5; ++k) U[k] = sUd[k * n3 + t];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) U[k] = u[k * n3];
+      for (int k = 0; k < 5; ++k) cp_async8(sUd + (5 + k) * n3 + t, du + k * n3);
     }
+    cp_async_commit();
+    cp_async_wait<1>();
+#pragma unroll
+    for (int k = 0; k < 5; ++k) U[k] = sUd[k * n3 + t];
     me = shifted_prim<T, true>(U, a.gm1, a.Rinv, cp, &p_full);
     // halved values: every arithmetic mean of the two-point flux is then one
     // addition, bit-identical to (a + b) / 2
-    if constexpr (aos) {
-      P4[px(t)] = make_float4(0.5f * me.rho, 0.5f * me.u, 0.5f * me.v, 0.5f * me.w);
-      P2[px(t)] = make_float2(0.5f * me.p, 0.5f * me.H);
+    P4[px(t)] = make_float4(0.5f * me.rho, 0.5f * me.u, 0.5f * me.v, 0.5f * me.w);
+    P2[px(t)] = make_float2(0.5f * me.p, 0.5f * me.H);
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        J4[d * Pn + px(t)] = make_float4(0.5f * metric_at<T>(a, e, 3 * d, t, n3), 0.5f * metric_at<T>(a, e, 3 * d + 1, t, n3),
-                                     0.5f * metric_at<T>(a, e, 3 * d + 2, t, n3), 0.0f);
-    } else {
-      P[t] = T(0.5) * me.rho;
-      P[n3 + t] = T(0.5) * me.u;
-      P[2 * n3 + t] = T(0.5) * me.v;
-      P[3 * n3 + t] = T(0.5) * me.w;
-      P[4 * n3 + t] = T(0.5) * me.p;
-      P[5 * n3 + t] = T(0.5) * me.H;
-#pragma unroll
-      for (int c = 0; c < 9; ++c) Jm[c * n3 + t] = T(0.5) * metric_at<T>(a, e, c, t, n3);
-    }
+    for (int d = 0; d < 3; ++d)
+      J4[d * Pn + px(t)] = make_float4(0.5f * metric_at<T>(a, e, 3 * d, t, n3), 0.5f * metric_at<T>(a, e, 3 * d + 1, t, n3),
+                                       0.5f * metric_at<T>(a, e, 3 * d + 2, t, n3), 0.0f);
     if (a.viscous) {
       const T* pg = TBuf<T>::g(a) + (size_t)e * 12 * n3 + t;
 #pragma unroll
@@ -1009,17 +984,12 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
   // ---- split-form KEP volume integral, one node per thread over its partners ----
   {
     const int idl[3] = {t % n, (t / n) % n, t / n2};
-    // halved primitives and direction-d metrics of a node, either layout
+    // halved primitives and direction-d metrics of a node
     auto node = [&](int d, int v, T& r, T& u0, T& u1, T& u2, T& pp, T& H, T& j0, T& j1, T& j2) {
-      if constexpr (aos) {
-        const float4 a4 = P4[px(v)];
-        const float2 a2 = P2[px(v)];
-        const float4 jj = J4[d * Pn + px(v)];
-        r = a4.x, u0 = a4.y, u1 = a4.z, u2 = a4.w, pp = a2.x, H = a2.y, j0 = jj.x, j1 = jj.y, j2 = jj.z;
-      } else {
-        r = P[v], u0 = P[n3 + v], u1 = P[2 * n3 + v], u2 = P[3 * n3 + v], pp = P[4 * n3 + v], H = P[5 * n3 + v];
-        j0 = Jm[(d * 3) * n3 + v], j1 = Jm[(d * 3 + 1) * n3 + v], j2 = Jm[(d * 3 + 2) * n3 + v];
-      }
+      const float4 a4 = P4[px(v)];
+      const float2 a2 = P2[px(v)];
+      const float4 jj = J4[d * Pn + px(v)];
+      r = a4.x, u0 = a4.y, u1 = a4.z, u2 = a4.w, pp = a2.x, H = a2.y, j0 = jj.x, j1 = jj.y, j2 = jj.z;
     };
 #pragma unroll
     for (int d = 0; d < 3; ++d) {  // (unrolled: the partners' padded offsets are then constants)
@@ -1061,12 +1031,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
         const T nv[3] = {T(2) * Jc(d, 0, t), T(2) * Jc(d, 1, t), T(2) * Jc(d, 2, t)};
         T fv[4];
         viscous_flux_n(tau, W, nv, fv);
-        if constexpr (aos) {
-          G4[px(t)] = make_float4(fv[0], fv[1], fv[2], fv[3]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) G[k * n3 + t] = fv[k];
-        }
+        G4[px(t)] = make_float4(fv[0], fv[1], fv[2], fv[3]);
       }
       __syncwarp();
       __syncthreads();
@@ -1075,17 +1040,11 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
 #pragma unroll
         for (int al = 0; al < n; ++al) {
           const T c = sDh[id * n + al];
-          const int nb = base + al * str[d];
-          if constexpr (aos) {
-            const float4 gv = G4[px(nb)];
-            acc[1] -= c * gv.x;
-            acc[2] -= c * gv.y;
-            acc[3] -= c * gv.z;
-            acc[4] -= c * gv.w;
-          } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[1 + k] -= c * G[k * n3 + nb];
-          }
+          const float4 gv = G4[px(base + al * str[d])];
+          acc[1] -= c * gv.x;
+          acc[2] -= c * gv.y;
+          acc[3] -= c * gv.z;
+          acc[4] -= c * gv.w;
         }
       }
       __syncwarp();
@@ -1158,7 +1117,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
       }
     }
   }
-  if constexpr (aos) cp_async_wait<0>();
+  cp_async_wait<0>();
   if (!valid) return;
   // a serving case that finished or sits this step out keeps its state (its
   // surface fluxes were not formed this step)
@@ -1194,7 +1153,7 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     const double sg = a.sponge_sigma[(size_t)e * n3 + t];
     const double* ub = a.sponge_base + (size_t)e * 5 * n3 + t;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) Ut[k] -= sg * ((aos ? sUd[k * n3 + t] : U[k]) - ub[k * n3]);
+    for (int k = 0; k < 5; ++k) Ut[k] -= sg * (sUd[k * n3 + t] - ub[k * n3]);
   }
   if (EXTRA && a.source) {  // manufactured-solution source, FP64
     double Q[5];
@@ -1212,9 +1171,8 @@ __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::templ
     double* uo = a.Urk + (size_t)e * 5 * n3 + t;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      // FP32-bulk: the state and the RK register from the shared-memory copies
-      const double duk = aos ? sUd[(5 + k) * n3 + t] : du[k * n3];
-      const double uk = aos ? sUd[k * n3 + t] : U[k];
+      // the state and the RK register from the shared-memory copies
+      const double duk = sUd[(5 + k) * n3 + t], uk = sUd[k * n3 + t];
       const double r = a.first_stage ? dt * Ut[k] : a.rkA * duk + dt * Ut[k];
       du[k * n3] = r;
       uo[k * n3] = uk + a.rkB * r;
@@ -1320,8 +1278,9 @@ inline size_t lift_smem_bytes() {
 }
 
 // Launch variants the autotuner chooses among: the default elements per
-// block D (fewer on small meshes: fx_epb, felem_variant) and 2D (lifting up to 1024 nodes, volume up to 512), and for FP64
-// the volume kernel's two forms (fixed point, or FP64 sums per node).
+// block D (fewer on small meshes: fx_epb, felem_variant) and 2D (lifting up to
+// 1024 nodes, volume up to 512), and for FP64 the volume kernel's two forms of
+// the sums (fixed point, or FP64).
 template <int N, typename T>
 struct Variants {
   static constexpr int D = Shape<N>::EPB_DEFAULT;
@@ -1370,26 +1329,22 @@ inline void launch_lift(const StageArgs& a, cudaStream_t st) {
     k_lift<N, T, E><<<(unsigned)((a.E + S::EPB - 1) / S::EPB), S::THREADS, lift_smem_bytes<N, T, E>(), st>>>(a);
   }
 }
-// FX: the fixed-point form (FP64); E = 0: the default elements per block
-template <int N, int MODE, typename T, int E, bool FX>
-inline void launch_vol(const StageArgs& a, cudaStream_t st) {
+// E = 0: the default elements per block; sums64 (FP64): the sums in FP64
+template <int N, int MODE, typename T, int E>
+inline void launch_vol(const StageArgs& a, cudaStream_t st, bool sums64 = false) {
   using S = Shape<N, E>;
-  if constexpr (FX) {
+  if constexpr (sizeof(T) == sizeof(double)) {
     const int epb = E == 0 ? fx_epb<N>(S::EPB, a.E, a.sms) : S::EPB;
     const unsigned nb = (unsigned)((a.E + epb - 1) / epb);
     StageArgs b = a;
     b.prefetch = fx_wave(Fix<N>::TPE * epb, a.sms);
+    b.sums64 = sums64;
     if (extras(a)) k_volume_fx<N, MODE, true><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
     else k_volume_fx<N, MODE, false><<<nb, Fix<N>::TPE * epb, VolFix<N>::bytes(epb), st>>>(b);
   } else {
     const unsigned nb = (unsigned)((a.E + S::EPB - 1) / S::EPB);
-    if constexpr (sizeof(T) == sizeof(float)) {
-      if (!extras(a)) {
-        k_volume<N, MODE, T, E, false><<<nb, S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
-        return;
-      }
-    }
-    k_volume<N, MODE, T, E, true><<<nb, S::THREADS, VolumeSmem<N, T, E>::bytes, st>>>(a);
+    if (extras(a)) k_volume<N, MODE, E, true><<<nb, S::THREADS, VolumeSmem<N, E>::bytes, st>>>(a);
+    else k_volume<N, MODE, E, false><<<nb, S::THREADS, VolumeSmem<N, E>::bytes, st>>>(a);
   }
 }
 template <int N, typename T, bool GL = false>
@@ -1415,21 +1370,12 @@ inline void vol_variant(const StageArgs& a, int epb, int pairs, cudaStream_t st)
   using V = Variants<N, T>;
   if constexpr (MODE == 0) {
     // dg_rhs and the diagnostics: the default variant
-    launch_vol<N, 0, T, 0, V::fp64>(a, st);
+    launch_vol<N, 0, T, 0>(a, st);
   } else {
-    const bool pr = V::fp64 && (pairs < 0 ? true : pairs != 0);
     if constexpr (V::vol2) {
-      if (epb == 2 * V::D) {
-        if constexpr (V::fp64) {
-          if (!pr) return launch_vol<N, 1, T, 2 * V::D, false>(a, st);
-        }
-        return launch_vol<N, 1, T, 2 * V::D, V::fp64>(a, st);
-      }
+      if (epb == 2 * V::D) return launch_vol<N, 1, T, 2 * V::D>(a, st, pairs == 0);
     }
-    if constexpr (V::fp64) {
-      if (!pr) return launch_vol<N, 1, T, 0, false>(a, st);
-    }
-    launch_vol<N, 1, T, 0, V::fp64>(a, st);
+    launch_vol<N, 1, T, 0>(a, st, pairs == 0);
   }
 }
 
@@ -1457,10 +1403,14 @@ cudaError_t stage_set_attrs() {
   } else {
     lift(k_lift<N, T, 0>, lift_smem_bytes<N, T, 0>());
     if constexpr (V::lift2) lift(k_lift<N, T, 2 * V::D>, lift_smem_bytes<N, T, 2 * V::D>());
-    lift(k_volume<N, 0, T, 0, true>, VolumeSmem<N, T, 0>::bytes);
-    lift(k_volume<N, 0, T, 0, false>, VolumeSmem<N, T, 0>::bytes);
-    lift(k_volume<N, 1, T, 0, false>, VolumeSmem<N, T, 0>::bytes);
-    if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D, false>, VolumeSmem<N, T, 2 * V::D>::bytes);
+    auto volume = [&](auto extra) {
+      constexpr bool X = decltype(extra)::value;
+      lift(k_volume<N, 0, 0, X>, VolumeSmem<N, 0>::bytes);
+      lift(k_volume<N, 1, 0, X>, VolumeSmem<N, 0>::bytes);
+      if constexpr (V::vol2) lift(k_volume<N, 1, 2 * V::D, X>, VolumeSmem<N, 2 * V::D>::bytes);
+    };
+    volume(std::false_type());
+    volume(std::true_type());
   }
   lift(k_prolong_gl<N>, gl_prolong_smem<N>());
   if constexpr (V::fp64) {
@@ -1472,8 +1422,6 @@ cudaError_t stage_set_attrs() {
     lift(k_volume_gl<N, 0, T>, gl_volume_smem<N, T>());
     lift(k_volume_gl<N, 1, T>, gl_volume_smem<N, T>());
   }
-  lift(k_volume<N, 1, T, 0, true>, VolumeSmem<N, T, 0>::bytes);
-  if constexpr (V::vol2) lift(k_volume<N, 1, T, 2 * V::D, true>, VolumeSmem<N, T, 2 * V::D>::bytes);
   if constexpr (!V::fp64) {
     lift(k_fprep<N>, FusedSmem<N>::bytes);
     auto felem = [&](auto extra) {
@@ -1753,8 +1701,8 @@ cudaError_t stage_launch(dg_ctx* c, const double* U, int mode, double rkA, doubl
 // arrays: the lifted gradients and surface fluxes (recomputed by every
 // stage), and an RK update redirected into the Ut and public-layout buffers;
 // the state is untouched.  ms[]: per variant, mean ms over the timed
-// repetitions, in the order lift D, lift 2D, volume (D, default mapping),
-// volume (D, other mapping), volume (2D, default), volume (2D, other), side
+// repetitions, in the order lift D, lift 2D, volume (D, default form),
+// volume (D, other form), volume (2D, default), volume (2D, other), side
 // 256, side 128 (-1 where a variant does not exist).
 // Autotuner of the two-kernel FP32-bulk stage: the element kernel at D and
 // 2D elements per block (ms[2], ms[4]) and the side kernel at 256 and 128
@@ -1878,16 +1826,12 @@ cudaError_t stage_autotune(dg_ctx* c, double* ms) {
         best.vol_pairs = pairs;
       }
     };
-    const bool other = !c->tune_keep_mapping;  // also try the other thread mapping
-    vol(2, timed([&] { launch_vol<N, 1, T, 0, V::fp64>(a, st); }), V::D, V::fp64 ? 1 : 0);
-    if constexpr (V::fp64) {
-      if (other) vol(3, timed([&] { launch_vol<N, 1, T, 0, false>(a, st); }), V::D, 0);
-    }
+    const bool other = !c->tune_keep_mapping;  // also try the other form of the sums
+    vol(2, timed([&] { launch_vol<N, 1, T, 0>(a, st); }), V::D, V::fp64 ? 1 : 0);
+    if (V::fp64 && other) vol(3, timed([&] { launch_vol<N, 1, T, 0>(a, st, true); }), V::D, 0);
     if constexpr (V::vol2) {
-      vol(4, timed([&] { launch_vol<N, 1, T, 2 * V::D, V::fp64>(a, st); }), 2 * V::D, V::fp64 ? 1 : 0);
-      if constexpr (V::fp64) {
-        if (other) vol(5, timed([&] { launch_vol<N, 1, T, 2 * V::D, false>(a, st); }), 2 * V::D, 0);
-      }
+      vol(4, timed([&] { launch_vol<N, 1, T, 2 * V::D>(a, st); }), 2 * V::D, V::fp64 ? 1 : 0);
+      if (V::fp64 && other) vol(5, timed([&] { launch_vol<N, 1, T, 2 * V::D>(a, st, true); }), 2 * V::D, 0);
     }
     ms[6] = timed([&] {
       if (c->prm.viscous) launch_side<N, T>(a, 256, st, true);

@@ -96,7 +96,7 @@ struct CaseData {
 struct StageConfig {
   int lift_epb = 0;     // elements per block of the lifting kernel (0: default)
   int vol_epb = 0;      // elements per block of the volume kernel (0: default)
-  int vol_pairs = -1;   // 1: line-pair two-point sums, 0: per node, -1: default
+  int vol_pairs = -1;   // FP64 volume kernel's sums: 1 fixed point, 0 FP64, -1 default
   int side_block = 256; // threads per block of the side kernels (128 or 256)
   // FP32-bulk stage: 0 the two-kernel stage where it applies (periodic LGL
   // meshes of a single context), else the four-kernel one; 1 always the
@@ -109,6 +109,7 @@ struct StageConfig {
 // Per-stage launch parameters of the RHS kernels.
 struct StageArgs {
   int E, S;
+  int sums64;            // FP64 volume kernel: every element's sums in FP64
   int sms;               // multiprocessors of the context's device (launch shapes; host only)
   const double* U;       // [E][5][n3] internal state
   const double* metric;  // [E][10][n3]: J a^d_c at d*3+c, then 1/J
