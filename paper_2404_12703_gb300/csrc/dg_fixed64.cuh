@@ -212,7 +212,10 @@ __device__ __forceinline__ bool lines_quiet(int v, unsigned cut, Mag mag) {
   return true;
 }
 // Which sums an element and its block take: direct (FP64), and whether any or
-// all elements of the block do
+// all elements of the block do.  Blocks of plain elements run code of their own
+// from here on, the others a copy out of line: beside each other in one body
+// the FP64 form's registers cost the fixed-point one 1 to 8 % (volume kernel,
+// 24^3, N = 7: 2,575 against 2,552 us; 16^3, N = 5: 373 against 345).
 struct SumForm {
   bool direct, any, all;
 };
@@ -221,7 +224,7 @@ struct SumForm {
 // quiet(v): whether node v is quiet in a group on all its lines; flag: a word
 // of the element's shared memory, zero when called.
 template <int N, class Quiet>
-__device__ __noinline__ SumForm sum_form(bool bad, int t, unsigned* flag, Quiet quiet) {
+__device__ __forceinline__ SumForm sum_form(bool bad, int t, unsigned* flag, Quiet quiet) {
   constexpr int n3 = Fix<N>::n3, TPE = Fix<N>::TPE;
   bool is = false;
   if (!bad)
@@ -391,11 +394,14 @@ __device__ __forceinline__ void lift_prims_fx(const StageArgs& a, int e, long lo
 // needs no such test: an error of 2^-60 of the element's largest gradient of a
 // component is below FP64's rounding of the pressure in the momentum's sums
 template <int N>
+__device__ __forceinline__ bool lift_plain(bool bad, const unsigned* fin) {
+  const bool ask = bad || ~fin[7] < fx_cut(fin[3]);
+  return !(blockDim.x == Fix<N>::TPE ? ask : __syncthreads_or(ask));
+}
+template <int N>
 __device__ __forceinline__ SumForm lift_form(bool bad, const long long* q, const unsigned* fin, int t, unsigned* flag) {
   constexpr int n = Fix<N>::n;
   const unsigned cut = fx_cut(fin[3]);
-  const bool ask = bad || ~fin[7] < cut;
-  if (!(blockDim.x == Fix<N>::TPE ? ask : __syncthreads_or(ask))) return {false, false, false};
   const double* T = reinterpret_cast<const double*>(q + 3 * Fix<N>::Pn);
   auto mag = [=](int v) { return fx_mag(T[fx_pad<n>(v)]); };
   return sum_form<N>(bad, t, flag, [=](int v) { return mag(v) < cut && lines_quiet<n>(v, cut, mag); });
@@ -555,45 +561,49 @@ __device__ __forceinline__ void lift_sums_f64(const Ops* o, const double* Me, co
   }
 }
 
+// the element's places in shared memory
 template <int N>
-__global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_lift_fx(StageArgs a) {
-  using F = Fix<N>;
+struct LiftMem {
   using L = LiftFix<N>;
-  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
-  Fx* sD = reinterpret_cast<Fx*>(smraw);
-  double* sDd = reinterpret_cast<double*>(sD + L::ntab);  // (filled by lift_sums_f64)
-  unsigned* red = reinterpret_cast<unsigned*>(smraw + 16 * L::ntab) + le * L::nred;
-  unsigned* fin = red + F::W * L::Q;
-  unsigned* flag = fin + L::Q;
-  long long* q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::planes * Pn;
-  long long* J = q + 4 * Pn;   // [2][3][Pn]
-  long long* W = J + 6 * Pn;   // [12][Pn]
-  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
-  if (a.elem_case && __syncthreads_and(!er.busy)) return;
-  const int e = er.e;
-  const double* Me = a.metric + (size_t)e * 10 * n3;
-  lift_table_fx<N>(a.ops, sD);
-  prefetch_sides64<N>(a, e, a.lflux, 12, t);
-  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
-  if (t == 0) *flag = 0u;
-  {
-    unsigned m[8];
-    lift_prims_fx<N>(a, e, q, m, t);
-    fx_reduce<N, 8>(m, red, fin, t);
-    __syncthreads();
+  Fx* sD;
+  double* sDd;  // (filled by lift_sums_f64)
+  unsigned *red, *fin, *flag;
+  long long *q, *J, *W;  // [4][Pn], [2][3][Pn], [12][Pn]
+  __device__ __forceinline__ LiftMem(unsigned char* smraw, int epb, int le) {
+    sD = reinterpret_cast<Fx*>(smraw);
+    sDd = reinterpret_cast<double*>(sD + L::ntab);
+    red = reinterpret_cast<unsigned*>(smraw + 16 * L::ntab) + le * L::nred;
+    fin = red + Fix<N>::W * L::Q;
+    flag = fin + L::Q;
+    q = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::planes * Fix<N>::Pn;
+    J = q + 4 * Fix<N>::Pn;
+    W = J + 6 * Fix<N>::Pn;
   }
+};
+template <int N>
+__device__ __forceinline__ bool lift_bad(const unsigned* fin) {
   bool bad = false;
 #pragma unroll
   for (int k = 0; k < 7; ++k) bad = bad || fx_bad(fin[k]);
+  return bad;
+}
+// the sums and what follows them; PLAIN: the block's elements are all in fixed point
+template <int N, bool PLAIN>
+__device__ __forceinline__ void lift_rest(const StageArgs& a, const LiftMem<N>& M, const ElemRef& er, int t) {
+  using F = Fix<N>;
+  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn;
+  const int e = er.e;
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+  const unsigned* fin = M.fin;
   const int eq[4] = {fx_exp(fin[0]), fx_exp(fin[1]), fx_exp(fin[2]), fx_exp(fin[3])};
   const int eJ[3] = {fx_exp(fin[4]), fx_exp(fin[5]), fx_exp(fin[6])};
-  const SumForm form = lift_form<N>(bad, q, fin, t, flag);
-  if (!form.all) lift_sums_fx<N>(Me, q, J, W, sD, t, eq, eJ, form.direct);
+  SumForm form = {false, false, false};
+  if constexpr (!PLAIN) form = lift_form<N>(lift_bad<N>(fin), M.q, fin, t, M.flag);
+  const bool bad = form.direct;
+  if (!form.all) lift_sums_fx<N>(Me, M.q, M.J, M.W, M.sD, t, eq, eJ, bad);
   if (form.any)
-    lift_sums_f64<N>(a.ops, Me, reinterpret_cast<const double*>(q), reinterpret_cast<double*>(J),
-                     reinterpret_cast<double*>(W), sDd, t, !form.direct);
+    lift_sums_f64<N>(a.ops, Me, reinterpret_cast<const double*>(M.q), reinterpret_cast<double*>(M.J),
+                     reinterpret_cast<double*>(M.W), M.sDd, t, !bad);
   if (!er.valid) return;
   const int pH = a.ops->fxH_bits - 2;
   const double* Lf = a.lflux;
@@ -602,8 +612,8 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
     double acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      const long long w = W[k * Pn + pv];
-      acc[k] = form.direct ? __longlong_as_double(w) : fx_to(w, pH - eq[k / 3] - eJ[k % 3]);
+      const long long w = M.W[k * Pn + pv];
+      acc[k] = bad ? __longlong_as_double(w) : fx_to(w, pH - eq[k / 3] - eJ[k % 3]);
     }
     // surface part: on LGL nodes only face nodes receive it
     const int idx[3] = {v % n, (v / n) % n, v / n2};
@@ -627,6 +637,36 @@ __global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_
 #pragma unroll
     for (int k = 0; k < 12; ++k) g[k * n3] = acc[k] * Ji;
   }
+}
+
+template <int N>
+__device__ __noinline__ void lift_mixed(const StageArgs& a, ElemRef er) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / Fix<N>::TPE, le = threadIdx.x / Fix<N>::TPE;
+  lift_rest<N, false>(a, LiftMem<N>(smraw, epb, le), er, threadIdx.x % Fix<N>::TPE);
+}
+
+template <int N>
+__global__ void __launch_bounds__(Fix<N>::TL, Fix<N>::min_blocks(Fix<N>::TL)) k_lift_fx(const __grid_constant__ StageArgs a) {
+  using F = Fix<N>;
+  constexpr int TPE = F::TPE;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
+  const LiftMem<N> M(smraw, epb, le);
+  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
+  if (a.elem_case && __syncthreads_and(!er.busy)) return;
+  lift_table_fx<N>(a.ops, M.sD);
+  prefetch_sides64<N>(a, er.e, a.lflux, 12, t);
+  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
+  if (t == 0) *M.flag = 0u;
+  {
+    unsigned m[8];
+    lift_prims_fx<N>(a, er.e, M.q, m, t);
+    fx_reduce<N, 8>(m, M.red, M.fin, t);
+    __syncthreads();
+  }
+  if (lift_plain<N>(lift_bad<N>(M.fin), M.fin)) lift_rest<N, true>(a, M, er, t);
+  else lift_mixed<N>(a, er);
 }
 
 // ---------------------------------------------------------------------------
@@ -926,7 +966,7 @@ __device__ __forceinline__ void kep_fx(const longlong2* P, const longlong2* Jab,
 // fluxes, so that an element whose sums are taken here costs the FP64 unit as
 // many of them
 template <int N>
-__device__ __noinline__ void kep_f64(const double2* P, const double2* Jab, const double* Jc, double* A,
+__device__ __forceinline__ void kep_f64(const double2* P, const double2* Jab, const double* Jc, double* A,
                                      const double* Dsplit, int t, bool skip) {
   using F = Fix<N>;
   constexpr int n = F::n, n3 = F::n3, Pn = F::Pn, LW = F::LW;
@@ -981,81 +1021,55 @@ __device__ __noinline__ void kep_f64(const double2* P, const double2* Jab, const
   }
 }
 
-// EXTRA: a run with shock capturing, a sponge or a source
-template <int N, int MODE, bool EXTRA>
-__global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_volume_fx(StageArgs a) {
+// the element's places in shared memory
+template <int N>
+struct VolMem {
+  using L = VolFix<N>;
+  Fx *sS, *sDh, *sW;  // [n2] w Dsplit, [n2] Dhat, [n] 1 / w
+  double* sVi;        // [n2]
+  unsigned *red, *fin;
+  VolScale* sc;
+  longlong2* Jab;  // [3][Pn] (m0, m1)
+  long long* Jc;   // [3][Pn] m2
+  long long* PT;   // the primitives' place
+  long long* A;    // [5][Pn]
+  __device__ __forceinline__ VolMem(unsigned char* smraw, int epb, int le) {
+    constexpr int n = Fix<N>::n, n2 = Fix<N>::n2, Pn = Fix<N>::Pn;
+    sS = reinterpret_cast<Fx*>(smraw);
+    sDh = sS + n2;
+    sW = sDh + n2;
+    sVi = reinterpret_cast<double*>(sW + n);
+    red = reinterpret_cast<unsigned*>(sVi + n2) + le * (L::nred + L::nscale);
+    fin = red + Fix<N>::W * VQ_N;
+    sc = reinterpret_cast<VolScale*>(fin + VQ_N);
+    long long* mine = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::per_elem;
+    Jab = reinterpret_cast<longlong2*>(mine);
+    Jc = mine + 6 * Pn;
+    PT = mine + L::offP;
+    A = mine + L::offA;
+  }
+};
+// What follows the scales.  EXTRA: a run with shock capturing, a sponge or a
+// source; PLAIN: the block's elements are all plain (vol_scale).
+template <int N, int MODE, bool EXTRA, bool PLAIN>
+__device__ __forceinline__ void vol_rest(const StageArgs& a, const VolMem<N>& M, const ElemRef& er, const CaseParams& cp, int t) {
   using F = Fix<N>;
   using L = VolFix<N>;
   constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn, R = F::R;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
-  Fx* sS = reinterpret_cast<Fx*>(smraw);  // [n2] w Dsplit
-  Fx* sDh = sS + n2;                      // [n2] Dhat
-  Fx* sW = sDh + n2;                      // [n] 1 / w
-  double* sVi = reinterpret_cast<double*>(sW + n);
-  unsigned* red = reinterpret_cast<unsigned*>(sVi + n2) + le * (L::nred + L::nscale);
-  unsigned* fin = red + F::W * VQ_N;
-  VolScale* sc = reinterpret_cast<VolScale*>(fin + VQ_N);
-  long long* mine = reinterpret_cast<long long*>(smraw + L::head(epb)) + (size_t)le * L::per_elem;
-  longlong2* Jab = reinterpret_cast<longlong2*>(mine);  // [3][Pn] (m0, m1)
-  long long* Jc = mine + 6 * Pn;                        // [3][Pn] m2
-  long long* PT = mine + L::offP;
-  longlong2* P = reinterpret_cast<longlong2*>(PT);      // [3][Pn]
-  long long* A = mine + L::offA;                        // [5][Pn]
-  longlong2* G = P;                                     // [2][Pn] (after the two-point sums)
-  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
-  if (a.elem_case && __syncthreads_and(!er.busy)) return;
+  const Fx *sS = M.sS, *sDh = M.sDh, *sW = M.sW;
+  const double* sVi = M.sVi;
+  unsigned *red = M.red, *fin = M.fin;
+  VolScale* sc = M.sc;
+  longlong2 *Jab = M.Jab, *P = reinterpret_cast<longlong2*>(M.PT);  // P: [3][Pn]
+  long long *Jc = M.Jc, *PT = M.PT, *A = M.A, *mine = reinterpret_cast<long long*>(M.Jab);
+  longlong2* G = P;  // [2][Pn] (after the two-point sums)
   const int e = er.e;
-  const CaseParams cp = case_params(a, er.ce);
   const double* Me = a.metric + (size_t)e * 10 * n3;
-  for (int k = threadIdx.x; k < n2; k += blockDim.x) {
-    sS[k] = fx_split(a.ops->fxS[k]);
-    sDh[k] = fx_split(a.ops->fxH[k]);
-    sVi[k] = a.ops->Vinv[k];
-    if (k < n) sW[k] = fx_split(a.ops->fxW[k]);
-  }
-  prefetch_sides64<N>(a, e, a.fstar, 5, t);
-  if (t == 6 && a.viscous) prefetch64(a.g, (size_t)e * 12 * n3, 12 * n3);
-  if (t == 7 && MODE == 1 && !a.first_stage) prefetch64(a.dU, (size_t)e * 5 * n3, 5 * n3);
-  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
-  // ---- primitives (FP64 in their planes until the scales are known), maxima ----
   bool iso = true;
   SumForm form = {false, false, false};
-  {
-    unsigned m[VQ_N];
-#pragma unroll
-    for (int k = 0; k < VQ_N; ++k) m[k] = 0;
-    for (int v = t; v < n3; v += TPE) {
-      double U[5];
-      load_state64<n>(a, e, v, U);
-      const Prim64 pr = prim64(U, a.gm1);
-      const double rH = U[4] + pr.p, H = rH * pr.ri;
-      double2* Pd = reinterpret_cast<double2*>(P) + fx_pad<n>(v);
-      Pd[0] = make_double2(pr.rho, pr.p);
-      Pd[Pn] = make_double2(pr.u, pr.v);
-      Pd[2 * Pn] = make_double2(pr.w, H);
-      m[VQ_RHO] = max(m[VQ_RHO], fx_mag(pr.rho)), m[VQ_LO] = max(m[VQ_LO], ~fx_mag(pr.rho));
-      m[VQ_U] = max(m[VQ_U], fx_mag(pr.u));
-      m[VQ_V] = max(m[VQ_V], fx_mag(pr.v));
-      m[VQ_W] = max(m[VQ_W], fx_mag(pr.w));
-      m[VQ_P] = max(m[VQ_P], fx_mag(pr.p)), m[VQ_LO + 1] = max(m[VQ_LO + 1], ~fx_mag(pr.p));
-      m[VQ_H] = max(m[VQ_H], fx_mag(H));
-      m[VQ_RHOH] = max(m[VQ_RHOH], fx_mag(rH)), m[VQ_LO + 2] = max(m[VQ_LO + 2], ~fx_mag(rH));
-      m[VQ_MOM] = max(max(m[VQ_MOM], fx_mag(U[1])), max(fx_mag(U[2]), fx_mag(U[3])));
-#pragma unroll
-      for (int c = 0; c < 9; ++c) m[VQ_J + c] = max(m[VQ_J + c], fx_mag(Me[c * n3 + v]));
-    }
-    fx_reduce<N, VQ_N>(m, red, fin, t);
-    bool plain = true, out = false;
-    if (t < 32) out = a.sums64 || vol_bad<N>(fin, t);
-    if (t < 3) plain = vol_scale(*sc, fin, a.ops, t, out);
-    __syncwarp();
-    if (t < 3) vol_align(*sc, t);
-    __syncwarp();
-    if (!__syncthreads_and(plain)) {  // (all of the block's elements)
-      iso = __syncthreads_and(sc->iso != 0u);
-      form = vol_form<N>(sc, fin, P, t);
-    }
+  if constexpr (!PLAIN) {
+    iso = __syncthreads_and(sc->iso != 0u);
+    form = vol_form<N>(sc, fin, P, t);
   }
   const bool bad = form.direct;
   for (int v = t; v < n3; v += TPE) {
@@ -1377,6 +1391,75 @@ __global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV)) k_
     }
     finish_node64<n, MODE, EXTRA>(a, e, er.ce, v, s);
   }
+}
+template <int N, int MODE, bool EXTRA>
+__device__ __noinline__ void vol_mixed(const StageArgs& a, ElemRef er) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / Fix<N>::TPE, le = threadIdx.x / Fix<N>::TPE;
+  vol_rest<N, MODE, EXTRA, false>(a, VolMem<N>(smraw, epb, le), er, case_params(a, er.ce), threadIdx.x % Fix<N>::TPE);
+}
+
+template <int N, int MODE, bool EXTRA>
+__global__ void __launch_bounds__(Fix<N>::TV, Fix<N>::min_blocks(Fix<N>::TV))
+    k_volume_fx(const __grid_constant__ StageArgs a) {
+  using F = Fix<N>;
+  constexpr int n = F::n, n2 = F::n2, n3 = F::n3, TPE = F::TPE, Pn = F::Pn;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int epb = blockDim.x / TPE, le = threadIdx.x / TPE, t = threadIdx.x % TPE;
+  const VolMem<N> M(smraw, epb, le);
+  longlong2* P = reinterpret_cast<longlong2*>(M.PT);
+  const ElemRef er = elem_ref(a, blockIdx.x * epb + le);
+  if (a.elem_case && __syncthreads_and(!er.busy)) return;
+  const int e = er.e;
+  const CaseParams cp = case_params(a, er.ce);
+  const double* Me = a.metric + (size_t)e * 10 * n3;
+  for (int k = threadIdx.x; k < n2; k += blockDim.x) {
+    M.sS[k] = fx_split(a.ops->fxS[k]);
+    M.sDh[k] = fx_split(a.ops->fxH[k]);
+    M.sVi[k] = a.ops->Vinv[k];
+    if (k < n) M.sW[k] = fx_split(a.ops->fxW[k]);
+  }
+  prefetch_sides64<N>(a, e, a.fstar, 5, t);
+  if (t == 6 && a.viscous) prefetch64(a.g, (size_t)e * 12 * n3, 12 * n3);
+  if (t == 7 && MODE == 1 && !a.first_stage) prefetch64(a.dU, (size_t)e * 5 * n3, 5 * n3);
+  prefetch_next64<N>(a, (blockIdx.x + a.prefetch) * epb + le, t - 32);
+  // ---- primitives (FP64 in their planes until the scales are known), maxima ----
+  bool plain = true;
+  {
+    unsigned m[VQ_N];
+#pragma unroll
+    for (int k = 0; k < VQ_N; ++k) m[k] = 0;
+    for (int v = t; v < n3; v += TPE) {
+      double U[5];
+      load_state64<n>(a, e, v, U);
+      const Prim64 pr = prim64(U, a.gm1);
+      const double rH = U[4] + pr.p, H = rH * pr.ri;
+      double2* Pd = reinterpret_cast<double2*>(P) + fx_pad<n>(v);
+      Pd[0] = make_double2(pr.rho, pr.p);
+      Pd[Pn] = make_double2(pr.u, pr.v);
+      Pd[2 * Pn] = make_double2(pr.w, H);
+      m[VQ_RHO] = max(m[VQ_RHO], fx_mag(pr.rho)), m[VQ_LO] = max(m[VQ_LO], ~fx_mag(pr.rho));
+      m[VQ_U] = max(m[VQ_U], fx_mag(pr.u));
+      m[VQ_V] = max(m[VQ_V], fx_mag(pr.v));
+      m[VQ_W] = max(m[VQ_W], fx_mag(pr.w));
+      m[VQ_P] = max(m[VQ_P], fx_mag(pr.p)), m[VQ_LO + 1] = max(m[VQ_LO + 1], ~fx_mag(pr.p));
+      m[VQ_H] = max(m[VQ_H], fx_mag(H));
+      m[VQ_RHOH] = max(m[VQ_RHOH], fx_mag(rH)), m[VQ_LO + 2] = max(m[VQ_LO + 2], ~fx_mag(rH));
+      m[VQ_MOM] = max(max(m[VQ_MOM], fx_mag(U[1])), max(fx_mag(U[2]), fx_mag(U[3])));
+#pragma unroll
+      for (int c = 0; c < 9; ++c) m[VQ_J + c] = max(m[VQ_J + c], fx_mag(Me[c * n3 + v]));
+    }
+    fx_reduce<N, VQ_N>(m, M.red, M.fin, t);
+    bool out = false;
+    if (t < 32) out = a.sums64 || vol_bad<N>(M.fin, t);
+    if (t < 3) plain = vol_scale(*M.sc, M.fin, a.ops, t, out);
+    __syncwarp();
+    if (t < 3) vol_align(*M.sc, t);
+    __syncwarp();
+    plain = __syncthreads_and(plain);  // (all of the block's elements)
+  }
+  if (plain) vol_rest<N, MODE, EXTRA, true>(a, M, er, cp, t);
+  else vol_mixed<N, MODE, EXTRA>(a, er);
 }
 
 }  // namespace dg

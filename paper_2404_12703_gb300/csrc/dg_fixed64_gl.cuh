@@ -33,11 +33,19 @@ struct LiftGlFix {
   static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * per_elem; }
 };
 
-// (out of line here, where its registers cost the fixed-point path more than a call: 337 against 347 us)
+// the volume sums of a block with elements whose sums are taken in FP64;
+// whether this element's are (out of line)
 template <int N>
-__device__ __noinline__ void lift_sums_f64_call(const Ops* o, const double* Me, const double* q, double* J, double* W,
-                                                double* sD, int t, bool skip) {
-  lift_sums_f64<N>(o, Me, q, J, W, sD, t, skip);
+__device__ __noinline__ bool lift_gl_mixed(const Ops* o, const double* Me, long long* q, long long* J, long long* W, Fx* sD,
+                                           double* sDd, unsigned* fin, unsigned* flag, bool bad, int t) {
+  const int eq[4] = {fx_exp(fin[0]), fx_exp(fin[1]), fx_exp(fin[2]), fx_exp(fin[3])};
+  const int eJ[3] = {fx_exp(fin[4]), fx_exp(fin[5]), fx_exp(fin[6])};
+  const SumForm form = lift_form<N>(bad, q, fin, t, flag);
+  if (!form.all) lift_sums_fx<N>(Me, q, J, W, sD, t, eq, eJ, form.direct);
+  if (form.any)
+    lift_sums_f64<N>(o, Me, reinterpret_cast<const double*>(q), reinterpret_cast<double*>(J),
+                     reinterpret_cast<double*>(W), sDd, t, !form.direct);
+  return form.direct;
 }
 
 template <int N>
@@ -86,12 +94,8 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
   for (int k = 0; k < 20; ++k) bad = bad || (k != 7 && fx_bad(fin[k]));
   const int eq[4] = {fx_exp(fin[0]), fx_exp(fin[1]), fx_exp(fin[2]), fx_exp(fin[3])};
   const int eJ[3] = {fx_exp(fin[4]), fx_exp(fin[5]), fx_exp(fin[6])};
-  const SumForm form = lift_form<N>(bad, q, fin, t, flag);
-  bad = form.direct;
-  if (!form.all) lift_sums_fx<N>(Me, q, J, W, sD, t, eq, eJ, bad);
-  if (form.any)
-    lift_sums_f64_call<N>(a.ops, Me, reinterpret_cast<const double*>(q), reinterpret_cast<double*>(J),
-                          reinterpret_cast<double*>(W), sDd, t, !bad);
+  if (lift_plain<N>(bad, fin)) lift_sums_fx<N>(Me, q, J, W, sD, t, eq, eJ, false);
+  else bad = lift_gl_mixed<N>(a.ops, Me, q, J, W, sD, sDd, fin, flag, bad, t);
   // the six faces' lifting fluxes q* (s n), signed for this element (the
   // slave's outward normal is minus the master's), in its face frames
   for (int s = t; s < 6 * n2; s += TPE) {
@@ -225,6 +229,26 @@ struct VolGlFix {
   static constexpr size_t bytes(int epb) { return head(epb) + 8 * (size_t)epb * per_elem; }
 };
 
+// whether the element's sums are taken in FP64 (as vol_form; out of line)
+template <int N>
+__device__ __noinline__ bool vol_gl_direct(const double* u, double gm1, const unsigned* fin, bool bad, int t, unsigned* flag) {
+  constexpr int n = Fix<N>::n, n3 = Fix<N>::n3;
+  const unsigned cR = fx_cut(fin[20]), cP = fx_cut(fin[21]), cH = fx_cut(fin[22]);
+  auto level = [=](int v, int k) {
+    double U[5];
+    for (int i = 0; i < 5; ++i) U[i] = u[i * n3 + v];
+    const double p = prim64(U, gm1).p;
+    return fx_mag(k == 0 ? U[0] : k == 1 ? p : U[4] + p);
+  };
+  auto rho = [=](int v) { return level(v, 0); };
+  auto prs = [=](int v) { return level(v, 1); };
+  auto rhoH = [=](int v) { return level(v, 2); };
+  return sum_form<N>(bad, t, flag, [=](int v) {
+           return (rho(v) < cR && lines_quiet<n>(v, cR, rho)) || (prs(v) < cP && lines_quiet<n>(v, cP, prs)) ||
+                  (rhoH(v) < cH && lines_quiet<n>(v, cH, rhoH));
+         }).direct;
+}
+
 template <int N, int MODE>
 __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fix<N>::TPE * Fix<N>::D))
     k_volume_gl_fx(StageArgs a) {
@@ -313,25 +337,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
     bool ask = bad;
 #pragma unroll
     for (int k = 0; k < 3; ++k) ask = ask || ~fin[23 + k] < fx_cut(fin[20 + k]);
-    if (blockDim.x == TPE ? ask : __syncthreads_or(ask)) {
-      const double* u = a.U + (size_t)e * 5 * n3;
-      const double gm1 = a.gm1;
-      const unsigned cR = fx_cut(fin[20]), cP = fx_cut(fin[21]), cH = fx_cut(fin[22]);
-      auto level = [=](int v, int k) {
-        double U[5];
-        for (int i = 0; i < 5; ++i) U[i] = u[i * n3 + v];
-        const double p = prim64(U, gm1).p;
-        return fx_mag(k == 0 ? U[0] : k == 1 ? p : U[4] + p);
-      };
-      auto rho = [=](int v) { return level(v, 0); };
-      auto prs = [=](int v) { return level(v, 1); };
-      auto rhoH = [=](int v) { return level(v, 2); };
-      const SumForm form = sum_form<N>(bad, t, flag, [=](int v) {
-        return (rho(v) < cR && lines_quiet<n>(v, cR, rho)) || (prs(v) < cP && lines_quiet<n>(v, cP, prs)) ||
-               (rhoH(v) < cH && lines_quiet<n>(v, cH, rhoH));
-      });
-      bad = form.direct;
-    }
+    if (blockDim.x == TPE ? ask : __syncthreads_or(ask)) bad = vol_gl_direct<N>(a.U + (size_t)e * 5 * n3, a.gm1, fin, bad, t, flag);
   }
   if (!bad)
     for (int v = t; v < n3; v += TPE) {
