@@ -52,7 +52,7 @@ VOLUME64_BYTES_PER_DOF = 366
 # DRAM bytes per DOF of one k_volume_fx<7,1> launch, from the ncu capture summarised
 # in profiles/k_volume_tgv12_N7_fp64.md (12^3 mesh; the traffic scales with
 # the DOF count).  Set to None whenever the kernel changes until re-measured.
-VOLUME_TRAFFIC_BYTES_PER_DOF = 347.4
+VOLUME_TRAFFIC_BYTES_PER_DOF = 348.2
 # FP32-bulk, four-kernel stage: algorithmic bytes per DOF of one volume-kernel
 # launch (reads U 40, FP32 metrics 40, FP32 lifted gradients 48, dU 40, surface
 # fluxes ~8; writes U 40, dU 40)

@@ -9,7 +9,7 @@
 // FP64 multiplication.  The kernels here were bound by the FP64 unit (84 - 96 %
 // busy); what they keep on it is ConsToPrim, the stress tensor and the
 // Runge-Kutta update.  Measured per launch on 24^3 elements, N = 7 (7.08 M
-// nodes): volume kernel 7.70 -> 2.57 ms, lifting 4.12 -> 1.42 ms; now bound by
+// nodes): volume kernel 7.70 -> 2.55 ms, lifting 4.12 -> 1.40 ms; now bound by
 // latency at two blocks per SM.
 //
 // Numbers.  Every element scales each group of quantities (density, velocity,
@@ -33,8 +33,9 @@
 //   hypersonic flow (vol_bad), stresses above the pressure: in FP64 too.
 // - A non-finite value, or a group whose largest value is outside 2^-200 ..
 //   2^200: in FP64, with its own treatment of such values.
-// FP64 sums cost what they did before (an all-FP64 step takes 0.76 - 1.0 of
-// the time it took with every element so, N = 1 .. 7).
+// FP64 sums cost what they did before: a step whose elements all take them
+// (density ratios of 1e6) has 0.78, 0.88, 0.87, 0.89, 0.97, 1.07 and 1.01 of the
+// time it had in FP64 kernels, N = 1 .. 7; one without any 0.42 - 0.65.
 // Scales depend on the element alone, so results do not depend on the launch
 // shape.  The bounds on every intermediate value stand beside it; none can
 // overflow.  Error of the right-hand side against the long-double oracle over
@@ -233,6 +234,7 @@ __device__ __forceinline__ SumForm sum_form(bool bad, int t, unsigned* flag, Qui
   __syncwarp();
   __syncthreads();
   const bool direct = bad || *flag != 0u;
+  __syncwarp();
   const bool any = __syncthreads_or(direct), all = __syncthreads_and(direct);
   return {direct, any, all};
 }
@@ -396,6 +398,7 @@ __device__ __forceinline__ void lift_prims_fx(const StageArgs& a, int e, long lo
 template <int N>
 __device__ __forceinline__ bool lift_plain(bool bad, const unsigned* fin) {
   const bool ask = bad || ~fin[7] < fx_cut(fin[3]);
+  __syncwarp();
   return !(blockDim.x == Fix<N>::TPE ? ask : __syncthreads_or(ask));
 }
 template <int N>

@@ -3,8 +3,9 @@
 // (see dg_fixed64.cuh for the numbers and why; the work is that of
 // k_lift_gl and k_volume_gl in dg_stage_gl.cuh, which FP32-bulk uses).
 // Measured per launch on 12^3 elements, N = 7 (0.88 M nodes): lifting
-// 864 -> 328 us, volume kernel 549 -> 265 us; error against the long-double
-// oracle 0.86 of the FP64 kernels' in the mean (N = 1 .. 7, Ma 0.1 - 1.25).
+// 864 -> 336 us, volume kernel 549 -> 271 us; error against the long-double
+// oracle 0.79 of the FP64 kernels' in the geometric mean, at most 0.999 in any
+// variable (N = 1 .. 7, Ma 0.1 - 1.25).
 #pragma once
 
 namespace dg {
@@ -337,6 +338,7 @@ __global__ void __launch_bounds__(Fix<N>::TPE * Fix<N>::D, Fix<N>::min_blocks(Fi
     bool ask = bad;
 #pragma unroll
     for (int k = 0; k < 3; ++k) ask = ask || ~fin[23 + k] < fx_cut(fin[20 + k]);
+    __syncwarp();
     if (blockDim.x == TPE ? ask : __syncthreads_or(ask)) bad = vol_gl_direct<N>(a.U + (size_t)e * 5 * n3, a.gm1, fin, bad, t, flag);
   }
   if (!bad)

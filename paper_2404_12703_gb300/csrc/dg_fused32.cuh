@@ -647,8 +647,8 @@ struct CoefOfStage {
 };
 
 // EXTRA: a run with shock capturing, a sponge or a source.  Without their code
-// the kernel keeps its registers: k_felem<7, 1> spills 8 bytes instead of 80,
-// k_felem<5, 1> none instead of 40 (24^3 elements, N = 7: 995 -> 939 us per launch).
+// the kernel keeps its registers: k_felem<7, 1> spills none instead of 80
+// bytes, k_felem<5, 1> none instead of 32 (24^3 elements, N = 7: 995 -> 939 us per launch).
 template <int N, int MODE, int EPB_, bool EXTRA>
 __global__ void __launch_bounds__(Shape<N, EPB_>::THREADS, Shape<N, EPB_>::vol_min_blocks())
     k_felem(StageArgs a) {

@@ -1,19 +1,21 @@
 // dg_stage.cuh -- the kernels of one evaluation of the DG time derivative
 // (Eq. dgsem with the split-form volume integral and BR1 lifting) and of the
-// fused low-storage RK stage, templated on the arithmetic type T of the
-// flux, volume and surface work (double: the FP64 path; float: the FP32-bulk
-// path, in which the state, the RK register, the metrics and the final
-// combination stay in FP64).
+// fused low-storage RK stage, and the host code that launches them.  The side
+// kernels are templates on the arithmetic type T (double: the FP64 path; float:
+// the FP32-bulk path, in which the state, the RK register, the metrics and the
+// final combination stay in FP64).  k_lift and k_volume here are FP32-bulk's;
+// FP64 runs k_lift_fx and k_volume_fx (dg_fixed64.cuh), which do the same work
+// with their sums in fixed point.
 //
-// Per stage:
+// Per stage (the FP64 path, and FP32-bulk in its four-kernel form):
 //   k_surf_prims  ProlongToFace of the lifted primitives (u, v, w, T) and the
 //                 BR1 surface flux q* (s n) on every side node   (Lift_FillFlux)
-//   k_lift        lifted gradients, weak form: volume part with Dhat, surface
+//   k_lift(_fx)   lifted gradients, weak form: volume part with Dhat, surface
 //                 part from the sides, 1/J                      (Lift_VolInt,
 //                                                                Lift_SurfInt,
 //                                                                Lift_ApplyJac)
 //   k_surf_flux   Roe / LF flux plus BR1 viscous flux times s   (FillFlux)
-//   k_volume      split-form KEP volume integral, viscous volume term,
+//   k_volume(_fx) split-form KEP volume integral, viscous volume term,
 //                 optional DG/FV blending, SurfInt, ApplyJac and either Ut or
 //                 the RK update dU = A dU + dt Ut, U += B dU   (VolInt, SurfInt,
 //                                                                ApplyJac, RK)
@@ -306,7 +308,8 @@ __device__ __forceinline__ void lf_flux_s(const SPrim<T>& L, const SPrim<T>& R, 
 // square from one reciprocal square root, the upwind terms collected by
 // direction, the stresses contracted with the normal before the work term,
 // and one scaling by s / 2.  k_surf_flux on 24^3 elements, N = 7: 1,373 -> 1,048
-// us per launch, 952 with 1 / rho and p from k_surf_prims.
+// us per launch, 952 with 1 / rho and p from k_surf_prims, 979 since the
+// pressures are added last.
 // ---------------------------------------------------------------------------
 // ConsToPrim in FP64 (the FP64 path's references are zero)
 struct Prim64 {
@@ -1562,7 +1565,9 @@ inline cudaError_t fprep_launch(dg_ctx* c, const double* U, int64_t e0 = 0, int6
   return cudaGetLastError();
 }
 // One element per block on small meshes (N = 3, where a block holds four):
-// 4^3 elements then reach 64 SMs instead of 16 (ten steps of 4^3 elements 912 -> 780 us)
+// 4^3 elements then reach 64 SMs instead of 16 (ten steps of 4^3 elements 912 ->
+// 780 us).  At N = 2 (nine to a block) and 4 (two) an element is no whole number
+// of warps and the last one would idle in part; not measured there.
 template <int N>
 constexpr bool felem_single() {
   return Shape<N>::EPB_DEFAULT > 1 && Shape<N>::n3 >= 64 && Shape<N>::n3 % 32 == 0;
